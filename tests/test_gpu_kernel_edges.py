@@ -1,0 +1,68 @@
+"""Kernels at the sizes where they can go wrong: edges of tiles and groups, remainders, both ends of
+each range, against the oracle's definitions."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import decoder as od  # noqa: E402
+from paper_2609_34977_gb300 import _native as N  # noqa: E402
+from paper_2609_34977_gb300 import synth  # noqa: E402
+from tests.gpu_util import bf16_np, rowwise_rel  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def _bf16(seed, *shape):
+    g = torch.Generator().manual_seed(seed)
+    return torch.randn(*shape, generator=g).to(torch.bfloat16)
+
+
+@pytest.mark.parametrize("heads,kv_heads,head_dim,pos,offset", [
+    (4, 4, 64, [0, 15, 16], 0),                     # one head a K/V head; key groups of 16 not full
+    (4, 4, 128, [17, 63, 64], 4),                   # a cache 8 bytes off a 16-byte boundary
+    (28, 4, 128, [65, 127, 128, 129, 500, 7], 0),   # seven heads a K/V head, shares of unequal length
+    (18, 2, 64, [31, 260, 511], 0),                 # nine heads a K/V head: a second chunk of one head
+    (16, 1, 128, [0, 1, 300, 511, 48, 47, 33, 2], 0),  # two full chunks; clusters of eight CTAs
+])
+def test_decode_attention_edges(heads, kv_heads, head_dim, pos, offset):
+    # one decoder layer over a given cache: logits and the appended K/V rows. Tolerance: every rounding of
+    # the path is one bf16 unit (2^-9), as in the prefill's parity tests (2e-2 normwise a row).
+    cfg = dict(synth.TINY_DECODER, n_layers=1, n_heads=heads, n_kv_heads=kv_heads, head_dim=head_dim, d_ffn=256)
+    B, max_len, D, kvd = len(pos), 512, cfg["d_model"], kv_heads * head_dim
+    w = synth.decoder_weights(3, cfg, std=0.05)
+    wd = {k: v.cuda() for k, v in w.items() if k != "layers"}
+    wd["layers"] = [{k: v.cuda() for k, v in lw.items()} for lw in w["layers"]]
+    model = N.SpdModel(cfg, wd)
+    c = _bf16(5, B, max_len, 2 * kvd)
+    for b, p in enumerate(pos):
+        c[b, p:] = 0
+    flat = torch.zeros(c.numel() + 8, dtype=torch.bfloat16, device="cuda")
+    cache = flat[offset:offset + c.numel()]
+    cache.copy_(c.reshape(-1).cuda())
+    x = _bf16(6, B, D)
+    out = torch.full((B, cfg["vocab"]), float("nan"), device="cuda")
+    ws = torch.zeros(N.spd_decode_workspace_size(model, B), dtype=torch.uint8, device="cuda")
+    N.spd_decode(model, x.cuda(), np.array(pos), cache, max_len, out, ws)
+    torch.cuda.synchronize()
+    assert N.spd_workspace_status(ws) == 0
+    om = od.model_from_torch(w, cfg)
+    lw, rnd = om["layers"][0], od.bf16_round
+    h, p = bf16_np(x).astype(np.float64), np.array(pos)
+    xa = rnd(od.rmsnorm(h, lw["attn_norm"], cfg["rms_eps"]))
+    q, k = (rnd(od.rope(xa @ lw[n].T, p, nh, head_dim, cfg["rope_theta"])) for n, nh in (("wq", heads), ("wk", kv_heads)))
+    v = rnd(xa @ lw["wv"].T)
+    o = np.zeros((B, heads * head_dim))
+    for b in range(B):
+        kv = bf16_np(c[b, :p[b]]).astype(np.float64)
+        ka, va = np.concatenate([kv[:, :kvd], k[b:b + 1]]), np.concatenate([kv[:, kvd:], v[b:b + 1]])
+        o[b] = od.causal_attention(q[b:b + 1], ka, va, p[b:b + 1], np.arange(p[b] + 1), heads, kv_heads, head_dim)
+    h += rnd(o) @ lw["wo"].T
+    y = rnd(od.rmsnorm(h, lw["ffn_norm"], cfg["rms_eps"]))
+    h += rnd(od.silu(y @ lw["w_gate"].T) * (y @ lw["w_up"].T)) @ lw["w_down"].T
+    z = rnd(od.rmsnorm(h, om["final_norm"], cfg["rms_eps"]))
+    assert rowwise_rel(out.cpu().numpy(), z @ om["lm_head"].T) < 2e-2
+    got = bf16_np(cache).reshape(B, max_len, 2 * kvd)
+    for b in range(B):
+        assert rowwise_rel(got[b, p[b]:p[b] + 1], np.concatenate([k[b:b + 1], v[b:b + 1]], 1)) < 2e-2
+        assert not got[b, p[b] + 1:].any()
