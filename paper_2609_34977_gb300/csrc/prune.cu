@@ -68,6 +68,11 @@ struct PruneWs {
   float* csum;      // [T][L][K][d]
   double* ssum;     // [T][L][16] MSE / KL: per-cluster sums of st1 (+ st3), in fp64
   float* score;     // [T][m]
+  int* arrive;      // [T][4] arrivals of a tile's CTAs: anchors, selection, K-means (cleared by rowstats)
+  float* gpart;     // K-means over the whole GPU: [T][G][L][K][D] column sums a CTA,
+  float* gcent;     // [T][K][D] centroids,
+  double* gdsum;    // [T][G][L][16] sums of st1 (+ st3),
+  int* gmeta;       // [T][G][32] sizes, flags and a_j sums
   int* status;
 };
 
@@ -99,46 +104,68 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// Ascending bitonic sort of N (power of two) keys in shared memory by the whole block.
-__device__ void bitonic_sort(uint64_t* keys, int N) {
-  for (int k = 2; k <= N; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const int ixj = i ^ j;
-        if (ixj > i) {
-          const bool up = (i & k) == 0;
-          const uint64_t a = keys[i], b = keys[ixj];
-          if ((a > b) == up) {
-            keys[i] = b;
-            keys[ixj] = a;
-          }
-        }
-      }
-      __syncthreads();
-    }
+// Ranks of list positions [i0, i1) among keys[0..N) (ascending, ties to the lower position): block of
+// kRankThreads threads, i1 - i0 <= kRankThreads. keys is padded with the type's largest value to a
+// multiple of 16 bytes; rank (shared, [i1 - i0]) receives the counts after a barrier by the caller.
+// A lane takes one position and counts the smaller keys with 16-byte broadcast loads, two integer
+// instructions a key: the ranking is bound by instruction issue, so 32-bit keys without the index
+// are compared where they can be (a tie counts where the other position is lower: <= before the warp's
+// positions, < after them). The warps left over split the keys into segments.
+constexpr int kRankThreads = 1024;
+template <typename T>
+__device__ __forceinline__ void count_ranks(const T* keys, int N, int i0, int i1, int* rank) {
+  constexpr int V = 16 / int(sizeof(T));
+  struct alignas(16) Vec {
+    T v[V];
+  };
+  const Vec* kv = reinterpret_cast<const Vec*>(keys);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wt = (i1 - i0 + 31) >> 5, nseg = (kRankThreads / 32) / wt;
+  for (int i = threadIdx.x; i < i1 - i0; i += kRankThreads) rank[i] = 0;
+  __syncthreads();
+  const int blk = warp % wt, seg = warp / wt;
+  if (seg >= nseg) return;
+  const int first = i0 + 32 * blk, i = min(first + lane, i1 - 1);
+  const T ki = keys[i];
+  const int nv = (N + V - 1) / V, v0 = seg * nv / nseg, v1 = (seg + 1) * nv / nseg;
+  const int below = max(v0, min(v1, first / V)), above = max(below, min(v1, (first + 31) / V + 1));
+  int cnt[2] = {0, 0};
+#pragma unroll 4
+  for (int e = v0; e < below; ++e) {
+    const Vec x = kv[e];
+#pragma unroll
+    for (int u = 0; u < V; ++u) cnt[u & 1] += x.v[u] <= ki;
   }
+  for (int e = below; e < above; ++e) {
+    const Vec x = kv[e];
+#pragma unroll
+    for (int u = 0; u < V; ++u) cnt[u & 1] += x.v[u] < ki || (x.v[u] == ki && V * e + u < i);
+  }
+#pragma unroll 4
+  for (int e = above; e < v1; ++e) {
+    const Vec x = kv[e];
+#pragma unroll
+    for (int u = 0; u < V; ++u) cnt[u & 1] += x.v[u] < ki;
+  }
+  if (first + lane < i1) atomicAdd(&rank[i - i0], cnt[0] + cnt[1]);
 }
+// CTAs that rank one tile's list of n positions: one while its threads suffice, else 128 positions a
+// CTA, the last of them to finish going on with the whole list. (2739 keys: 48 us for one CTA sorting
+// them, 8 us so; 576 keys: 12.5 us with 64-bit keys, 7 us so.)
+__host__ __device__ inline int rank_ctas(int n) { return n <= kRankThreads ? 1 : (n + 127) / 128; }
 
-// Position of every key in the ascending order of keys[0..N) (distinct keys): the number of smaller
-// keys, counted by each thread for its keys (broadcast shared-memory reads, no barriers). rank_of
-// is called with (i, rank) for i < N.
-template <typename F>
-__device__ __forceinline__ void rank_keys(const uint64_t* keys, int N, F rank_of) {
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    const uint64_t ki = keys[i];
-    int r0 = 0, r1 = 0, r2 = 0, r3 = 0;
-    int j = 0;
-    for (; j + 4 <= N; j += 4) {
-      r0 += keys[j] < ki;
-      r1 += keys[j + 1] < ki;
-      r2 += keys[j + 2] < ki;
-      r3 += keys[j + 3] < ki;
-    }
-    for (; j < N; ++j) r0 += keys[j] < ki;
-    rank_of(i, r0 + r1 + r2 + r3);
-  }
+// True in every thread of the last of the tile's nb CTAs to arrive; what the others wrote before is
+// then visible through L2 (__ldcg). The counter was cleared by an earlier kernel of the call.
+__device__ __forceinline__ bool last_cta(int* counter, int nb) {
+  __shared__ int last;
+  if (nb == 1) return true;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(counter, 1) == nb - 1;
+  __syncthreads();
+  __threadfence();
+  return last;
 }
-constexpr int kRankMax = 2048;  // longest list ranked by counting; longer ones are sorted
 
 // Exclusive prefix sum of one int per thread over a block of 1024 threads.
 __device__ int block_scan_excl(int v, int* tmp, int* total) {
@@ -179,6 +206,7 @@ __global__ void __launch_bounds__(256) rowstats_kernel(PruneDims p, const float*
   pdl_wait();
   const int t = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * 8 + warp;
+  if (blockIdx.x == 0 && threadIdx.x < 4) w.arrive[4 * t + threadIdx.x] = 0;
   if (i >= p.n) return;
   for (int l = 0; l < p.L; ++l) {
     const float4* r = reinterpret_cast<const float4*>(feat_row(p, l, t, i));
@@ -233,32 +261,29 @@ __global__ void __launch_bounds__(256) rowstats_kernel(PruneDims p, const float*
 }
 
 // ---- 2. anchors (Eq. 1) and stable token lists ------------------------------------------------
-__global__ void __launch_bounds__(1024) anchor_kernel(PruneDims p, PruneWs w) {
+__global__ void __launch_bounds__(kRankThreads) anchor_kernel(PruneDims p, PruneWs w) {
   pdl_launch_dependents();
   pdl_wait();
-  __shared__ uint64_t keys[4096];
+  __shared__ __align__(16) uint32_t keys[4096];
+  __shared__ int rank[kRankThreads];
+  __shared__ int8_t role[4096];
   __shared__ int tmp[32];
-  const int t = blockIdx.x;
-  int N = 1;
-  while (N < p.n) N <<= 1;
-  // (a_v descending, index ascending) as ascending 64-bit keys
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    uint64_t k = ~0ull;
-    if (i < p.n)
-      k = (uint64_t(~ordered_key(w.a_v[size_t(t) * p.n + i])) << 32) | uint32_t(i);
-    keys[i] = k;
-  }
+  const int t = blockIdx.y, nb = gridDim.x;
+  // a_v descending as ascending keys; ties to the lower index
+  for (int i = threadIdx.x; i < ((p.n + 3) & ~3); i += blockDim.x)
+    keys[i] = i < p.n ? ~ordered_key(w.a_v[size_t(t) * p.n + i]) : ~0u;
   __syncthreads();
-  int8_t* role = w.role + size_t(t) * p.n;
-  if (p.n <= kRankMax) {
-    // anchor iff its key is among the n_anc smallest
-    rank_keys(keys, p.n, [&](int i, int r) { role[i] = r < p.n_anc ? 1 : 0; });
-  } else {
-    bitonic_sort(keys, N);
-    for (int i = threadIdx.x; i < p.n; i += blockDim.x) role[i] = 0;
-    __syncthreads();
-    for (int r = threadIdx.x; r < p.n_anc; r += blockDim.x) role[keys[r] & 0xffffffffu] = 1;
+  const int i0 = blockIdx.x * p.n / nb, i1 = (blockIdx.x + 1) * p.n / nb;
+  count_ranks(keys, p.n, i0, i1, rank);
+  __syncthreads();
+  int8_t* grole = w.role + size_t(t) * p.n;
+  for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+    role[i] = rank[i - i0] < p.n_anc ? 1 : 0;  // anchor iff its key is among the n_anc smallest
+    grole[i] = role[i];
   }
+  if (!last_cta(&w.arrive[4 * t], nb)) return;
+  if (nb > 1)
+    for (int i = threadIdx.x; i < p.n; i += blockDim.x) role[i] = __ldcg(grole + i);
   __syncthreads();
   // stable lists: each thread owns 4 consecutive tokens
   const int base = threadIdx.x * 4;
@@ -648,6 +673,58 @@ __device__ __forceinline__ void column_sums(float* part, int K, int D, int nl, c
   }
 }
 
+// Nearest centroid (squared Euclidean, ties to the lower cluster) of each of this CTA's nl rows, one
+// warp a row; *changed is raised where an assignment differs from asg's (or `first`).
+template <int KN, typename Row>
+__device__ __forceinline__ void assign_rows(const float* cent, int K, int D, int nl, bool first, int8_t* asg,
+                                            int* changed, Row xrow) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int jj = warp; jj < nl; jj += nw) {
+    const float* x = xrow(jj);
+    float part_d[KN];
+#pragma unroll
+    for (int k = 0; k < KN; ++k) part_d[k] = 0.0f;
+    // 16-byte loads, four in flight per lane (D is a multiple of 4)
+    for (int cb = 4 * lane; cb < D; cb += 512) {
+      float4 xv[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int c = cb + 128 * u;
+        xv[u] = c < D ? *reinterpret_cast<const float4*>(x + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int c = cb + 128 * u;
+        if (c < D) {
+#pragma unroll
+          for (int k = 0; k < KN; ++k)
+            if (k < K) {
+              const float4 ce = *reinterpret_cast<const float4*>(cent + k * D + c);
+              const float d0 = xv[u].x - ce.x, d1 = xv[u].y - ce.y, d2 = xv[u].z - ce.z,
+                          d3 = xv[u].w - ce.w;
+              part_d[k] += d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3;
+            }
+        }
+      }
+    }
+    int best = 0;
+    float bd = 0.0f;
+#pragma unroll
+    for (int k = 0; k < KN; ++k)
+      if (k < K) {
+        const float dk = warp_sum(part_d[k]);
+        if (k == 0 || dk < bd) {
+          bd = dk;
+          best = k;
+        }
+      }
+    if (lane == 0) {
+      if (first || asg[jj] != best) *changed = 1;
+      asg[jj] = int8_t(best);
+    }
+  }
+}
+
 // Sums over the KC CTAs of the cluster, in rank order, of the per-CTA column sums `part` (K x D in
 // every CTA's shared memory), for this CTA's slice of columns; `emit(k, c, value)` consumes them.
 template <int KC, typename F>
@@ -803,50 +880,7 @@ __global__ void __launch_bounds__(kmeans_threads<KN>()) kmeans_kernel(PruneDims 
         }
       }
     }
-    for (int jj = done_assign ? nl : warp; jj < nl; jj += nw) {
-      const float* x = xrow(jj);
-      float part_d[KN];
-#pragma unroll
-      for (int k = 0; k < KN; ++k) part_d[k] = 0.0f;
-      // 16-byte loads, four in flight per lane (D is a multiple of 4)
-      for (int cb = 4 * lane; cb < D; cb += 512) {
-        float4 xv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int c = cb + 128 * u;
-          xv[u] = c < D ? *reinterpret_cast<const float4*>(x + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int c = cb + 128 * u;
-          if (c < D) {
-#pragma unroll
-            for (int k = 0; k < KN; ++k)
-              if (k < K) {
-                const float4 ce = *reinterpret_cast<const float4*>(cent + k * D + c);
-                const float d0 = xv[u].x - ce.x, d1 = xv[u].y - ce.y, d2 = xv[u].z - ce.z,
-                            d3 = xv[u].w - ce.w;
-                part_d[k] += d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3;
-              }
-          }
-        }
-      }
-      int best = 0;
-      float bd = 0.0f;
-#pragma unroll
-      for (int k = 0; k < KN; ++k)
-        if (k < K) {
-          const float dk = warp_sum(part_d[k]);
-          if (k == 0 || dk < bd) {
-            bd = dk;
-            best = k;
-          }
-        }
-      if (lane == 0) {
-        if (it == 0 || asg[jj] != best) changed = 1;
-        asg[jj] = int8_t(best);
-      }
-    }
+    if (!done_assign) assign_rows<KN>(cent, K, D, nl, it == 0, asg, &changed, xrow);
     __syncthreads();
     // this CTA's column sums (token order, in registers) and sizes
     if (threadIdx.x < K) cnt[threadIdx.x] = 0;
@@ -993,6 +1027,215 @@ __global__ void __launch_bounds__(kmeans_threads<KN>()) kmeans_kernel(PruneDims 
   }
   if constexpr (FUSED) fused_select<KC>(p, w, out, cl, rank, t, j0, nl, asg, idx, av, sacc, ncl, ak,
                                         reinterpret_cast<uint64_t*>(rows));
+}
+
+// ---- 4b. K-means of a few large tiles over the whole GPU -----------------------------------------
+// G CTAs per tile (all resident: a cooperative launch of at most one CTA an SM), CTA r owning the
+// non-anchor tokens [r m / G, (r+1) m / G), whose F^L rows it keeps in shared memory where they fit. A
+// cluster holds at most 16 CTAs, so one image of thousands of tokens (11.5 MB of rows at 2260 x 1280)
+// ran on 8 SMs that read every row from L2 twice an iteration: 522 us. Here an iteration is the
+// assignment, the column sums (per-CTA, in token order) to L2, a barrier over the tile's CTAs, each
+// CTA's share of the columns summed over the CTAs in a fixed order, a second barrier and the new
+// centroids back: bound by the two barriers and the L2 round trips behind them (about 8 us), no longer by
+// the rows.
+constexpr int kGridThreads = 512;
+constexpr int kGridMaxCtas = 160;  // all tiles (workspace)
+constexpr int kGridMaxRows = 512;  // a CTA
+constexpr int kGridMeta = 2 * SPD_MAX_CLUSTERS;  // ints a CTA: sizes, [15 + 1]: changed flag; then a_j sums
+
+// Barrier number `phase` (1, 2, ...) of the G CTAs sharing *counter (zero at the start of the call). The
+// wait is bounded: on expiry the status is set and the counter raised past every later target, so that
+// every CTA of the tile runs on to its end.
+__device__ __forceinline__ void tile_barrier(int* counter, int G, int phase, int* status) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(counter, 1);
+    const long long t0 = clock64();
+    while (true) {
+      int v;
+      asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
+      if (v >= G * phase) break;
+      if (clock64() - t0 > kWaitBudget) {
+        set_status(status, SPD_ETIMEOUT);
+        atomicAdd(counter, 1 << 28);
+        break;
+      }
+    }
+  }
+  __syncthreads();
+}
+
+template <int KN, bool COS>
+__global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, PruneWs w, int G, int res) {
+  extern __shared__ __align__(16) float ksm[];
+  const int K = p.K, D = p.d, m = p.m, KD = K * D;
+  const int t = blockIdx.x / G, r = blockIdx.x - t * G;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int NW = kGridThreads / 32;
+  float* cent = ksm;       // [K][D]
+  float* rows = ksm + KD;  // res: [nl][D]
+  __shared__ int8_t asg[kGridMaxRows];
+  __shared__ int idx[kGridMaxRows];
+  __shared__ float av[kGridMaxRows], rinv[kGridMaxRows];
+  __shared__ int cnt[SPD_MAX_CLUSTERS], ncl[SPD_MAX_CLUSTERS];
+  __shared__ int changed, any_changed;
+  __shared__ float seg[NW][33];
+  __shared__ uint64_t rows_bar;
+  const int j0 = int((long long)r * m / G), j1 = int((long long)(r + 1) * m / G), nl = j1 - j0;
+  const int* ul = w.ulist + size_t(t) * m;
+  const size_t row0 = size_t(t) * p.n_tok + p.off;
+  const float* fin = p.feat[p.fin];
+  int* meta = w.gmeta + size_t(t) * G * kGridMeta;          // [G][kGridMeta]
+  float* part = w.gpart + size_t(t) * G * p.L * KD;         // [G][L][K][D] column sums of each CTA
+  double* dsum = w.gdsum + size_t(t) * G * p.L * 16;        // [G][L][16] MSE / KL: sums of st1 (+ st3)
+  float* gcent = w.gcent + size_t(t) * KD;                  // [K][D]
+  int* bar = &w.arrive[4 * t + 2];
+  int phase = 0;
+  pdl_wait();
+  for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) {
+    idx[jj] = ul[j0 + jj];
+    av[jj] = ordered_val(w.asim[size_t(t) * p.n + ul[j0 + jj]]);
+  }
+  if (threadIdx.x == 0) {
+    mbar_init(&rows_bar, 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (res && warp == 0 && nl > 0) {
+    if (lane == 0) mbar_arrive_expect_tx(&rows_bar, uint32_t(nl) * D * 4);
+    __syncwarp();
+    for (int jj = lane; jj < nl; jj += 32)
+      bulk_load(rows + size_t(jj) * D, fin + (row0 + idx[jj]) * D, uint32_t(D) * 4, &rows_bar);
+  }
+  for (int e = threadIdx.x; e < KD; e += blockDim.x) {
+    const int k = e / D, c = e - k * D;
+    cent[e] = feat_row(p, p.fin, t, ul[int((long long)k * m / K)])[c];
+  }
+  if (res && nl > 0) {
+    volatile int no_abort = 0;
+    if (!mbar_wait(&rows_bar, 0, &no_abort, kWaitBudget)) {
+      set_status(w.status, SPD_ETIMEOUT);
+      mbar_wait(&rows_bar, 0, &no_abort, kWaitBudget);  // the copies land before anything reuses it
+    }
+  }
+  auto xrow = [&](int jj) -> const float* { return res ? rows + size_t(jj) * D : fin + (row0 + idx[jj]) * D; };
+  // emit(e, sum over the CTAs of src[e] of their blocks of `ld` floats) for this CTA's share of [0, n):
+  // the warps sum contiguous ranges of CTAs in rank order, their sums are added in warp order
+  auto reduce = [&](const float* src, size_t ld, int n, auto emit) {
+    const int e0 = int((long long)r * n / G), e1 = int((long long)(r + 1) * n / G);
+    for (int eb = e0; eb < e1; eb += 32) {
+      const int e = eb + lane;
+      float sum = 0.0f;
+      if (e < e1) {
+        const int c0 = warp * G / NW, c1 = (warp + 1) * G / NW;
+#pragma unroll 10
+        for (int cc = c0; cc < c1; ++cc) sum += __ldcg(src + cc * ld + e);
+      }
+      seg[warp][lane] = sum;
+      __syncthreads();
+      if (warp == 0 && e < e1) {
+        float tot = 0.0f;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) tot += seg[q][lane];
+        emit(e, tot);
+      }
+      __syncthreads();
+    }
+  };
+  for (int it = 0; it < p.iters; ++it) {
+    if (threadIdx.x == 0) changed = 0;
+    if (threadIdx.x < SPD_MAX_CLUSTERS) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    assign_rows<KN>(cent, K, D, nl, it == 0, asg, &changed, xrow);
+    __syncthreads();
+    for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) atomicAdd(&cnt[asg[jj]], 1);
+    column_sums<KN>(part + size_t(r) * p.L * KD, K, D, nl, asg, RowAccess{res ? rows : nullptr, fin, row0, idx, D, nullptr});
+    __syncthreads();
+    // sizes of K <= 16 clusters and the flag in the first 16 ints of the CTA's block (a flag bit on size 0)
+    if (threadIdx.x < K) meta[r * kGridMeta + threadIdx.x] = cnt[threadIdx.x] | (changed ? 1 << 30 : 0);
+    tile_barrier(bar, G, ++phase, w.status);
+    if (threadIdx.x == 0) any_changed = 0;
+    __syncthreads();
+    if (warp < K) {
+      int n = 0, f = 0;
+      for (int cc = lane; cc < G; cc += 32) {
+        const int v = __ldcg(meta + cc * kGridMeta + warp);
+        n += v & ((1 << 30) - 1);
+        f |= v >> 30;
+      }
+#pragma unroll
+      for (int off = 16; off; off >>= 1) {
+        n += __shfl_xor_sync(0xffffffffu, n, off);
+        f |= __shfl_xor_sync(0xffffffffu, f, off);
+      }
+      if (lane == 0) {
+        ncl[warp] = n;
+        if (f) any_changed = 1;
+      }
+    }
+    __syncthreads();
+    if (it > 0 && !any_changed) break;  // the same in every CTA of the tile
+    if (it + 1 == p.iters) break;       // the centroids are read by assignments only
+    reduce(part, size_t(p.L) * KD, KD, [&](int e, float sum) {
+      const int n = ncl[e / D];
+      gcent[e] = n > 0 ? sum / float(n) : cent[e];
+    });
+    tile_barrier(bar, G, ++phase, w.status);
+    for (int e = 4 * threadIdx.x; e < KD; e += 4 * blockDim.x)
+      *reinterpret_cast<float4*>(cent + e) = __ldcg(reinterpret_cast<const float4*>(gcent + e));
+    __syncthreads();
+  }
+  // the final assignment, this CTA's sums of a_j (token order) and, a layer, of the unit feature rows (raw
+  // rows and st1 for the MSE and KL similarities). The loop left right after a barrier, without a reduction
+  // behind it: no CTA still reads the blocks written here.
+  for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) w.assign[size_t(t) * m + j0 + jj] = asg[jj];
+  if (threadIdx.x < K) {
+    float a = 0.0f;
+    for (int jj = 0; jj < nl; ++jj)
+      if (asg[jj] == int(threadIdx.x)) a += av[jj];
+    meta[r * kGridMeta + SPD_MAX_CLUSTERS + threadIdx.x] = __float_as_int(a);
+  }
+  for (int l = 0; l < p.L; ++l) {
+    const float* rstat = (COS ? w.inv : w.st1) + (size_t(l) * p.n_tiles + t) * p.n;
+    __syncthreads();  // the previous layer's statistics are no longer read
+    for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) rinv[jj] = rstat[idx[jj]];
+    __syncthreads();
+    if (!COS && threadIdx.x < K) {  // token order, fp64 (KL: the fp64 log-sum-exps)
+      const float* lo = p.sim == SPD_SIM_KL ? w.st3 + (size_t(l) * p.n_tiles + t) * p.n : nullptr;
+      double a = 0.0;
+      for (int jj = 0; jj < nl; ++jj)
+        if (asg[jj] == int(threadIdx.x)) a += double(rinv[jj]) + (lo ? double(lo[idx[jj]]) : 0.0);
+      dsum[(size_t(r) * p.L + l) * 16 + threadIdx.x] = a;
+    }
+    column_sums<KN>(part + (size_t(r) * p.L + l) * KD, K, D, nl, asg,
+                    RowAccess{res && l == p.fin ? rows : nullptr, p.feat[l], row0, idx, D, COS ? rinv : static_cast<float*>(nullptr)});
+  }
+  tile_barrier(bar, G, ++phase, w.status);
+  pdl_launch_dependents();
+  reduce(part, size_t(p.L) * KD, p.L * KD, [&](int e, float sum) { w.csum[size_t(t) * p.L * KD + e] = sum; });
+  if (r != 0) return;
+  if (warp < K) {  // lane sums over CTAs lane, lane + 32, ..., then a butterfly: a fixed order
+    float a = 0.0f;
+    for (int cc = lane; cc < G; cc += 32) a += __int_as_float(__ldcg(meta + cc * kGridMeta + SPD_MAX_CLUSTERS + warp));
+    a = warp_sum(a);
+    if (lane == 0) {
+      w.counts[t * 16 + warp] = ncl[warp];
+      w.asum[t * 16 + warp] = a;
+    }
+    if (!COS)
+      for (int l = 0; l < p.L; ++l) {
+        double d = 0.0;
+        for (int cc = lane; cc < G; cc += 32) d += __ldcg(dsum + (size_t(cc) * p.L + l) * 16 + warp);
+        d = warp_sum_d(d);
+        if (lane == 0) w.ssum[(size_t(t) * p.L + l) * 16 + warp] = d;
+      }
+  }
+  if (threadIdx.x == 0) {
+    int q[SPD_MAX_CLUSTERS];
+    compute_quotas(ncl, K, p.n_cmp, q);
+    for (int k = 0; k < K; ++k) w.quotas[t * 16 + k] = q[k];
+  }
 }
 
 // ---- 6. per-token Eq. 3 scores ----------------------------------------------------------------
@@ -1147,27 +1390,24 @@ __global__ void __launch_bounds__(256) received_finish_kernel(const float* parti
 }
 
 // ---- 7. per-cluster bottom-N_k, compaction, outputs -------------------------------------------
-__global__ void __launch_bounds__(1024) select_kernel(PruneDims p, PruneWs w, int32_t* keep_idx,
-                                                      uint8_t* kind, int8_t* cluster, float* scores) {
+__global__ void __launch_bounds__(kRankThreads) select_kernel(PruneDims p, PruneWs w, int32_t* keep_idx,
+                                                              uint8_t* kind, int8_t* cluster, float* scores) {
   pdl_launch_dependents();
   pdl_wait();
-  __shared__ uint64_t keys[4096];
+  __shared__ __align__(16) uint64_t keys[4096];  // (cluster, score) of the non-anchor list
+  __shared__ int rank[kRankThreads];
   __shared__ uint8_t kept[4096];
   __shared__ int tmp[32];
   __shared__ int seg[SPD_MAX_CLUSTERS + 1];
   __shared__ int quota[SPD_MAX_CLUSTERS];
-  const int t = blockIdx.x, m = p.m;
+  const int t = blockIdx.y, nb = gridDim.x, m = p.m;
   const int* ul = w.ulist + size_t(t) * m;
-  int N = 1;
-  while (N < max(m, 1)) N <<= 1;
-  for (int j = threadIdx.x; j < N; j += blockDim.x) {
-    uint64_t key = ~0ull;
-    if (j < m)
-      key = (uint64_t(w.assign[size_t(t) * m + j]) << 45) |
-            (uint64_t(ordered_key(w.score[size_t(t) * m + j])) << 13) | uint64_t(ul[j]);
-    keys[j] = key;
-  }
-  for (int i = threadIdx.x; i < p.n; i += blockDim.x) kept[i] = uint8_t(w.role[size_t(t) * p.n + i]);
+  int8_t* role = w.role + size_t(t) * p.n;
+  for (int j = threadIdx.x; j < ((m + 1) & ~1); j += blockDim.x)
+    keys[j] = j < m ? (uint64_t(w.assign[size_t(t) * m + j]) << 32) | ordered_key(w.score[size_t(t) * m + j])
+                    : ~0ull;
+  if (nb == 1)
+    for (int i = threadIdx.x; i < p.n; i += blockDim.x) kept[i] = uint8_t(role[i]);
   if (threadIdx.x == 0) {
     int acc = 0;
     for (int k = 0; k < p.K; ++k) {
@@ -1178,19 +1418,22 @@ __global__ void __launch_bounds__(1024) select_kernel(PruneDims p, PruneWs w, in
     seg[p.K] = acc;
   }
   __syncthreads();
-  if (m <= kRankMax) {
+  const int j0 = blockIdx.x * m / nb, j1 = (blockIdx.x + 1) * m / nb;
+  if (j0 < j1) {  // m > 0 (block-uniform)
+    count_ranks(keys, m, j0, j1, rank);
+    __syncthreads();
     // the key at sorted position r of cluster k's segment is kept iff r - seg[k] < quota[k]
-    rank_keys(keys, m, [&](int j, int r) {
-      const int k = int(keys[j] >> 45);
-      if (r - seg[k] < quota[k]) kept[keys[j] & 0x1fffu] = 2;
-    });
-  } else {
-    bitonic_sort(keys, N);
-    for (int r = threadIdx.x; r < m; r += blockDim.x) {
-      const int k = int(keys[r] >> 45);
-      if (r - seg[k] < quota[k]) kept[keys[r] & 0x1fffu] = 2;
+    for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
+      const int k = int(keys[j] >> 32);
+      if (rank[j - j0] - seg[k] < quota[k]) {
+        if (nb == 1) kept[ul[j]] = 2;
+        else role[ul[j]] = 2;  // the anchors' flags are 1
+      }
     }
   }
+  if (!last_cta(&w.arrive[4 * t + 1], nb)) return;
+  if (nb > 1)
+    for (int i = threadIdx.x; i < p.n; i += blockDim.x) kept[i] = uint8_t(__ldcg(role + i));
   __syncthreads();
   const int base = threadIdx.x * 4;
   int nk = 0;
@@ -1287,6 +1530,10 @@ int validate(const spd_prune_cfg* c, PruneDims* p) {
   return SPD_OK;
 }
 
+// Whether a call is of the few, large tiles that K-means spreads over the whole GPU (grid_plan below
+// decides with the device's SM count): workspace is set aside for them.
+bool grid_tile(const PruneDims& p) { return p.n_tiles <= 10 && p.m > 0; }
+
 PruneWs carve(const PruneDims& p, Carve& cv) {
   PruneWs w;
   const size_t T = p.n_tiles;
@@ -1308,6 +1555,12 @@ PruneWs carve(const PruneDims& p, Carve& cv) {
   w.csum = cv.take<float>(T * p.L * p.K * p.d);
   w.ssum = cv.take<double>(T * p.L * 16);
   w.score = cv.take<float>(T * (p.m + 1));
+  w.arrive = cv.take<int>(T * 4);
+  const size_t gc = grid_tile(p) ? kGridMaxCtas : 0;  // CTAs of all tiles
+  w.gpart = cv.take<float>(gc * p.L * p.K * p.d);
+  w.gcent = cv.take<float>(gc ? T * p.K * p.d : 0);
+  w.gdsum = cv.take<double>(gc * p.L * 16);
+  w.gmeta = cv.take<int>(gc * kGridMeta);
   return w;
 }
 
@@ -1362,6 +1615,13 @@ int kmeans_setup() {
     if (err == cudaSuccess) err = resident(kmeans_kernel<16, true, SPD_MAX_CLUSTERS, false>);
     if (err == cudaSuccess) err = resident(kmeans_kernel<16, true, 4, true, true>);
     if (err == cudaSuccess) err = resident(kmeans_kernel<16, true, SPD_MAX_CLUSTERS, true, true>);
+    auto wide = [](auto kern) {
+      return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kResSmem));
+    };
+    if (err == cudaSuccess) err = wide(kmeans_grid_kernel<4, true>);
+    if (err == cudaSuccess) err = wide(kmeans_grid_kernel<4, false>);
+    if (err == cudaSuccess) err = wide(kmeans_grid_kernel<SPD_MAX_CLUSTERS, true>);
+    if (err == cudaSuccess) err = wide(kmeans_grid_kernel<SPD_MAX_CLUSTERS, false>);
     g_res_clusters = 0;
     if (err == cudaSuccess) {
       cudaLaunchConfig_t cfg = {};
@@ -1391,6 +1651,9 @@ int kmeans_setup() {
 // Which kernels spd_prune launches for p (after kmeans_setup).
 struct PrunePlan {
   bool anchor_sim, res, fused;
+  int grid;        // CTAs a tile of the whole-GPU K-means, 0: clusters
+  bool grid_res;   // its rows fit in shared memory
+  size_t grid_smem;
   int launches;
 };
 PrunePlan prune_plan(const PruneDims& p) {
@@ -1408,6 +1671,21 @@ PrunePlan prune_plan(const PruneDims& p) {
   const size_t row_bytes = size_t((p.m + 15) / 16) * p.d * sizeof(float);
   q.fused = q.res && p.sim == SPD_SIM_COS && (p.m + 15) / 16 <= 512 &&
             row_bytes >= size_t(8) * (p.m + 1) + p.n;
+  // Tiles whose rows do not fit the 16 CTAs of a cluster (or more tiles than such clusters), few enough
+  // for 15 SMs each: the whole GPU. One image of 700 / 1024 / 2739 / 4096 x 1280: 199 / 279 / 671 / 976 ->
+  // 104 / 135 / 204 / 330 us a call; 9 / 10 tiles of 576 x 1024: 170 / 176 -> 149 / 160 us, but 12 of
+  // them 183 -> 187 us.
+  q.grid = 0;
+  if (!q.res && grid_tile(p)) {
+    const int G = std::min({num_sms() / p.n_tiles, kGridMaxCtas / p.n_tiles, (p.m + 3) / 4});
+    const size_t nl = (p.m + G - 1) / std::max(G, 1);
+    if (G >= 15 && nl <= size_t(kGridMaxRows)) {
+      q.grid = G;
+      q.grid_smem = size_t(p.K) * p.d * sizeof(float);
+      q.grid_res = q.grid_smem + nl * p.d * sizeof(float) <= kResSmem;
+      if (q.grid_res) q.grid_smem += nl * p.d * sizeof(float);
+    }
+  }
   q.launches = 2 + int(q.anchor_sim) + 1 + (q.fused ? 0 : int(p.m > 0) + 1);
   return q;
 }
@@ -1452,7 +1730,7 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
   SPD_CUDA_TRY(launch_pdl(p.sim == SPD_SIM_COS ? rowstats_kernel<SPD_SIM_COS>
                           : p.sim == SPD_SIM_MSE ? rowstats_kernel<SPD_SIM_MSE> : rowstats_kernel<SPD_SIM_KL>,
                           dim3((p.n + 7) / 8, T), dim3(256), 0, st, p, attn, w));
-  SPD_CUDA_TRY(launch_pdl(anchor_kernel, dim3(T), dim3(1024), 0, st, p, w));
+  SPD_CUDA_TRY(launch_pdl(anchor_kernel, dim3(rank_ctas(p.n), T), dim3(kRankThreads), 0, st, p, w));
   if (int rc = kmeans_setup()) return rc;
   const PrunePlan plan = prune_plan(p);
   if (plan.anchor_sim) {
@@ -1472,7 +1750,22 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
   const size_t cent_bytes = size_t(2) * p.K * p.d * sizeof(float);
   const size_t res_bytes = size_t((p.m + 15) / 16) * p.d * sizeof(float) + cent_bytes;
   const PruneOut out{keep_idx, kind, cluster, scores};
-  if (plan.fused && p.K == 4)
+  if (plan.grid) {
+    auto kern = p.K == 4 ? (p.sim == SPD_SIM_COS ? kmeans_grid_kernel<4, true> : kmeans_grid_kernel<4, false>)
+                : p.sim == SPD_SIM_COS ? kmeans_grid_kernel<SPD_MAX_CLUSTERS, true>
+                                       : kmeans_grid_kernel<SPD_MAX_CLUSTERS, false>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(plan.grid * T);
+    cfg.blockDim = dim3(kGridThreads);
+    cfg.dynamicSmemBytes = plan.grid_smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];  // every CTA resident: they wait on one another
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SPD_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, p, w, plan.grid, int(plan.grid_res)));
+  } else if (plan.fused && p.K == 4)
     SPD_CUDA_TRY((launch_kmeans<16, true, 4, true>(p, w, out, res_bytes, st)));
   else if (plan.fused)
     SPD_CUDA_TRY((launch_kmeans<16, true, SPD_MAX_CLUSTERS, true>(p, w, out, res_bytes, st)));
@@ -1492,7 +1785,7 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
                    : p.sim == SPD_SIM_MSE ? score_kernel<SPD_SIM_MSE> : score_kernel<SPD_SIM_KL>;
       SPD_CUDA_TRY(launch_pdl(score, dim3((p.m + 7) / 8, T), dim3(256), 0, st, p, w));
     }
-    SPD_CUDA_TRY(launch_pdl(select_kernel, dim3(T), dim3(1024), 0, st, p, w, keep_idx, kind, cluster,
+    SPD_CUDA_TRY(launch_pdl(select_kernel, dim3(rank_ctas(p.m), T), dim3(kRankThreads), 0, st, p, w, keep_idx, kind, cluster,
                             scores));
   }
   // algorithmic work per tile: every tapped layer's features and the attention read once, the

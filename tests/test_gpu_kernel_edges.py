@@ -8,7 +8,8 @@ torch = pytest.importorskip("torch")
 from oracle import decoder as od  # noqa: E402
 from paper_2609_34977_gb300 import _native as N  # noqa: E402
 from paper_2609_34977_gb300 import synth  # noqa: E402
-from tests.gpu_util import bf16_np, rowwise_rel  # noqa: E402
+from oracle import prune as op  # noqa: E402
+from tests.gpu_util import assert_prune_parity, bf16_np, conditioned_vision, gpu_prune, rowwise_rel  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -66,3 +67,55 @@ def test_decode_attention_edges(heads, kv_heads, head_dim, pos, offset):
     for b in range(B):
         assert rowwise_rel(got[b, p[b]:p[b] + 1], np.concatenate([k[b:b + 1], v[b:b + 1]], 1)) < 2e-2
         assert not got[b, p[b] + 1:].any()
+
+
+# ---- MSV-Prune: K-means over the whole GPU, rankings over several CTAs --------------------------------
+def _shuffled_tile(seed0, n, d, keep, **kw):
+    # a tile whose planted groups lie scattered over the token order: the seeds fall into any of them, so
+    # K-means takes several iterations; first seed with margins above 1e-3 at every decision
+    for seed in range(seed0, seed0 + 200):
+        v = synth.vision_tiles(seed, 1, n, d, 2, 4, has_cls=False, attn_form=1)
+        perm = np.random.default_rng(seed).permutation(n)
+        v = dict(feats=[np.ascontiguousarray(f[:, perm]) for f in v["feats"]],
+                 attn=np.ascontiguousarray(v["attn"][:, :, perm]))
+        res = op.prune(v["feats"], v["attn"], has_cls=False, attn_form=1, final_layer=1, keep=keep, **kw)
+        if op.well_conditioned(res[0]):
+            return v, res
+    raise RuntimeError("no well-conditioned seed found")
+
+
+@pytest.mark.parametrize("tiles,n,d,keep,kw", [
+    (1, 1025, 1280, 200, {}),                       # one CTA more than a ranking block holds
+    (1, 1500, 128, 300, dict(n_clusters=8)),        # the run-time number of clusters; many short rows
+    (2, 1030, 768, 100, dict(kmeans_iters=1)),      # two tiles; one assignment step
+    (8, 600, 2048, 64, {}),                         # rows too wide to stay in shared memory
+    (10, 576, 1024, 64, {}),                        # the most tiles of this form, rows resident
+    (1, 1100, 1024, 150, dict(sim="mse")),
+    (1, 1100, 1024, 150, dict(sim="kl")),
+])
+def test_whole_gpu_kmeans(tiles, n, d, keep, kw):
+    vs, res = [], []
+    for i in range(tiles):
+        _, v1, r1 = conditioned_vision(20263001 + 101 * i, 1, n, d, 2, 4, keep, 1, has_cls=False, attn_form=1, **kw)
+        vs.append(v1)
+        res += r1
+    v = {"feats": [np.concatenate([x["feats"][l] for x in vs]) for l in range(2)],
+         "attn": np.concatenate([x["attn"] for x in vs])}
+    assert_prune_parity(gpu_prune(v, keep, 1, has_cls=False, attn_form=1, **kw), res)
+
+
+def test_whole_gpu_kmeans_iterations():
+    v, res = _shuffled_tile(20264001, 900, 1280, 180)
+    a = gpu_prune(v, 180, 1, has_cls=False, attn_form=1)
+    assert_prune_parity(a, res)
+    b = gpu_prune(v, 180, 1, has_cls=False, attn_form=1)  # sums in a fixed order: the same bits again
+    np.testing.assert_array_equal(a["scores"].view(np.uint32), b["scores"].view(np.uint32))
+
+
+@pytest.mark.parametrize("n", [1024, 1025, 4096])
+def test_anchor_ranking_with_ties(n):
+    # equal importances fall to the lower index, on one CTA (up to 1024 tokens) and on several
+    v = synth.vision_tiles(5, 1, n, 64, 1, 1, has_cls=False, attn_form=1)
+    v["attn"][:] = np.random.default_rng(n).integers(0, 7, v["attn"].shape).astype(np.float32)
+    g = gpu_prune(v, n // 2, 0, has_cls=False, attn_form=1, n_clusters=1, anchor_ratio=1.0)
+    np.testing.assert_array_equal(g["keep_idx"][0], op.select_anchors(v["attn"][0, 0].astype(np.float64), n // 2))
