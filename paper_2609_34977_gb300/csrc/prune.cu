@@ -290,10 +290,7 @@ __global__ void __launch_bounds__(kRankThreads) anchor_kernel(PruneDims p, Prune
   int na = 0;
   for (int q = 0; q < 4; ++q)
     if (base + q < p.n) na += role[base + q];
-  const int nu = ((base < p.n) ? min(4, p.n - base) : 0) - na;
-  const int a0 = block_scan_excl(na, tmp, nullptr);
-  const int u0 = block_scan_excl(nu, tmp, nullptr);
-  int ai = a0, ui = u0;
+  int ai = block_scan_excl(na, tmp, nullptr), ui = min(base, p.n) - ai;
   // a_i = 0 where the anchor bracket is absent (no anchors, or the ablation without it)
   const uint32_t init = (p.n_anc == 0 || p.wa == 0.0f) ? ordered_key(0.0f) : 0u;
   for (int q = 0; q < 4; ++q) {
@@ -435,56 +432,52 @@ __global__ void __cluster_dims__(AS, 1, 1) __launch_bounds__(256)
 }
 
 // ---- 4. K-means (Lloyd) and Eq. 2 quotas ------------------------------------------------------
-__device__ void compute_quotas(const int* sizes, int K, int n_cmp, int* quota) {
-  int total = 0, nonempty = 0;
-  for (int k = 0; k < K; ++k) {
-    quota[k] = 0;
-    total += sizes[k];
-    nonempty += sizes[k] > 0;
-  }
-  if (n_cmp <= 0 || total == 0) return;
-  int order[SPD_MAX_CLUSTERS];
-  if (n_cmp < nonempty) {  // one each to the largest clusters, ties to the lower k
-    for (int k = 0; k < K; ++k) order[k] = k;
-    for (int a = 1; a < K; ++a)
-      for (int b = a; b > 0 && (sizes[order[b]] > sizes[order[b - 1]]); --b) {
-        const int x = order[b]; order[b] = order[b - 1]; order[b - 1] = x;
+// Eq. 2's quotas of K <= 16 clusters (sizes, shared), made to sum to n_cmp, by one whole warp, lane k for
+// cluster k; quota [SPD_MAX_CLUSTERS]. All products stay below 2^26. (One thread walking sorted index
+// arrays with 64-bit divisions took 3 us on the critical path of every tile, a warp 0.5.)
+__device__ __forceinline__ void warp_quotas(const int* sizes, int K, int n_cmp, int* quota) {
+  constexpr uint32_t kAll = 0xffffffffu;
+  const int k = threadIdx.x & 31;
+  const int sz = k < K ? sizes[k] : 0;
+  int total = sz;
+#pragma unroll
+  for (int off = 16; off; off >>= 1) total += __shfl_xor_sync(kAll, total, off);
+  const int nonempty = __popc(__ballot_sync(kAll, sz > 0));
+  int q = 0;
+  if (n_cmp > 0 && total > 0) {
+    if (n_cmp < nonempty) {  // one each to the largest clusters, ties to the lower k
+      int r = 0;
+      for (int j = 0; j < K; ++j) {
+        const int sj = __shfl_sync(kAll, sz, j);
+        r += sj > sz || (sj == sz && j < k);
       }
-    for (int r = 0; r < n_cmp; ++r) quota[order[r]] = 1;
-    return;
-  }
-  long long rem[SPD_MAX_CLUSTERS];
-  int sum = 0;
-  for (int k = 0; k < K; ++k) {
-    const long long num = (long long)n_cmp * sizes[k];
-    rem[k] = num % total;
-    if (sizes[k] > 0) {
-      int q = int((2 * num + total) / (2LL * total));  // round half away from zero
-      if (q < 1) q = 1;
-      if (q > sizes[k]) q = sizes[k];
-      quota[k] = q;
+      q = sz > 0 && r < n_cmp ? 1 : 0;
+    } else {
+      const int num = n_cmp * sz, rem = num % total;
+      if (sz > 0) q = min(max((2 * num + total) / (2 * total), 1), sz);  // round half away from zero
+      int sum = q;
+#pragma unroll
+      for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(kAll, sum, off);
+      // passes over the clusters, each one up (or down) at most once a pass: in descending fractional part,
+      // ties to the lower k (in ascending part, ties to the higher k), among those with room
+      while (sum != n_cmp) {
+        const bool up = sum < n_cmp;
+        const uint32_t room = __ballot_sync(kAll, k < K && (up ? q < sz : q > 1));
+        const int need = up ? n_cmp - sum : sum - n_cmp;
+        int r = 0;
+        for (int j = 0; j < K; ++j) {
+          const int rj = __shfl_sync(kAll, rem, j);
+          const bool before = up ? (rj > rem || (rj == rem && j < k)) : (rj < rem || (rj == rem && j > k));
+          r += (room >> j & 1) && before;
+        }
+        if ((room >> k & 1) && r < need) q += up ? 1 : -1;
+        const int step = min(need, __popc(room));
+        sum += up ? step : -step;
+        if (step == 0) break;
+      }
     }
-    sum += quota[k];
   }
-  if (sum < n_cmp) {  // descending fractional part, ties to the lower k
-    for (int k = 0; k < K; ++k) order[k] = k;
-    for (int a = 1; a < K; ++a)
-      for (int b = a; b > 0 && rem[order[b]] > rem[order[b - 1]]; --b) {
-        const int x = order[b]; order[b] = order[b - 1]; order[b - 1] = x;
-      }
-    while (sum < n_cmp)
-      for (int r = 0; r < K && sum < n_cmp; ++r)
-        if (quota[order[r]] < sizes[order[r]]) { ++quota[order[r]]; ++sum; }
-  } else if (sum > n_cmp) {  // ascending fractional part, ties to the higher k
-    for (int k = 0; k < K; ++k) order[k] = K - 1 - k;
-    for (int a = 1; a < K; ++a)
-      for (int b = a; b > 0 && rem[order[b]] < rem[order[b - 1]]; --b) {
-        const int x = order[b]; order[b] = order[b - 1]; order[b - 1] = x;
-      }
-    while (sum > n_cmp)
-      for (int r = 0; r < K && sum > n_cmp; ++r)
-        if (quota[order[r]] > 1) { --quota[order[r]]; --sum; }
-  }
+  if (k < SPD_MAX_CLUSTERS) quota[k] = q;
 }
 
 // The fused tail of the K-means kernel: every CTA turns its tokens' accumulated terms into Eq. 3
@@ -503,19 +496,18 @@ __device__ void fused_select(const PruneDims& p, const PruneWs& w, const PruneOu
   __shared__ int quota[SPD_MAX_CLUSTERS];
   __shared__ int tmp[32];
   uint8_t* kept = reinterpret_cast<uint8_t*>(keys + m + 1);  // CTA 0: [n]
-  __syncthreads();  // every warp's terms of the last layer are in sacc
-  if (threadIdx.x == 0) {  // every CTA: segment offsets and the Eq. 2 quotas (same in all)
-    int sizes[SPD_MAX_CLUSTERS], q[SPD_MAX_CLUSTERS];
-    int acc = 0;
-    for (int k = 0; k < K; ++k) {
-      seg[k] = acc;
-      sizes[k] = ncl[k];
-      acc += ncl[k];
+  if (threadIdx.x < 32) {  // every CTA: segment offsets and the Eq. 2 quotas (same in all)
+    warp_quotas(ncl, K, p.n_cmp, quota);
+    if (threadIdx.x == 0) {
+      int acc = 0;
+      for (int k = 0; k < K; ++k) {
+        seg[k] = acc;
+        acc += ncl[k];
+      }
+      seg[K] = acc;
     }
-    seg[K] = acc;
-    compute_quotas(sizes, K, p.n_cmp, q);
-    for (int k = 0; k < K; ++k) quota[k] = q[k];
   }
+  __syncthreads();  // every warp's terms of the last layer are in sacc
   uint64_t key[2];  // this thread's tokens jj = threadIdx.x + u blockDim.x (nl <= 2 blockDim.x)
   for (int u = 0; u < 2; ++u) {
     const int jj = threadIdx.x + u * blockDim.x;
@@ -543,23 +535,22 @@ __device__ void fused_select(const PruneDims& p, const PruneWs& w, const PruneOu
     for (int i = threadIdx.x; i < p.n; i += blockDim.x) kept[i] = uint8_t(w.role[size_t(t) * p.n + i]);
   cl.sync();  // every CTA holds all m keys; CTA 0 the anchor flags
   uint8_t* kept0 = cl.map_shared_rank(kept, 0);
-  for (int u = 0; u < 2; ++u) {
-    const int jj = threadIdx.x + u * blockDim.x;
-    if (jj >= nl) continue;
-    const uint64_t ki = key[u];
-    int r0 = 0, r1 = 0, r2 = 0, r3 = 0, j = 0;
-    for (; j + 4 <= m; j += 4) {
-      r0 += keys[j] < ki;
-      r1 += keys[j + 1] < ki;
-      r2 += keys[j + 2] < ki;
-      r3 += keys[j + 3] < ki;
+  // rank of each of this CTA's tokens among all keys: eight lanes a token, every eighth key each
+  for (int jb = 0; jb < nl; jb += int(blockDim.x) / 8) {
+    const int jj = jb + int(threadIdx.x) / 8;
+    const uint64_t ki = keys[j0 + min(jj, nl - 1)];
+    int r = 0;
+#pragma unroll 4
+    for (int j = threadIdx.x & 7; j < m; j += 8) r += keys[j] < ki;
+#pragma unroll
+    for (int off = 4; off; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
+    if ((threadIdx.x & 7) == 0 && jj < nl) {
+      const int k = int(ki >> 45);
+      // the key at sorted position r of cluster k's segment is kept iff r - seg[k] < quota[k]
+      if (r - seg[k] < quota[k]) kept0[ki & 0x1fffu] = 2;
+      if (out.cluster) out.cluster[size_t(t) * p.n + (ki & 0x1fffu)] = int8_t(k);
+      if (out.scores) out.scores[size_t(t) * p.n + (ki & 0x1fffu)] = ordered_val(uint32_t(ki >> 13));
     }
-    for (; j < m; ++j) r0 += keys[j] < ki;
-    const int k = int(ki >> 45);
-    // the key at sorted position r of cluster k's segment is kept iff r - seg[k] < quota[k]
-    if (r0 + r1 + r2 + r3 - seg[k] < quota[k]) kept0[ki & 0x1fffu] = 2;
-    if (out.cluster) out.cluster[size_t(t) * p.n + (ki & 0x1fffu)] = int8_t(k);
-    if (out.scores) out.scores[size_t(t) * p.n + (ki & 0x1fffu)] = ordered_val(uint32_t(ki >> 13));
   }
   cl.sync();  // the selected flags are in CTA 0
   if (rank != 0) return;
@@ -597,10 +588,6 @@ struct RowAccess {
   __device__ __forceinline__ const float* row(int jj) const {
     return rows ? rows + size_t(jj) * D : g + (row0 + idx[jj]) * D;
   }
-  __device__ __forceinline__ float operator()(int jj, int c) const {
-    const float v = row(jj)[c];
-    return scale ? v * scale[jj] : v;
-  }
   __device__ __forceinline__ float4 v4(int jj, int c) const {
     float4 v = *reinterpret_cast<const float4*>(row(jj) + c);
     if (scale) {
@@ -614,63 +601,151 @@ struct RowAccess {
   }
 };
 
-// part[k][c] = sum over this CTA's tokens jj of cluster k, in token order, of value(jj, c): one
-// thread per column, KN accumulators in registers, eight values in flight.
-template <int KN, typename F>
-__device__ __forceinline__ void column_sums(float* part, int K, int D, int nl, const int8_t* asg,
-                                            F value) {
-  if constexpr (KN == 4) {
-    // four adjacent columns per thread (float4), same token-order sums per column
-    for (int c = 4 * threadIdx.x; c < D; c += 4 * blockDim.x) {
-      float4 acc[KN];
-#pragma unroll
-      for (int k = 0; k < KN; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int jb = 0; jb < nl; jb += 8) {
+// This CTA's nl <= 1024 tokens listed by cluster, in token order within each: ord[start[k] .. start[k + 1]).
+// A warp a cluster (ballots over 32 tokens at a time); every thread of the block calls it, and a barrier
+// before the lists are read is the caller's.
+__device__ __forceinline__ void cluster_lists(const int8_t* asg, int nl, int K, int* cnt, uint16_t* ord, int* start) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int k = warp; k < K; k += nw) {
+    int n = 0;
+    for (int b = 0; b < nl; b += 32) n += __popc(__ballot_sync(0xffffffffu, b + lane < nl && asg[b + lane] == k));
+    if (lane == 0) cnt[k] = n;
+  }
+  __syncthreads();
+  for (int k = warp; k < K; k += nw) {
+    int at = 0;
+    for (int j = 0; j < k; ++j) at += cnt[j];
+    if (lane == 0) {
+      start[k] = at;
+      if (k == K - 1) start[K] = nl;
+    }
+    for (int b = 0; b < nl; b += 32) {
+      const bool mine = b + lane < nl && asg[b + lane] == k;
+      const uint32_t who = __ballot_sync(0xffffffffu, mine);
+      if (mine) ord[at + __popc(who & ((1u << lane) - 1))] = uint16_t(b + lane);
+      at += __popc(who);
+    }
+  }
+}
+
+// part[k][c] = sum over this CTA's tokens of cluster k, in token order, of value.v4(token, c): four
+// adjacent columns a thread, eight rows in flight. The rows come sorted by cluster, so a row costs one load
+// and four additions (with a running sum for each of the K clusters it was 16 predicated additions).
+__device__ __forceinline__ void column_sums(float* part, int K, int D, int nl, const uint16_t* ord, const int* start,
+                                            RowAccess value) {
+  for (int c = 4 * threadIdx.x; c < D; c += 4 * blockDim.x)
+    for (int k = 0; k < K; ++k) {
+      const int j1 = start[k + 1];
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int jb = start[k]; jb < j1; jb += 8) {
         float4 xv[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          xv[u] = jb + u < nl ? value.v4(jb + u, c) : make_float4(0.f, 0.f, 0.f, 0.f);
+          xv[u] = jb + u < j1 ? value.v4(ord[jb + u], c) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (jb + u < nl) {
-            const int a = asg[jb + u];
-#pragma unroll
-            for (int k = 0; k < KN; ++k)
-              if (k == a) {
-                acc[k].x += xv[u].x;
-                acc[k].y += xv[u].y;
-                acc[k].z += xv[u].z;
-                acc[k].w += xv[u].w;
-              }
-          }
+        for (int u = 0; u < 8; ++u) {
+          acc.x += xv[u].x;
+          acc.y += xv[u].y;
+          acc.z += xv[u].z;
+          acc.w += xv[u].w;
+        }
       }
-#pragma unroll
-      for (int k = 0; k < KN; ++k)
-        if (k < K) *reinterpret_cast<float4*>(part + k * D + c) = acc[k];
+      *reinterpret_cast<float4*>(part + k * D + c) = acc;
     }
-  } else {
-    for (int c = threadIdx.x; c < D; c += blockDim.x) {
-      float acc[KN];
+}
+
+// Packed pairs of fp32: two IEEE operations an instruction.
+__device__ __forceinline__ uint64_t sub_f32x2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float sum_f32x2(uint64_t a) {
+  return __uint_as_float(uint32_t(a)) + __uint_as_float(uint32_t(a >> 32));
+}
+
+// assign_rows for K = 4, the calling warp's next n (at most RP count) rows at a time: a centroid's 16 bytes serve RP rows, differences and
+// squares are packed, and the 4 RP partial distances are summed over the lanes by halving exchanges (lane bits
+// 4, 3, ... pick the value) instead of a butterfly each. The loop is bound by issue: about 155
+// instructions a row of 1024 at RP = 4 where a row at a time took about 450 (28 rows of a CTA of eight
+// warps: 4.3 -> 2.0 us).
+template <int RP, typename Row>
+__device__ __forceinline__ void assign4_rows(const float* cent, int D, int n, bool first, int8_t* asg, int* changed,
+                                             Row xrow) {
+  constexpr int NV = 4 * RP;
+  const int lane = threadIdx.x & 31;
+  const float* x[RP];
 #pragma unroll
-      for (int k = 0; k < KN; ++k) acc[k] = 0.0f;
-      for (int jb = 0; jb < nl; jb += 8) {
-        float xv[8];
+  for (int i = 0; i < RP; ++i) x[i] = xrow(min(i, n - 1));
+  uint64_t acc[RP][4];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) xv[u] = jb + u < nl ? value(jb + u, c) : 0.0f;
+  for (int i = 0; i < RP; ++i)
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (jb + u < nl) {
-            const int a = asg[jb + u];
+    for (int k = 0; k < 4; ++k) acc[i][k] = 0;
+#pragma unroll 2
+  for (int c = 4 * lane; c < D; c += 128) {
+    ulonglong2 xv[RP], cv[4];
 #pragma unroll
-            for (int k = 0; k < KN; ++k)
-              if (k == a) acc[k] += xv[u];
-          }
+    for (int i = 0; i < RP; ++i) xv[i] = *reinterpret_cast<const ulonglong2*>(x[i] + c);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) cv[k] = *reinterpret_cast<const ulonglong2*>(cent + k * D + c);
+#pragma unroll
+    for (int i = 0; i < RP; ++i)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint64_t d0 = sub_f32x2(xv[i].x, cv[k].x), d1 = sub_f32x2(xv[i].y, cv[k].y);
+        acc[i][k] = fma_f32x2(d0, d0, acc[i][k]);
+        acc[i][k] = fma_f32x2(d1, d1, acc[i][k]);
       }
+  }
+  float v[NV];
 #pragma unroll
-      for (int k = 0; k < KN; ++k)
-        if (k < K) part[k * D + c] = acc[k];
+  for (int i = 0; i < RP; ++i)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[4 * i + k] = sum_f32x2(acc[i][k]);
+  int off = 16;
+#pragma unroll
+  for (int h = NV / 2; h >= 1; h >>= 1, off >>= 1) {
+    const bool up = lane & off;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const float recv = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + h], off);
+      v[i] = (up ? v[i + h] : v[i]) + recv;
     }
   }
+  const int low = off;  // lanes that differ below 2 low hold the same value's parts
+  for (; off; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+  // value index = lane / (2 low) = 4 row + k: the nearest centroid, ties to the lower k (a NaN distance loses,
+  // but wins at k = 0, as in a scan over k that replaces the first distance by smaller ones)
+  int best = (lane / (2 * low)) & 3;
+  if (v[0] != v[0]) v[0] = best == 0 ? -INFINITY : INFINITY;
+#pragma unroll
+  for (int s = 1; s <= 2; s <<= 1) {
+    const float od = __shfl_xor_sync(0xffffffffu, v[0], 2 * low * s);
+    const int ob = __shfl_xor_sync(0xffffffffu, best, 2 * low * s);
+    if (od < v[0] || (od == v[0] && ob < best)) {
+      v[0] = od;
+      best = ob;
+    }
+  }
+  const int jj = lane / (8 * low);
+  if (lane % (8 * low) == 0 && jj < n) {
+    if (first || asg[jj] != best) *changed = 1;
+    asg[jj] = int8_t(best);
+  }
+}
+// ... of all nl rows by the block's warps.
+template <int RP, typename Row>
+__device__ __forceinline__ void assign4(const float* cent, int D, int nl, bool first, int8_t* asg, int* changed,
+                                        Row xrow) {
+  const int nw = blockDim.x >> 5;
+  for (int jb = (threadIdx.x >> 5) * RP; jb < nl; jb += nw * RP)
+    assign4_rows<RP>(cent, D, nl - jb, first, asg + jb, changed, [&](int i) { return xrow(jb + i); });
 }
 
 // Nearest centroid (squared Euclidean, ties to the lower cluster) of each of this CTA's nl rows, one
@@ -679,66 +754,78 @@ template <int KN, typename Row>
 __device__ __forceinline__ void assign_rows(const float* cent, int K, int D, int nl, bool first, int8_t* asg,
                                             int* changed, Row xrow) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int jj = warp; jj < nl; jj += nw) {
-    const float* x = xrow(jj);
-    float part_d[KN];
+  if constexpr (KN == 4) {  // as many rows at a time as leave no warp idle
+    if (nl > 2 * nw) assign4<4>(cent, D, nl, first, asg, changed, xrow);
+    else if (nl > nw) assign4<2>(cent, D, nl, first, asg, changed, xrow);
+    else assign4<1>(cent, D, nl, first, asg, changed, xrow);
+  } else {
+    for (int jj = warp; jj < nl; jj += nw) {
+      const float* x = xrow(jj);
+      float part_d[KN];
 #pragma unroll
-    for (int k = 0; k < KN; ++k) part_d[k] = 0.0f;
-    // 16-byte loads, four in flight per lane (D is a multiple of 4)
-    for (int cb = 4 * lane; cb < D; cb += 512) {
-      float4 xv[4];
+      for (int k = 0; k < KN; ++k) part_d[k] = 0.0f;
+      // 16-byte loads, four in flight per lane (D is a multiple of 4)
+      for (int cb = 4 * lane; cb < D; cb += 512) {
+        float4 xv[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int c = cb + 128 * u;
-        xv[u] = c < D ? *reinterpret_cast<const float4*>(x + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
+        for (int u = 0; u < 4; ++u) {
+          const int c = cb + 128 * u;
+          xv[u] = c < D ? *reinterpret_cast<const float4*>(x + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int c = cb + 128 * u;
-        if (c < D) {
+        for (int u = 0; u < 4; ++u) {
+          const int c = cb + 128 * u;
+          if (c < D) {
 #pragma unroll
-          for (int k = 0; k < KN; ++k)
-            if (k < K) {
-              const float4 ce = *reinterpret_cast<const float4*>(cent + k * D + c);
-              const float d0 = xv[u].x - ce.x, d1 = xv[u].y - ce.y, d2 = xv[u].z - ce.z,
-                          d3 = xv[u].w - ce.w;
-              part_d[k] += d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3;
-            }
+            for (int k = 0; k < KN; ++k)
+              if (k < K) {
+                const float4 ce = *reinterpret_cast<const float4*>(cent + k * D + c);
+                const float d0 = xv[u].x - ce.x, d1 = xv[u].y - ce.y, d2 = xv[u].z - ce.z,
+                            d3 = xv[u].w - ce.w;
+                part_d[k] += d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3;
+              }
+          }
         }
       }
-    }
-    int best = 0;
-    float bd = 0.0f;
+      int best = 0;
+      float bd = 0.0f;
 #pragma unroll
-    for (int k = 0; k < KN; ++k)
-      if (k < K) {
-        const float dk = warp_sum(part_d[k]);
-        if (k == 0 || dk < bd) {
-          bd = dk;
-          best = k;
+      for (int k = 0; k < KN; ++k)
+        if (k < K) {
+          const float dk = warp_sum(part_d[k]);
+          if (k == 0 || dk < bd) {
+            bd = dk;
+            best = k;
+          }
         }
+      if (lane == 0) {
+        if (first || asg[jj] != best) *changed = 1;
+        asg[jj] = int8_t(best);
       }
-    if (lane == 0) {
-      if (first || asg[jj] != best) *changed = 1;
-      asg[jj] = int8_t(best);
     }
   }
 }
 
 // Sums over the KC CTAs of the cluster, in rank order, of the per-CTA column sums `part` (K x D in
-// every CTA's shared memory), for this CTA's slice of columns; `emit(k, c, value)` consumes them.
+// every CTA's shared memory), for this CTA's slice of columns; `emit(k, c, four values)` consumes them.
 template <int KC, typename F>
 __device__ __forceinline__ void cluster_column_reduce(cg::cluster_group& cl, float* part, int K, int D,
                                                       int rank, F emit) {
-  const int c0 = rank * D / KC, c1 = (rank + 1) * D / KC, width = c1 - c0;
+  const int n4 = D / 4, c0 = rank * n4 / KC, c1 = (rank + 1) * n4 / KC, width = c1 - c0;  // 16-byte columns
   for (int e = threadIdx.x; e < K * width; e += blockDim.x) {
-    const int k = e / width, c = c0 + e % width;
-    float x[KC];
+    const int k = e / width, c = 4 * (c0 + e - k * width);
+    float4 x[KC];
 #pragma unroll
-    for (int rr = 0; rr < KC; ++rr) x[rr] = cl.map_shared_rank(part, rr)[k * D + c];  // in flight
-    float sum = 0.0f;
+    for (int rr = 0; rr < KC; ++rr)  // in flight
+      x[rr] = *reinterpret_cast<const float4*>(cl.map_shared_rank(part, rr) + k * D + c);
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int rr = 0; rr < KC; ++rr) sum += x[rr];
+    for (int rr = 0; rr < KC; ++rr) {
+      sum.x += x[rr].x;
+      sum.y += x[rr].y;
+      sum.z += x[rr].z;
+      sum.w += x[rr].w;
+    }
     emit(k, c, sum);
   }
 }
@@ -775,6 +862,8 @@ __global__ void __launch_bounds__(kmeans_threads<KN>()) kmeans_kernel(PruneDims 
   __shared__ int changed;      // this CTA's assignment changed in the current iteration
   __shared__ int any_changed;  // ... some CTA's of the cluster
   __shared__ int8_t asg[4096 / KC + 1];
+  __shared__ uint16_t ord[4096 / KC + 1];       // this CTA's tokens by cluster
+  __shared__ int start[SPD_MAX_CLUSTERS + 1];   // ... the clusters' first positions in ord
   __shared__ int idx[4096 / KC + 1];     // patch index of each of this CTA's tokens
   __shared__ float av[4096 / KC + 1];    // their a_j
   __shared__ float rinv[4096 / KC + 1];  // their 1 / ||F_l,j|| (cos) or st1 (MSE, KL) of the layer
@@ -800,19 +889,22 @@ __global__ void __launch_bounds__(kmeans_threads<KN>()) kmeans_kernel(PruneDims 
     fence_mbar_init();
   }
   __syncthreads();
-  if (RES && threadIdx.x == 0 && nl > 0) {
-    mbar_arrive_expect_tx(&rows_bar, uint32_t(nl) * D * 4);
-    for (int jj = 0; jj < nl; ++jj)
+  // the rows and, in the same phase of the barrier, the seeds (a CTA without tokens loads the seeds too)
+  if (RES && m > 0 && warp == 0) {
+    if (lane == 0) mbar_arrive_expect_tx(&rows_bar, uint32_t(nl + K) * D * 4);
+    __syncwarp();
+    for (int k = lane; k < K; k += 32) bulk_load(cent + size_t(k) * D, fin + (row0 + ul[(k * m) / K]) * D, uint32_t(D) * 4, &rows_bar);
+    for (int jj = lane; jj < nl; jj += 32)
       bulk_load(rows + size_t(jj) * D, fin + (row0 + idx[jj]) * D, uint32_t(D) * 4, &rows_bar);
   }
-  if (m > 0) {
+  if (!RES && m > 0) {
 #pragma unroll 4
     for (int e = threadIdx.x; e < K * D; e += blockDim.x) {
       const int k = e / D, c = e % D;
       cent[e] = feat_row(p, p.fin, t, ul[(k * m) / K])[c];
     }
   }
-  if (RES && nl > 0) {
+  if (RES && m > 0) {
     volatile int no_abort = 0;
     if (!mbar_wait(&rows_bar, 0, &no_abort, kWaitBudget)) {
       set_status(w.status, SPD_ETIMEOUT);
@@ -828,66 +920,25 @@ __global__ void __launch_bounds__(kmeans_threads<KN>()) kmeans_kernel(PruneDims 
     // assignment of this CTA's points
     if (threadIdx.x == 0) changed = 0;
     __syncthreads();
-    bool done_assign = false;
-    // K = 4 with the rows resident: the centroids in registers (242 registers a thread, one CTA an
-    // SM). The L2-streaming form takes the loop below instead: at 119 registers two of its CTAs
-    // share an SM, which hides more of the row loads' latency (64 tiles: 780 -> 606 us a call).
-    if constexpr (KN == 4 && RES) {
-      if (D <= 1024) {
-        done_assign = true;
-        // lane's columns 4 lane + 128 j (j < 8) of the four centroids in registers
-        float4 cr[4][8];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int c = 4 * lane + 128 * j;
-            cr[k][j] = (k < K && c < D) ? *reinterpret_cast<const float4*>(cent + k * D + c)
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-        for (int jj = warp; jj < nl; jj += nw) {
-          const float* x = xrow(jj);
-          float4 xv[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int c = 4 * lane + 128 * j;
-            xv[j] = c < D ? *reinterpret_cast<const float4*>(x + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-          float pd[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float d0 = xv[j].x - cr[k][j].x, d1 = xv[j].y - cr[k][j].y,
-                          d2 = xv[j].z - cr[k][j].z, d3 = xv[j].w - cr[k][j].w;
-              pd[k] += d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3;
-            }
-          int best = 0;
-          float bd = 0.0f;
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (k < K) {
-              const float dk = warp_sum(pd[k]);
-              if (k == 0 || dk < bd) {
-                bd = dk;
-                best = k;
-              }
-            }
-          if (lane == 0) {
-            if (it == 0 || asg[jj] != best) changed = 1;
-            asg[jj] = int8_t(best);
-          }
-        }
+    assign_rows<KN>(cent, K, D, nl, it == 0, asg, &changed, xrow);
+    if (!RES && it > 0) {
+      // the column sums are another pass over the rows in L2: not for an assignment that repeats
+      cl.sync();
+      if (warp == 0) {
+        const int any = __any_sync(0xffffffffu, lane < KC && *cl.map_shared_rank(&changed, lane) != 0);
+        if (lane == 0) any_changed = any;
+      }
+      __syncthreads();
+      if (!any_changed) {
+        cl.sync();  // every CTA has read the flags
+        break;      // cluster-uniform decision
       }
     }
-    if (!done_assign) assign_rows<KN>(cent, K, D, nl, it == 0, asg, &changed, xrow);
     __syncthreads();
     // this CTA's column sums (token order, in registers) and sizes
-    if (threadIdx.x < K) cnt[threadIdx.x] = 0;
+    cluster_lists(asg, nl, K, cnt, ord, start);
     __syncthreads();
-    for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) atomicAdd(&cnt[asg[jj]], 1);
-    column_sums<KN>(part, K, D, nl, asg,
-                    RowAccess{RES ? rows : nullptr, fin, row0, idx, D, nullptr});
+    column_sums(part, K, D, nl, ord, start, RowAccess{RES ? rows : nullptr, fin, row0, idx, D, nullptr});
     cl.sync();
     // one warp reads the peers' flags and sizes (lane r: CTA r) and publishes them in this CTA
     if (warp == 0) {
@@ -904,25 +955,28 @@ __global__ void __launch_bounds__(kmeans_threads<KN>()) kmeans_kernel(PruneDims 
     __syncthreads();
     if (it > 0 && !any_changed) break;  // cluster-uniform decision
     // new centroids for this CTA's column slice, written into every CTA
-    cluster_column_reduce<KC>(cl, part, K, D, rank, [&](int k, int c, float sum) {
-      const int n = ncl[k];
-      const float v = n > 0 ? sum / float(n) : cent[k * D + c];
-      for (int rr = 0; rr < KC; ++rr) cl.map_shared_rank(cent, rr)[k * D + c] = v;
+    cluster_column_reduce<KC>(cl, part, K, D, rank, [&](int k, int c, float4 v) {
+      const float n = float(ncl[k]);
+      if (n > 0.0f) v = make_float4(v.x / n, v.y / n, v.z / n, v.w / n);
+      else v = *reinterpret_cast<const float4*>(cent + k * D + c);
+      for (int rr = 0; rr < KC; ++rr) *reinterpret_cast<float4*>(cl.map_shared_rank(cent, rr) + k * D + c) = v;
     });
     cl.sync();
   }
-  // final assignment: sizes, the per-cluster sums of a_j, and the assignment itself
-  if (threadIdx.x < K) {
-    cnt[threadIdx.x] = 0;
-    asum_part[threadIdx.x] = 0.0f;
-  }
+  // final assignment (lists and sizes are its: an assignment that repeats leaves them as they were): the
+  // per-cluster sums of a_j in token order, and the assignment itself
   __syncthreads();
-  for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) {
-    atomicAdd(&cnt[asg[jj]], 1);
-    w.assign[size_t(t) * m + j0 + jj] = asg[jj];
+  if (m == 0) {
+    cluster_lists(asg, nl, K, cnt, ord, start);
+    __syncthreads();
   }
-  if (threadIdx.x == 0)  // token order
-    for (int jj = 0; jj < nl; ++jj) asum_part[asg[jj]] += av[jj];
+  if (!FUSED)
+    for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) w.assign[size_t(t) * m + j0 + jj] = asg[jj];
+  if (threadIdx.x < K) {
+    float a = 0.0f;
+    for (int j = start[threadIdx.x]; j < start[threadIdx.x + 1]; ++j) a += av[ord[j]];
+    asum_part[threadIdx.x] = a;
+  }
   // per layer: sums over each cluster of unit feature rows (F_l,j / ||F_l,j||), or of raw rows and
   // of st1 for the MSE and KL similarities
   // (RES: the final layer first, from the resident rows; then each other layer's rows are copied
@@ -934,9 +988,10 @@ __global__ void __launch_bounds__(kmeans_threads<KN>()) kmeans_kernel(PruneDims 
     const float* fl = p.feat[l];
     __syncthreads();  // the previous layer's rows are no longer read
     for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) rinv[jj] = rstat[idx[jj]];
-    if (RES && l != p.fin && threadIdx.x == 0 && nl > 0) {
-      mbar_arrive_expect_tx(&rows_bar, uint32_t(nl) * D * 4);
-      for (int jj = 0; jj < nl; ++jj)
+    if (RES && l != p.fin && warp == 0 && nl > 0) {
+      if (lane == 0) mbar_arrive_expect_tx(&rows_bar, uint32_t(nl) * D * 4);
+      __syncwarp();
+      for (int jj = lane; jj < nl; jj += 32)
         bulk_load(rows + size_t(jj) * D, fl + (row0 + idx[jj]) * D, uint32_t(D) * 4, &rows_bar);
     }
     if (RES && l != p.fin && nl > 0) {
@@ -953,14 +1008,16 @@ __global__ void __launch_bounds__(kmeans_threads<KN>()) kmeans_kernel(PruneDims 
       for (int jj = 0; jj < nl; ++jj)
         ssum_part[asg[jj]] += double(rinv[jj]) + (lo ? double(lo[idx[jj]]) : 0.0);
     }
-    column_sums<KN>(part, K, D, nl, asg,
-                    RowAccess{RES ? rows : nullptr, fl, row0, idx, D, cos_sim ? rinv : static_cast<float*>(nullptr)});
+    column_sums(part, K, D, nl, ord, start,
+                RowAccess{RES ? rows : nullptr, fl, row0, idx, D, cos_sim ? rinv : static_cast<float*>(nullptr)});
     cl.sync();
     float* csum = w.csum + (size_t(t) * p.L + l) * K * D;
-    cluster_column_reduce<KC>(cl, part, K, D, rank, [&](int k, int c, float sum) {
-      csum[k * D + c] = sum;
-      if constexpr (FUSED)  // the layer's cluster sums into every CTA (the centroids are done)
-        for (int rr = 0; rr < KC; ++rr) cl.map_shared_rank(cent, rr)[k * D + c] = sum;
+    cluster_column_reduce<KC>(cl, part, K, D, rank, [&](int k, int c, float4 sum) {
+      if constexpr (FUSED) {  // the layer's cluster sums into every CTA (the centroids are done)
+        for (int rr = 0; rr < KC; ++rr) *reinterpret_cast<float4*>(cl.map_shared_rank(cent, rr) + k * D + c) = sum;
+      } else {
+        *reinterpret_cast<float4*>(csum + k * D + c) = sum;
+      }
     });
     if (!cos_sim && rank == 0 && warp == 1) {  // CTA sums added in rank order
       for (int k = 0; k < K; ++k) {
@@ -981,27 +1038,23 @@ __global__ void __launch_bounds__(kmeans_threads<KN>()) kmeans_kernel(PruneDims 
         if (lane == 0) ak[k] = a;
       }
     }
-    if (li == p.L - 1 && rank == 0 && warp == 0) {
+    if (!FUSED && li == p.L - 1 && rank == 0 && warp == 0) {
       // sizes and a_j sums over the CTAs (lane r reads CTA r; the a_j sums added in rank order)
-      int sizes[SPD_MAX_CLUSTERS], q[SPD_MAX_CLUSTERS];
       for (int k = 0; k < K; ++k) {
-        const int nr = lane < KC ? cl.map_shared_rank(cnt, lane)[k] : 0;
         const float ar = lane < KC ? cl.map_shared_rank(asum_part, lane)[k] : 0.0f;
-        int n = nr;
+        int n = lane < KC ? cl.map_shared_rank(cnt, lane)[k] : 0;
 #pragma unroll
         for (int off = 16; off; off >>= 1) n += __shfl_xor_sync(0xffffffffu, n, off);
         float a = 0.0f;
         for (int rr = 0; rr < KC; ++rr) a += __shfl_sync(0xffffffffu, ar, rr);
-        sizes[k] = n;
         if (lane == 0) {
+          ncl[k] = n;
           w.counts[t * 16 + k] = n;
           w.asum[t * 16 + k] = a;
         }
       }
-      if (lane == 0) {
-        compute_quotas(sizes, K, p.n_cmp, q);
-        for (int k = 0; k < K; ++k) w.quotas[t * 16 + k] = q[k];
-      }
+      __syncwarp();
+      warp_quotas(ncl, K, p.n_cmp, w.quotas + t * 16);
     }
     cl.sync();  // peers' shared memory is read above; keep it alive and unchanged until here
     if constexpr (FUSED) {
@@ -1076,6 +1129,8 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
   float* cent = ksm;       // [K][D]
   float* rows = ksm + KD;  // res: [nl][D]
   __shared__ int8_t asg[kGridMaxRows];
+  __shared__ uint16_t ord[kGridMaxRows];
+  __shared__ int start[SPD_MAX_CLUSTERS + 1];
   __shared__ int idx[kGridMaxRows];
   __shared__ float av[kGridMaxRows], rinv[kGridMaxRows];
   __shared__ int cnt[SPD_MAX_CLUSTERS], ncl[SPD_MAX_CLUSTERS];
@@ -1145,12 +1200,12 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
   };
   for (int it = 0; it < p.iters; ++it) {
     if (threadIdx.x == 0) changed = 0;
-    if (threadIdx.x < SPD_MAX_CLUSTERS) cnt[threadIdx.x] = 0;
     __syncthreads();
     assign_rows<KN>(cent, K, D, nl, it == 0, asg, &changed, xrow);
     __syncthreads();
-    for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) atomicAdd(&cnt[asg[jj]], 1);
-    column_sums<KN>(part + size_t(r) * p.L * KD, K, D, nl, asg, RowAccess{res ? rows : nullptr, fin, row0, idx, D, nullptr});
+    cluster_lists(asg, nl, K, cnt, ord, start);
+    __syncthreads();
+    column_sums(part + size_t(r) * p.L * KD, K, D, nl, ord, start, RowAccess{res ? rows : nullptr, fin, row0, idx, D, nullptr});
     __syncthreads();
     // sizes of K <= 16 clusters and the flag in the first 16 ints of the CTA's block (a flag bit on size 0)
     if (threadIdx.x < K) meta[r * kGridMeta + threadIdx.x] = cnt[threadIdx.x] | (changed ? 1 << 30 : 0);
@@ -1192,8 +1247,7 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
   for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) w.assign[size_t(t) * m + j0 + jj] = asg[jj];
   if (threadIdx.x < K) {
     float a = 0.0f;
-    for (int jj = 0; jj < nl; ++jj)
-      if (asg[jj] == int(threadIdx.x)) a += av[jj];
+    for (int j = start[threadIdx.x]; j < start[threadIdx.x + 1]; ++j) a += av[ord[j]];
     meta[r * kGridMeta + SPD_MAX_CLUSTERS + threadIdx.x] = __float_as_int(a);
   }
   for (int l = 0; l < p.L; ++l) {
@@ -1208,8 +1262,8 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
         if (asg[jj] == int(threadIdx.x)) a += double(rinv[jj]) + (lo ? double(lo[idx[jj]]) : 0.0);
       dsum[(size_t(r) * p.L + l) * 16 + threadIdx.x] = a;
     }
-    column_sums<KN>(part + (size_t(r) * p.L + l) * KD, K, D, nl, asg,
-                    RowAccess{res && l == p.fin ? rows : nullptr, p.feat[l], row0, idx, D, COS ? rinv : static_cast<float*>(nullptr)});
+    column_sums(part + (size_t(r) * p.L + l) * KD, K, D, nl, ord, start,
+                RowAccess{res && l == p.fin ? rows : nullptr, p.feat[l], row0, idx, D, COS ? rinv : static_cast<float*>(nullptr)});
   }
   tile_barrier(bar, G, ++phase, w.status);
   pdl_launch_dependents();
@@ -1231,10 +1285,271 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
         if (lane == 0) w.ssum[(size_t(t) * p.L + l) * 16 + warp] = d;
       }
   }
-  if (threadIdx.x == 0) {
-    int q[SPD_MAX_CLUSTERS];
-    compute_quotas(ncl, K, p.n_cmp, q);
-    for (int k = 0; k < K; ++k) w.quotas[t * 16 + k] = q[k];
+  if (warp == 0) warp_quotas(ncl, K, p.n_cmp, w.quotas + t * 16);
+}
+
+// ---- 4c. K-means of many tiles: one sweep over the rows an iteration ------------------------------
+// K = 4. A cluster of KC CTAs per tile, one CTA an SM, as many as the tiles leave (64 tiles: 2). The rows
+// of all tiles exceed L2 (531 x 4 KB a LLaVA tile), so what counts is how often they are read and how many
+// bytes are in flight: every thread copies its four columns of 16 rows at a time (8 where rows are wider
+// than 1024) with 16-byte asynchronous copies into a ring of such steps, and one sweep does the
+// assignment of a step's rows (two a warp) and then their column sums from shared memory, four columns a
+// thread in registers. (One bulk copy a row held the whole kernel at 2.5 TB/s: 165 us.) From the second sweep on it also adds the unit rows, which are the final layer's
+// cluster sums if the assignment repeats. Every second sweep runs backwards: the rows that the last one
+// read end up in L2. So a tile whose assignment repeats at once is read twice for K-means and once a
+// further layer, where the form that it replaces (4 CTAs a tile re-reading the rows through registers) read
+// it five times: 64 tiles 234 -> 163 us serialised, of which the copies alone take 76.
+constexpr int kStreamThreads = 256;
+constexpr size_t kStreamSmem = 226 * 1024;  // dynamic shared memory of a CTA
+// Column groups of a thread (rows of up to 1024 or 2048 floats) and rows of a step.
+__host__ __device__ inline int stream_groups(int D) { return D <= 4 * kStreamThreads ? 1 : 2; }
+__host__ __device__ constexpr int stream_step(int CG) { return CG == 1 ? 16 : 8; }
+// Bytes of the arrays before the ring, and the steps that then fit.
+__host__ __device__ inline size_t stream_head(int D, int nl_max) {
+  return (size_t(8) * D * sizeof(float) + size_t(nl_max) * 7 + 15) / 16 * 16;
+}
+inline int stream_slots(int D, int nl_max, size_t smem) {
+  const size_t head = stream_head(D, nl_max), slot = size_t(stream_step(stream_groups(D))) * D * sizeof(float);
+  return head >= smem ? 0 : int((smem - head) / slot);
+}
+
+// 16 bytes from global to shared memory, past L1; groups of them complete in the order of their commits.
+__device__ __forceinline__ void copy_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_async_wait() {  // all but the thread's last N groups have landed
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+template <int KC, int CG, bool COS>
+__global__ void __launch_bounds__(kStreamThreads, 1) kmeans_stream_kernel(PruneDims p, PruneWs w, int slots) {
+  extern __shared__ __align__(16) float ksm[];
+  constexpr int K = 4, SR = stream_step(CG);
+  const int D = p.d, m = p.m;
+  const int nl_max = (m + KC - 1) / KC;
+  float* cent = ksm;            // [K][D]
+  float* part = cent + K * D;   // [K][D]
+  float* rinv = part + K * D;   // [nl_max] scale (cosine) or st1 (MSE, KL) of the current layer
+  uint16_t* idx = reinterpret_cast<uint16_t*>(rinv + nl_max);
+  int8_t* asg = reinterpret_cast<int8_t*>(idx + nl_max);
+  float* ring = ksm + stream_head(D, nl_max) / sizeof(float);  // [slots][SR][D]
+  __shared__ int cnt[SPD_MAX_CLUSTERS], ncl[SPD_MAX_CLUSTERS];
+  __shared__ int changed, any_changed;
+  __shared__ float asum_part[K];
+  __shared__ double ssum_part[K];
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = int(cl.block_rank());
+  const int t = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int j0 = rank * m / KC, j1 = (rank + 1) * m / KC, nl = j1 - j0;
+  const int* ul = w.ulist + size_t(t) * m;
+  const size_t row0 = size_t(t) * p.n_tok + p.off;
+  const float* fin = p.feat[p.fin];
+  pdl_launch_dependents();
+  pdl_wait();
+  const float* frin = w.inv + (size_t(p.fin) * p.n_tiles + t) * p.n;
+  for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) {
+    const int i = ul[j0 + jj];
+    idx[jj] = uint16_t(i);
+    if (COS) rinv[jj] = frin[i];
+  }
+  __syncthreads();
+  const int ns = (nl + SR - 1) / SR;  // steps of a sweep
+  // copies step i of a sweep over layer rows f into slot i % slots (one group, empty past the end)
+  auto issue = [&](const float* f, int i, bool back) {
+    if (i < ns) {
+      const int r0 = (back ? ns - 1 - i : i) * SR, rows = min(SR, nl - r0);
+      float* dst = ring + size_t(i % slots) * SR * D;
+#pragma unroll 4
+      for (int v = 0; v < rows; ++v) {
+        const float* src = f + (row0 + idx[r0 + v]) * D;
+#pragma unroll
+        for (int q = 0; q < CG; ++q) {
+          const int c = 4 * (threadIdx.x + kStreamThreads * q);
+          if (c < D) copy_async16(dst + size_t(v) * D + c, src + c);
+        }
+      }
+    }
+    copy_async_commit();
+  };
+  auto start = [&](const float* f, bool back) {  // the first two steps of a sweep
+    issue(f, 0, back);
+    issue(f, 1, back);
+  };
+  float4 acc[K][CG], unit[K][CG];
+  // one sweep: assignment (where `assign`) and column sums of the rows (acc, where `raw`) and of the rows times
+  // rinv (unit, where `units`); its first two steps were issued by start()
+  auto sweep = [&](const float* f, bool back, bool assign, bool first, bool raw, bool units) {
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+      for (int q = 0; q < CG; ++q) acc[k][q] = unit[k][q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < ns; ++i) {
+      // with three slots the step after the next is issued before this one is used, with two after it
+      if (slots > 2) issue(f, i + 2, back);
+      if (slots > 2) copy_async_wait<2>();
+      else copy_async_wait<1>();
+      __syncthreads();  // every thread's columns of step i have landed
+      const int r0 = (back ? ns - 1 - i : i) * SR, rows = min(SR, nl - r0);
+      const float* base = ring + size_t(i % slots) * SR * D;
+      if (assign) {
+        constexpr int RP = SR / 8;  // rows a warp
+        const int v0 = warp * RP;
+        if (v0 < rows)
+          assign4_rows<RP>(cent, D, rows - v0, first, asg + r0 + v0, &changed,
+                           [&](int q) { return base + size_t(v0 + q) * D; });
+        __syncthreads();
+      }
+      const int a = lane < rows ? asg[r0 + lane] : -1;
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        uint32_t mk = __ballot_sync(0xffffffffu, a == k);
+        while (mk) {  // four rows of the cluster at a time, in token order (the same in every lane)
+          float4 x[4][CG];
+          float sc[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int v = mk ? __ffs(int(mk)) - 1 : -1;
+            mk &= mk - 1;
+            sc[e] = units && v >= 0 ? rinv[r0 + v] : 0.0f;
+#pragma unroll
+            for (int q = 0; q < CG; ++q) {
+              const int c = 4 * (threadIdx.x + kStreamThreads * q);
+              x[e][q] = v >= 0 && c < D ? *reinterpret_cast<const float4*>(base + size_t(v) * D + c)
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int q = 0; q < CG; ++q) {
+              if (raw) {
+                acc[k][q].x += x[e][q].x;
+                acc[k][q].y += x[e][q].y;
+                acc[k][q].z += x[e][q].z;
+                acc[k][q].w += x[e][q].w;
+              }
+              if (units) {
+                unit[k][q].x += x[e][q].x * sc[e];
+                unit[k][q].y += x[e][q].y * sc[e];
+                unit[k][q].z += x[e][q].z * sc[e];
+                unit[k][q].w += x[e][q].w * sc[e];
+              }
+            }
+        }
+      }
+      __syncthreads();  // the step's slot may be refilled
+      if (slots <= 2) issue(f, i + 2, back);
+    }
+    copy_async_wait<0>();  // (empty groups past the end)
+  };
+  auto to_part = [&](float4 (&v)[K][CG]) {
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+      for (int q = 0; q < CG; ++q) {
+        const int c = 4 * threadIdx.x + 4 * kStreamThreads * q;
+        if (c < D) *reinterpret_cast<float4*>(part + k * D + c) = v[k][q];
+      }
+  };
+  start(fin, false);
+  for (int e = 4 * threadIdx.x; e < K * D; e += 4 * blockDim.x) {
+    const int k = e / D, c = e - k * D;
+    *reinterpret_cast<float4*>(cent + e) = *reinterpret_cast<const float4*>(feat_row(p, p.fin, t, ul[(k * m) / K]) + c);
+  }
+  bool done = false;  // the last sweep's unit sums are the final layer's cluster sums
+  for (int it = 0; it < p.iters; ++it) {
+    const bool units = COS && (it > 0 || it + 1 == p.iters);
+    if (threadIdx.x == 0) changed = 0;
+    if (threadIdx.x < SPD_MAX_CLUSTERS) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    sweep(fin, it & 1, true, it == 0, true, units);
+    for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) atomicAdd(&cnt[asg[jj]], 1);
+    to_part(acc);
+    cl.sync();
+    if (warp == 0) {
+      const int f = lane < KC ? *cl.map_shared_rank(&changed, lane) : 0;
+      const int any = __any_sync(0xffffffffu, f != 0);
+      for (int k = 0; k < K; ++k) {
+        int n = lane < KC ? cl.map_shared_rank(cnt, lane)[k] : 0;
+#pragma unroll
+        for (int off = 16; off; off >>= 1) n += __shfl_xor_sync(0xffffffffu, n, off);
+        if (lane == 0) ncl[k] = n;
+      }
+      if (lane == 0) any_changed = any;
+    }
+    __syncthreads();
+    done = (it > 0 && !any_changed) || it + 1 == p.iters;  // the same in every CTA of the cluster
+    if (done) break;
+    start(fin, (it + 1) & 1);
+    cluster_column_reduce<KC>(cl, part, K, D, rank, [&](int k, int c, float4 v) {
+      const float n = float(ncl[k]);
+      if (n > 0.0f) v = make_float4(v.x / n, v.y / n, v.z / n, v.w / n);
+      else v = *reinterpret_cast<const float4*>(cent + k * D + c);
+      for (int rr = 0; rr < KC; ++rr) *reinterpret_cast<float4*>(cl.map_shared_rank(cent, rr) + k * D + c) = v;
+    });
+    cl.sync();
+  }
+  // the layers, the final one first (its sums are there): the next one's rows are on their way meanwhile
+  const int last = p.L == 1 ? p.fin : (p.fin == p.L - 1 ? p.L - 2 : p.L - 1);
+  auto layer = [&](int li) { return li == 0 ? p.fin : (li <= p.fin ? li - 1 : li); };
+  if (p.L > 1) start(p.feat[layer(1)], false);
+  for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) w.assign[size_t(t) * m + j0 + jj] = asg[jj];
+  if (threadIdx.x < 32 * K) {  // a warp a cluster: its a_j, lanes' shares in token order, then a butterfly
+    float a = 0.0f;
+    for (int jj = lane; jj < nl; jj += 32)
+      if (asg[jj] == warp) a += ordered_val(w.asim[size_t(t) * p.n + idx[jj]]);
+    a = warp_sum(a);
+    if (lane == 0) asum_part[warp] = a;
+  }
+  for (int li = 0; li < p.L; ++li) {
+    const int l = layer(li);
+    const float* rstat = (COS ? w.inv : w.st1) + (size_t(l) * p.n_tiles + t) * p.n;
+    if (li > 0 || !COS) {
+      __syncthreads();
+      for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) rinv[jj] = rstat[idx[jj]];
+      __syncthreads();
+    }
+    if (!COS && threadIdx.x == 0) {  // token order, fp64 (KL: the fp64 log-sum-exps)
+      const float* lo = p.sim == SPD_SIM_KL ? w.st3 + (size_t(l) * p.n_tiles + t) * p.n : nullptr;
+      for (int k = 0; k < K; ++k) ssum_part[k] = 0.0;
+      for (int jj = 0; jj < nl; ++jj)
+        ssum_part[asg[jj]] += double(rinv[jj]) + (lo ? double(lo[idx[jj]]) : 0.0);
+    }
+    if (li > 0) {
+      sweep(p.feat[l], false, false, false, !COS, COS);
+      if (li + 1 < p.L) start(p.feat[layer(li + 1)], false);
+    }
+    // (no peer reads the sums of the last iteration, which the loop left before its reduction)
+    if (COS) to_part(unit);
+    else to_part(acc);
+    cl.sync();
+    float* csum = w.csum + (size_t(t) * p.L + l) * K * D;
+    cluster_column_reduce<KC>(cl, part, K, D, rank, [&](int k, int c, float4 sum) {
+      *reinterpret_cast<float4*>(csum + k * D + c) = sum;
+    });
+    if (!COS && rank == 0 && warp == 1) {  // CTA sums added in rank order
+      for (int k = 0; k < K; ++k) {
+        const double sr = lane < KC ? cl.map_shared_rank(ssum_part, lane)[k] : 0.0;
+        double a = 0.0;
+        for (int rr = 0; rr < KC; ++rr) a += __shfl_sync(0xffffffffu, sr, rr);
+        if (lane == 0) w.ssum[(size_t(t) * p.L + l) * 16 + k] = a;
+      }
+    }
+    if (l == last && rank == 0 && warp == 0) {
+      for (int k = 0; k < K; ++k) {
+        const float ar = lane < KC ? cl.map_shared_rank(asum_part, lane)[k] : 0.0f;
+        float a = 0.0f;
+        for (int rr = 0; rr < KC; ++rr) a += __shfl_sync(0xffffffffu, ar, rr);
+        if (lane == 0) {
+          w.counts[t * 16 + k] = ncl[k];
+          w.asum[t * 16 + k] = a;
+        }
+      }
+      warp_quotas(ncl, K, p.n_cmp, w.quotas + t * 16);
+    }
+    cl.sync();  // the peers' shared memory is read above
   }
 }
 
@@ -1566,6 +1881,7 @@ PruneWs carve(const PruneDims& p, Carve& cv) {
 
 constexpr size_t kResSmem = 200 * 1024;  // dynamic shared memory of the resident K-means
 int g_res_clusters = -1;                 // 16-CTA clusters of it the GPU holds at once
+int g_stream_clusters[9] = {};           // KC-CTA clusters of the one-sweep form, by KC
 
 template <int KC, bool RES, int KN, bool FUSED = false>
 cudaError_t launch_kmeans(const PruneDims& p, const PruneWs& w, const PruneOut& out, size_t smem,
@@ -1589,6 +1905,21 @@ cudaError_t launch_kmeans(const PruneDims& p, const PruneWs& w, const PruneOut& 
   return cudaLaunchKernelEx(&cfg, kern, p, w, out);
 }
 
+const void* stream_kernel(int KC, int CG, bool cos) {
+#define SPD_STREAM(kc)                                                                                  \
+  if (KC == kc)                                                                                         \
+    return CG == 1 ? (cos ? (const void*)kmeans_stream_kernel<kc, 1, true>                              \
+                          : (const void*)kmeans_stream_kernel<kc, 1, false>)                            \
+                   : (cos ? (const void*)kmeans_stream_kernel<kc, 2, true>                              \
+                          : (const void*)kmeans_stream_kernel<kc, 2, false>);
+  SPD_STREAM(1)
+  SPD_STREAM(2)
+  SPD_STREAM(4)
+  SPD_STREAM(8)
+#undef SPD_STREAM
+  return nullptr;
+}
+
 // Kernel attributes (once per process) and whether 16-CTA clusters of the resident kernel fit.
 int kmeans_setup() {
   static std::once_flag once;
@@ -1604,8 +1935,6 @@ int kmeans_setup() {
       return e;
     };
     err = streamed(kmeans_kernel<8, false, 4, true>);
-    if (err == cudaSuccess) err = streamed(kmeans_kernel<4, false, 4, true>);
-    if (err == cudaSuccess) err = streamed(kmeans_kernel<4, false, 4, false>);
     if (err == cudaSuccess) err = streamed(kmeans_kernel<8, false, SPD_MAX_CLUSTERS, true>);
     if (err == cudaSuccess) err = resident(kmeans_kernel<16, true, 4, true>);
     if (err == cudaSuccess) err = resident(kmeans_kernel<16, true, SPD_MAX_CLUSTERS, true>);
@@ -1622,6 +1951,9 @@ int kmeans_setup() {
     if (err == cudaSuccess) err = wide(kmeans_grid_kernel<4, false>);
     if (err == cudaSuccess) err = wide(kmeans_grid_kernel<SPD_MAX_CLUSTERS, true>);
     if (err == cudaSuccess) err = wide(kmeans_grid_kernel<SPD_MAX_CLUSTERS, false>);
+    for (int i = 0; i < 16 && err == cudaSuccess; ++i)
+      err = cudaFuncSetAttribute(stream_kernel(1 << (i & 3), i & 4 ? 2 : 1, i & 8),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, int(kStreamSmem));
     g_res_clusters = 0;
     if (err == cudaSuccess) {
       cudaLaunchConfig_t cfg = {};
@@ -1635,6 +1967,22 @@ int kmeans_setup() {
       attr[0].val.clusterDim.z = 1;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
+      for (int kc = 2; kc <= 8 && err == cudaSuccess; kc *= 2) {
+        cudaLaunchConfig_t sc = cfg;
+        cudaLaunchAttribute sa[1];
+        sc.gridDim = dim3(kc);
+        sc.blockDim = dim3(kStreamThreads);
+        sc.dynamicSmemBytes = kStreamSmem;
+        sa[0].id = cudaLaunchAttributeClusterDimension;
+        sa[0].val.clusterDim.x = kc;
+        sa[0].val.clusterDim.y = 1;
+        sa[0].val.clusterDim.z = 1;
+        sc.attrs = sa;
+        if (cudaOccupancyMaxActiveClusters(&g_stream_clusters[kc], stream_kernel(kc, 1, true), &sc) != cudaSuccess) {
+          cudaGetLastError();
+          g_stream_clusters[kc] = 0;
+        }
+      }
       int n = 0;
       if (cudaOccupancyMaxActiveClusters(&n, kmeans_kernel<16, true, SPD_MAX_CLUSTERS, true>, &cfg) !=
           cudaSuccess) {
@@ -1654,6 +2002,8 @@ struct PrunePlan {
   int grid;        // CTAs a tile of the whole-GPU K-means, 0: clusters
   bool grid_res;   // its rows fit in shared memory
   size_t grid_smem;
+  int stream;      // CTAs a tile of the one-sweep K-means, 0: none
+  int stream_slots;
   int launches;
 };
 PrunePlan prune_plan(const PruneDims& p) {
@@ -1686,8 +2036,37 @@ PrunePlan prune_plan(const PruneDims& p) {
       if (q.grid_res) q.grid_smem += nl * p.d * sizeof(float);
     }
   }
+  // Many tiles: one sweep an iteration, over as many CTAs a tile as the SMs hold at one each
+  q.stream = 0;
+  if (!q.res && !q.grid && p.K == 4 && p.d <= 8 * kStreamThreads && p.m > 0) {
+    int KC = 8;
+    while (KC > 1 && p.n_tiles > g_stream_clusters[KC]) KC /= 2;
+    q.stream_slots = std::min(3, stream_slots(p.d, (p.m + KC - 1) / KC, kStreamSmem));
+    if (q.stream_slots >= 2) q.stream = KC;
+  }
   q.launches = 2 + int(q.anchor_sim) + 1 + (q.fused ? 0 : int(p.m > 0) + 1);
   return q;
+}
+
+cudaError_t launch_stream(const PruneDims& p, const PruneWs& w, const PrunePlan& q, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(q.stream, p.n_tiles);
+  cfg.blockDim = dim3(kStreamThreads);
+  cfg.dynamicSmemBytes = kStreamSmem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = q.stream;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  using Fn = void (*)(PruneDims, PruneWs, int);
+  auto kern = reinterpret_cast<Fn>(const_cast<void*>(stream_kernel(q.stream, stream_groups(p.d),
+                                                                   p.sim == SPD_SIM_COS)));
+  return cudaLaunchKernelEx(&cfg, kern, p, w, q.stream_slots);
 }
 
 }  // namespace
@@ -1773,8 +2152,8 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
     SPD_CUDA_TRY((launch_kmeans<16, true, 4>(p, w, out, res_bytes, st)));
   else if (plan.res)
     SPD_CUDA_TRY((launch_kmeans<16, true, SPD_MAX_CLUSTERS>(p, w, out, res_bytes, st)));
-  else if (p.K == 4 && size_t(p.n_tiles) * 8 > 2 * size_t(num_sms()))
-    SPD_CUDA_TRY((launch_kmeans<4, false, 4>(p, w, out, cent_bytes, st)));
+  else if (plan.stream)
+    SPD_CUDA_TRY(launch_stream(p, w, plan, st));
   else if (p.K == 4)
     SPD_CUDA_TRY((launch_kmeans<8, false, 4>(p, w, out, cent_bytes, st)));
   else

@@ -104,12 +104,27 @@ def test_whole_gpu_kmeans(tiles, n, d, keep, kw):
     assert_prune_parity(gpu_prune(v, keep, 1, has_cls=False, attn_form=1, **kw), res)
 
 
+@pytest.mark.parametrize("tiles,n,d,keep,kw", [
+    (11, 333, 1024, 50, {}),                        # eight CTAs a tile, each fewer rows than the ring holds
+    (20, 576, 1028, 64, dict(kmeans_iters=1)),      # four CTAs; columns past 1024; one assignment step
+    (80, 100, 2048, 20, {}),                        # one CTA a tile
+    (12, 300, 256, 40, dict(sim="mse")),
+    (12, 300, 256, 40, dict(sim="kl")),
+    (12, 576, 1024, 64, dict(n_clusters=2)),        # K other than 4: rows re-read from L2 in clusters of eight
+])
+def test_many_tiles_kmeans(tiles, n, d, keep, kw):
+    test_whole_gpu_kmeans(tiles, n, d, keep, kw)
+
+
 def test_whole_gpu_kmeans_iterations():
     v, res = _shuffled_tile(20264001, 900, 1280, 180)
     a = gpu_prune(v, 180, 1, has_cls=False, attn_form=1)
     assert_prune_parity(a, res)
     b = gpu_prune(v, 180, 1, has_cls=False, attn_form=1)  # sums in a fixed order: the same bits again
     np.testing.assert_array_equal(a["scores"].view(np.uint32), b["scores"].view(np.uint32))
+    # the same tile among 24 (one sweep an iteration, every second one backwards)
+    many = dict(feats=[np.repeat(f, 24, 0) for f in v["feats"]], attn=np.repeat(v["attn"], 24, 0))
+    assert_prune_parity(gpu_prune(many, 180, 1, has_cls=False, attn_form=1), res * 24)
 
 
 @pytest.mark.parametrize("n", [1024, 1025, 4096])
