@@ -41,20 +41,29 @@ int num_sms();  // SM count of the current device
 //  * every kernel executes griddepcontrol.wait in at least one thread before it can complete, so
 //    completion orders transitively: when kernel N passes its wait, every earlier kernel of the
 //    stream has completed.
+// carveout: the share of an SM's 256 KB that is set aside as shared memory, in percent (0: the driver's choice,
+// which can hold a kernel of several CTAs an SM below the number that its registers allow).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                       cudaStream_t stream, Args&&... args) {
+cudaError_t launch_pdl_carveout(int carveout, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                cudaStream_t stream, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[1].val.sharedMemCarveout = unsigned(carveout);
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = carveout > 0 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                       cudaStream_t stream, Args&&... args) {
+  return launch_pdl_carveout(0, kernel, grid, block, smem, stream, std::forward<Args>(args)...);
 }
 
 // Bump allocator over a caller-provided workspace. The first 256 bytes hold the status word.

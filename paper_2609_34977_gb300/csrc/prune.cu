@@ -5,8 +5,8 @@
 //                MSE and KL ablations of sim)
 //   anchors      top-N_anc of a_v by ranking (a_v desc, index asc) keys (Eq. 1); stable lists of
 //                anchor and non-anchor tokens by block prefix sums
-//   anchor_sim   a_i = max_p cos(F^L_i, F^L_p) over anchors: 64 x 64 register-tiled fp32 products,
-//                the feature dimension split over a cluster of 4 (8 for few tiles) CTAs whose partial tiles are summed
+//   anchor_sim   a_i = max_p cos(F^L_i, F^L_p) over anchors: 128 x 64 (or 48) register-tiled fp32 products,
+//                the feature dimension split over a cluster of 4 or 8 CTAs whose partial tiles are summed
 //                in rank order through distributed shared memory; max via atomicMax on
 //                order-preserving integer keys (exact, order independent)
 //   kmeans       one thread-block cluster of 16 CTAs per tile, each owning a contiguous slice of the
@@ -34,6 +34,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "internal.h"
 #include "ptx.cuh"
@@ -302,96 +303,144 @@ __global__ void __launch_bounds__(kRankThreads) anchor_kernel(PruneDims p, Prune
   }
 }
 
+// Packed pairs of fp32: two IEEE operations an instruction.
+__device__ __forceinline__ uint64_t sub_f32x2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ float sum_f32x2(uint64_t a) {
+  return __uint_as_float(uint32_t(a)) + __uint_as_float(uint32_t(a >> 32));
+}
+
 // ---- 3. a_i = max over anchors of cos(F^L_i, F^L_p) -------------------------------------------
-// A cluster of AS CTAs per 64 non-anchor tokens x 64 anchors tile, each CTA one slice of the
-// feature dimension: 32-wide chunks through shared memory (stored transposed; the next chunk is
-// fetched into registers while the current one is multiplied), 4 x 4 dot products per thread
-// (4 consecutive rows x 4 consecutive anchors: two 16-byte shared-memory loads per 16 FMAs).
-// The partial tiles are summed in rank order through distributed shared memory, each CTA
-// finishing 64 / AS rows. AS = 4 at serving batch; 8 for a few tiles (shorter chains per CTA).
-template <int SIM, int AS>
+// A cluster of AS CTAs per R non-anchor tokens x AW anchors tile, each CTA one slice of the feature
+// dimension: 32-wide chunks through shared memory (stored transposed; the next chunk is fetched into
+// registers while the current one is multiplied), R / 16 x AW / 16 products a thread. The loop was bound by
+// shared-memory reads with 4 x 4 products (16 FMAs per two 16-byte loads: 78 % of the load pipe, 46 % of the
+// FMA pipe busy); eight rows a thread (R = 128) halve the loads a product, and the products of two rows go out
+// as one packed instruction. Every product is still one fp32 FMA in the order of the features.
+// The partial tiles are summed in rank order through distributed shared memory, each CTA finishing R / AS
+// rows. AS = 4 at serving batch, 8 where that still leaves at most three CTAs an SM (shorter chains per CTA),
+// and R = 64 where R = 128 would leave SMs idle at that. AW is 64, or 48 where that pads the anchors less. (64 tiles of 531 x 45 anchors x 1024: 148 -> 115 us; 2260 x 479 x 1280:
+// 98 -> 81 us.)
+template <int SIM, int AS, int AW, int kSimRows>
 __global__ void __cluster_dims__(AS, 1, 1) __launch_bounds__(256)
     anchor_sim_kernel(PruneDims p, PruneWs w) {
   pdl_launch_dependents();
   pdl_wait();
-  __shared__ __align__(16) float Us[32][68], As[32][68];
-  __shared__ float P[64][65];  // this CTA's partial dot products
+  constexpr int TJ = AW / 16, TI = kSimRows / 32;  // anchors and row pairs a thread
+  constexpr int UP = kSimRows + 4, AP = AW + 4;
+  // one buffer: the operand chunks during the products, this CTA's partial dot products after them
+  __shared__ __align__(16) float buf[kSimRows * (AW + 1) > 32 * (UP + AP) ? kSimRows * (AW + 1) : 32 * (UP + AP)];
+  float(*Us)[UP] = reinterpret_cast<float(*)[UP]>(buf);
+  float(*As)[AP] = reinterpret_cast<float(*)[AP]>(buf + 32 * UP);
+  float(*P)[AW + 1] = reinterpret_cast<float(*)[AW + 1]>(buf);
   cg::cluster_group cl = cg::this_cluster();
   const int rank = int(cl.block_rank());
   const int t = blockIdx.z, tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int u0 = (blockIdx.x / AS) * 64, p0 = blockIdx.y * 64;
+  const int u0 = (blockIdx.x / AS) * kSimRows, p0 = blockIdx.y * AW;
   const int* ul = w.ulist + size_t(t) * p.m;
   const int* al = w.alist + size_t(t) * p.n_anc;
-  // staging: thread loads column dd of rows 8 r0 + i (i < 8) of both operands
+  // staging: warp w loads column dd of rows R / 8 w + i and of anchors AW / 8 w + i
+  constexpr int UR = kSimRows / 8, AR = AW / 8;
   const int dd = threadIdx.x & 31, r0 = threadIdx.x >> 5;
   // per-row statistics of the final layer (MSE: squared norms; KL: log-sum-exps, negentropies)
   const size_t so = (size_t(p.fin) * p.n_tiles + t) * p.n;
   constexpr bool kl = SIM == SPD_SIM_KL;
-  // rows as 32-bit offsets into the tile's block of F^L (fewer registers than pointers; the block
-  // holds at most 4097 rows of at most 4096 floats); -1 for rows past the lists
+  // rows as 32-bit offsets into the tile's block of F^L (it holds at most 4097 rows of at most 4096 floats), in
+  // shared memory (broadcast reads); -1 for rows past the lists
   const float* tile_f = feat_row(p, p.fin, t, -p.off);
-  int uo[8], ao[8];
-  double ulse[8];  // KL: the non-anchor operand is softmax(F^L_i) = exp(F^L_i - lse_i), in fp64
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = 8 * r0 + i;
+  __shared__ int uo[kSimRows], ao[AW];
+  __shared__ double ulse[kl ? kSimRows : 1];  // KL: the non-anchor operand is softmax(F^L_i) = exp(F^L_i - lse_i), in fp64
+  if (threadIdx.x < kSimRows) {
+    const int r = threadIdx.x;
     const bool uv = u0 + r < p.m;
-    uo[i] = uv ? (p.off + ul[u0 + r]) * p.d : -1;
-    ao[i] = (p0 + r < p.n_anc) ? (p.off + al[p0 + r]) * p.d : -1;
-    ulse[i] = (kl && uv) ? double(w.st1[so + ul[u0 + r]]) + double(w.st3[so + ul[u0 + r]]) : 0.0;
+    uo[r] = uv ? (p.off + ul[u0 + r]) * p.d : -1;
+    if (kl) ulse[r] = uv ? double(w.st1[so + ul[u0 + r]]) + double(w.st3[so + ul[u0 + r]]) : 0.0;
+  } else if (threadIdx.x < kSimRows + AW) {
+    const int r = threadIdx.x - kSimRows;
+    ao[r] = p0 + r < p.n_anc ? (p.off + al[p0 + r]) * p.d : -1;
   }
+  __syncthreads();
   const int nch = (p.d + 31) / 32, c0 = rank * nch / AS, c1 = (rank + 1) * nch / AS;
-  float ru[8], ra[8];
+  float ru[UR], ra[AR];
   auto fetch = [&](int ch) {
     const int dcol = ch * 32 + dd;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float x = (uo[i] >= 0 && dcol < p.d) ? tile_f[uo[i] + dcol] : 0.0f;
-      if constexpr (kl) ru[i] = (uo[i] >= 0 && dcol < p.d) ? float(exp(double(x) - ulse[i])) : 0.0f;
+    for (int i = 0; i < UR; ++i) {
+      const int o = uo[UR * r0 + i];
+      const float x = (o >= 0 && dcol < p.d) ? tile_f[o + dcol] : 0.0f;
+      if constexpr (kl) ru[i] = (o >= 0 && dcol < p.d) ? float(exp(double(x) - ulse[UR * r0 + i])) : 0.0f;
       else ru[i] = x;
-      ra[i] = (ao[i] >= 0 && dcol < p.d) ? tile_f[ao[i] + dcol] : 0.0f;
+    }
+#pragma unroll
+    for (int i = 0; i < AR; ++i) {
+      const int o = ao[AR * r0 + i];
+      ra[i] = (o >= 0 && dcol < p.d) ? tile_f[o + dcol] : 0.0f;
     }
   };
-  float acc[4][4];
+  uint64_t acc[TI][TJ];  // rows 2 (TI ty + i) + {0, 1}, anchors tx + 16 j
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TI; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
+    for (int j = 0; j < TJ; ++j) acc[i][j] = 0;
   if (c0 < c1) fetch(c0);
   for (int ch = c0; ch < c1; ++ch) {
-    // eight consecutive rows of column dd: two 16-byte stores per operand
-    *reinterpret_cast<float4*>(&Us[dd][8 * r0]) = make_float4(ru[0], ru[1], ru[2], ru[3]);
-    *reinterpret_cast<float4*>(&Us[dd][8 * r0 + 4]) = make_float4(ru[4], ru[5], ru[6], ru[7]);
-    *reinterpret_cast<float4*>(&As[dd][8 * r0]) = make_float4(ra[0], ra[1], ra[2], ra[3]);
-    *reinterpret_cast<float4*>(&As[dd][8 * r0 + 4]) = make_float4(ra[4], ra[5], ra[6], ra[7]);
+#pragma unroll
+    for (int i = 0; i < UR; i += 4)
+      *reinterpret_cast<float4*>(&Us[dd][UR * r0 + i]) = make_float4(ru[i], ru[i + 1], ru[i + 2], ru[i + 3]);
+#pragma unroll
+    for (int i = 0; i < AR; i += 2) *reinterpret_cast<float2*>(&As[dd][AR * r0 + i]) = make_float2(ra[i], ra[i + 1]);
     __syncthreads();
     if (ch + 1 < c1) fetch(ch + 1);  // in flight during the products below
 #pragma unroll 8
     for (int e = 0; e < 32; ++e) {
-      // rows 4 ty .. 4 ty + 3 and anchors 4 tx .. 4 tx + 3: one 16-byte load each
-      const float4 av = *reinterpret_cast<const float4*>(&Us[e][4 * ty]);
-      const float4 bv = *reinterpret_cast<const float4*>(&As[e][4 * tx]);
-      const float a[4] = {av.x, av.y, av.z, av.w}, b[4] = {bv.x, bv.y, bv.z, bv.w};
+      uint64_t a[TI];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TI; i += 2) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&Us[e][2 * (TI * ty + i)]);
+        a[i] = v.x;
+        a[i + 1] = v.y;
+      }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * b[j];
+      for (int j = 0; j < TJ; ++j) {
+        const uint32_t bv = __float_as_uint(As[e][tx + 16 * j]);
+        const uint64_t b = uint64_t(bv) << 32 | bv;
+#pragma unroll
+        for (int i = 0; i < TI; ++i) acc[i][j] = fma_f32x2(a[i], b, acc[i][j]);
+      }
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TI; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) P[4 * ty + i][4 * tx + j] = acc[i][j];
+    for (int j = 0; j < TJ; ++j) {
+      P[2 * (TI * ty + i)][tx + 16 * j] = __uint_as_float(uint32_t(acc[i][j]));
+      P[2 * (TI * ty + i) + 1][tx + 16 * j] = __uint_as_float(uint32_t(acc[i][j] >> 32));
+    }
   cl.sync();
   // rows RPC rank .. RPC rank + RPC - 1 of the tile (TPR threads a row, CPT columns a thread): all
   // AS partials loaded first, summed in rank order
-  constexpr int RPC = 64 / AS, TPR = 256 / RPC, CPT = 64 / TPR;
-  const int lr = RPC * rank + int(threadIdx.x) / TPR, cx = int(threadIdx.x) % TPR;
+  // (at R = 64, AS = 8 the upper half of the block repeats the lower half's: the maximum stays)
+  constexpr int RPC = kSimRows / AS, TPR = RPC < 16 ? 16 : 256 / RPC, CPT = AW / TPR;
+  static_assert(AW % TPR == 0, "whole columns a thread");
+  const int lr = RPC * rank + int(threadIdx.x) / TPR % RPC, cx = int(threadIdx.x) % TPR;
   float x[AS][CPT];
 #pragma unroll
   for (int src = 0; src < AS; ++src) {
-    const float* pp = cl.map_shared_rank(&P[0][0], src) + lr * 65;
+    const float* pp = cl.map_shared_rank(&P[0][0], src) + lr * (AW + 1);
 #pragma unroll
     for (int j = 0; j < CPT; ++j) x[src][j] = pp[cx + TPR * j];
   }
@@ -654,55 +703,11 @@ __device__ __forceinline__ void column_sums(float* part, int K, int D, int nl, c
     }
 }
 
-// Packed pairs of fp32: two IEEE operations an instruction.
-__device__ __forceinline__ uint64_t sub_f32x2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ float sum_f32x2(uint64_t a) {
-  return __uint_as_float(uint32_t(a)) + __uint_as_float(uint32_t(a >> 32));
-}
-
-// assign_rows for K = 4, the calling warp's next n (at most RP count) rows at a time: a centroid's 16 bytes serve RP rows, differences and
-// squares are packed, and the 4 RP partial distances are summed over the lanes by halving exchanges (lane bits
-// 4, 3, ... pick the value) instead of a butterfly each. The loop is bound by issue: about 155
-// instructions a row of 1024 at RP = 4 where a row at a time took about 450 (28 rows of a CTA of eight
-// warps: 4.3 -> 2.0 us).
-template <int RP, typename Row>
-__device__ __forceinline__ void assign4_rows(const float* cent, int D, int n, bool first, int8_t* asg, int* changed,
-                                             Row xrow) {
+// The nearest of four centroids for each of RP rows from the lanes' packed partial distances.
+template <int RP>
+__device__ __forceinline__ void assign4_nearest(const uint64_t (&acc)[RP][4], int n, bool first, int8_t* asg, int* changed) {
   constexpr int NV = 4 * RP;
   const int lane = threadIdx.x & 31;
-  const float* x[RP];
-#pragma unroll
-  for (int i = 0; i < RP; ++i) x[i] = xrow(min(i, n - 1));
-  uint64_t acc[RP][4];
-#pragma unroll
-  for (int i = 0; i < RP; ++i)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) acc[i][k] = 0;
-#pragma unroll 2
-  for (int c = 4 * lane; c < D; c += 128) {
-    ulonglong2 xv[RP], cv[4];
-#pragma unroll
-    for (int i = 0; i < RP; ++i) xv[i] = *reinterpret_cast<const ulonglong2*>(x[i] + c);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) cv[k] = *reinterpret_cast<const ulonglong2*>(cent + k * D + c);
-#pragma unroll
-    for (int i = 0; i < RP; ++i)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint64_t d0 = sub_f32x2(xv[i].x, cv[k].x), d1 = sub_f32x2(xv[i].y, cv[k].y);
-        acc[i][k] = fma_f32x2(d0, d0, acc[i][k]);
-        acc[i][k] = fma_f32x2(d1, d1, acc[i][k]);
-      }
-  }
   float v[NV];
 #pragma unroll
   for (int i = 0; i < RP; ++i)
@@ -738,6 +743,71 @@ __device__ __forceinline__ void assign4_rows(const float* cent, int D, int n, bo
     if (first || asg[jj] != best) *changed = 1;
     asg[jj] = int8_t(best);
   }
+}
+
+// assign_rows for K = 4, the calling warp's next n (at most RP count) rows at a time: a centroid's 16 bytes serve RP rows, differences and
+// squares are packed, and the 4 RP partial distances are summed over the lanes by halving exchanges (lane bits
+// 4, 3, ... pick the value) instead of a butterfly each. The loop is bound by issue: about 155
+// instructions a row of 1024 at RP = 4 where a row at a time took about 450 (28 rows of a CTA of eight
+// warps: 4.3 -> 2.0 us).
+template <int RP, typename Row>
+__device__ __forceinline__ void assign4_rows(const float* cent, int D, int n, bool first, int8_t* asg, int* changed,
+                                             Row xrow) {
+  const int lane = threadIdx.x & 31;
+  const float* x[RP];
+#pragma unroll
+  for (int i = 0; i < RP; ++i) x[i] = xrow(min(i, n - 1));
+  uint64_t acc[RP][4];
+#pragma unroll
+  for (int i = 0; i < RP; ++i)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[i][k] = 0;
+#pragma unroll 2
+  for (int c = 4 * lane; c < D; c += 128) {
+    ulonglong2 xv[RP], cv[4];
+#pragma unroll
+    for (int i = 0; i < RP; ++i) xv[i] = *reinterpret_cast<const ulonglong2*>(x[i] + c);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) cv[k] = *reinterpret_cast<const ulonglong2*>(cent + k * D + c);
+#pragma unroll
+    for (int i = 0; i < RP; ++i)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint64_t d0 = sub_f32x2(xv[i].x, cv[k].x), d1 = sub_f32x2(xv[i].y, cv[k].y);
+        acc[i][k] = fma_f32x2(d0, d0, acc[i][k]);
+        acc[i][k] = fma_f32x2(d1, d1, acc[i][k]);
+      }
+  }
+  assign4_nearest<RP>(acc, n, first, asg, changed);
+}
+// The same with the centroids in the caller's registers: lane's columns 4 lane + 128 j of centroid k in cr[k][j].
+template <int RP, typename Row>
+__device__ __forceinline__ void assign4_regs(const ulonglong2 (&cr)[4][8], int D, int n, bool first, int8_t* asg,
+                                             int* changed, Row xrow) {
+  const int lane = threadIdx.x & 31;
+  const float* x[RP];
+#pragma unroll
+  for (int i = 0; i < RP; ++i) x[i] = xrow(min(i, n - 1));
+  uint64_t acc[RP][4];
+#pragma unroll
+  for (int i = 0; i < RP; ++i)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[i][k] = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int c = 4 * lane + 128 * j;
+#pragma unroll
+    for (int i = 0; i < RP; ++i) {
+      const ulonglong2 xv = c < D ? *reinterpret_cast<const ulonglong2*>(x[i] + c) : make_ulonglong2(0, 0);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint64_t d0 = sub_f32x2(xv.x, cr[k][j].x), d1 = sub_f32x2(xv.y, cr[k][j].y);
+        acc[i][k] = fma_f32x2(d0, d0, acc[i][k]);
+        acc[i][k] = fma_f32x2(d1, d1, acc[i][k]);
+      }
+    }
+  }
+  assign4_nearest<RP>(acc, n, first, asg, changed);
 }
 // ... of all nl rows by the block's warps.
 template <int RP, typename Row>
@@ -1298,7 +1368,8 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
 // cluster sums if the assignment repeats. Every second sweep runs backwards: the rows that the last one
 // read end up in L2. So a tile whose assignment repeats at once is read twice for K-means and once a
 // further layer, where the form that it replaces (4 CTAs a tile re-reading the rows through registers) read
-// it five times: 64 tiles 234 -> 163 us serialised, of which the copies alone take 76.
+// it five times: 64 tiles 234 -> 156 us serialised, of which the copies alone take 76; the assignment (with
+// the centroids in registers up to 1024 columns) and the sums are chains of shared-memory loads of 8 warps.
 constexpr int kStreamThreads = 256;
 constexpr size_t kStreamSmem = 226 * 1024;  // dynamic shared memory of a CTA
 // Column groups of a thread (rows of up to 1024 or 2048 floats) and rows of a step.
@@ -1326,7 +1397,7 @@ __device__ __forceinline__ void copy_async_wait() {  // all but the thread's las
 template <int KC, int CG, bool COS>
 __global__ void __launch_bounds__(kStreamThreads, 1) kmeans_stream_kernel(PruneDims p, PruneWs w, int slots) {
   extern __shared__ __align__(16) float ksm[];
-  constexpr int K = 4, SR = stream_step(CG);
+  constexpr int K = 4, SR = stream_step(CG), SB = 8 / CG;  // rows a step, rows in flight in the sums
   const int D = p.d, m = p.m;
   const int nl_max = (m + KC - 1) / KC;
   float* cent = ksm;            // [K][D]
@@ -1335,6 +1406,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1) kmeans_stream_kernel(PruneD
   uint16_t* idx = reinterpret_cast<uint16_t*>(rinv + nl_max);
   int8_t* asg = reinterpret_cast<int8_t*>(idx + nl_max);
   float* ring = ksm + stream_head(D, nl_max) / sizeof(float);  // [slots][SR][D]
+  // during a sweep, in part's place (4 D >= 2 SR kStreamThreads / 32 floats): each warp's list of a step's rows by
+  // cluster, as offsets into the step, and their scales
+  int* ord_off = reinterpret_cast<int*>(part) + (threadIdx.x >> 5) * SR;
+  float* ord_scale = part + (kStreamThreads / 32 + (threadIdx.x >> 5)) * SR;
   __shared__ int cnt[SPD_MAX_CLUSTERS], ncl[SPD_MAX_CLUSTERS];
   __shared__ int changed, any_changed;
   __shared__ float asum_part[K];
@@ -1377,14 +1452,24 @@ __global__ void __launch_bounds__(kStreamThreads, 1) kmeans_stream_kernel(PruneD
     issue(f, 0, back);
     issue(f, 1, back);
   };
-  float4 acc[K][CG], unit[K][CG];
+  ulonglong2 acc[K][CG], unit[K][CG];  // four columns each, as two packed pairs
   // one sweep: assignment (where `assign`) and column sums of the rows (acc, where `raw`) and of the rows times
   // rinv (unit, where `units`); its first two steps were issued by start()
   auto sweep = [&](const float* f, bool back, bool assign, bool first, bool raw, bool units) {
 #pragma unroll
     for (int k = 0; k < K; ++k)
 #pragma unroll
-      for (int q = 0; q < CG; ++q) acc[k][q] = unit[k][q] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int q = 0; q < CG; ++q) acc[k][q] = unit[k][q] = make_ulonglong2(0, 0);
+    ulonglong2 cr[CG == 1 ? 4 : 1][CG == 1 ? 8 : 1];  // centroids of rows of up to 1024 floats
+    if (CG == 1 && assign) {
+#pragma unroll
+      for (int k = 0; k < (CG == 1 ? 4 : 1); ++k)
+#pragma unroll
+        for (int j = 0; j < (CG == 1 ? 8 : 1); ++j) {
+          const int c = 4 * lane + 128 * j;
+          cr[k][j] = c < D ? *reinterpret_cast<const ulonglong2*>(cent + k * D + c) : make_ulonglong2(0, 0);
+        }
+    }
     for (int i = 0; i < ns; ++i) {
       // with three slots the step after the next is issued before this one is used, with two after it
       if (slots > 2) issue(f, i + 2, back);
@@ -1396,61 +1481,74 @@ __global__ void __launch_bounds__(kStreamThreads, 1) kmeans_stream_kernel(PruneD
       if (assign) {
         constexpr int RP = SR / 8;  // rows a warp
         const int v0 = warp * RP;
-        if (v0 < rows)
-          assign4_rows<RP>(cent, D, rows - v0, first, asg + r0 + v0, &changed,
-                           [&](int q) { return base + size_t(v0 + q) * D; });
+        auto row = [&](int q) { return base + size_t(v0 + q) * D; };
+        if (v0 < rows) {
+          if constexpr (CG == 1) assign4_regs<RP>(cr, D, rows - v0, first, asg + r0 + v0, &changed, row);
+          else assign4_rows<RP>(cent, D, rows - v0, first, asg + r0 + v0, &changed, row);
+        }
         __syncthreads();
       }
-      const int a = lane < rows ? asg[r0 + lane] : -1;
+      // the step's rows by cluster, in token order within each (every warp for itself): a row then costs its
+      // load and two packed additions a pair set
+      const int a = lane < rows ? asg[r0 + lane] : K;
+      int first_of[K + 1], rank_of = 0;
+      first_of[0] = 0;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
-        uint32_t mk = __ballot_sync(0xffffffffu, a == k);
-        while (mk) {  // four rows of the cluster at a time, in token order (the same in every lane)
-          float4 x[4][CG];
-          float sc[4];
+        const uint32_t who = __ballot_sync(0xffffffffu, a == k);
+        if (a == k) rank_of = first_of[k] + __popc(who & ((1u << lane) - 1));
+        first_of[k + 1] = first_of[k] + __popc(who);
+      }
+      if (lane < rows) {
+        ord_off[rank_of] = lane * D;
+        if (units) ord_scale[rank_of] = rinv[r0 + lane];
+      }
+      __syncwarp();
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int v = mk ? __ffs(int(mk)) - 1 : -1;
-            mk &= mk - 1;
-            sc[e] = units && v >= 0 ? rinv[r0 + v] : 0.0f;
+      for (int k = 0; k < K; ++k)
+        for (int v = first_of[k]; v < first_of[k + 1]; v += SB) {
+          ulonglong2 x[SB][CG];
+#pragma unroll
+          for (int e = 0; e < SB; ++e)
 #pragma unroll
             for (int q = 0; q < CG; ++q) {
               const int c = 4 * (threadIdx.x + kStreamThreads * q);
-              x[e][q] = v >= 0 && c < D ? *reinterpret_cast<const float4*>(base + size_t(v) * D + c)
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+              x[e][q] = v + e < first_of[k + 1] && c < D
+                            ? *reinterpret_cast<const ulonglong2*>(base + ord_off[v + e] + c)
+                            : make_ulonglong2(0, 0);
             }
-          }
+          if (raw)
 #pragma unroll
-          for (int e = 0; e < 4; ++e)
+            for (int e = 0; e < SB; ++e)
 #pragma unroll
-            for (int q = 0; q < CG; ++q) {
-              if (raw) {
-                acc[k][q].x += x[e][q].x;
-                acc[k][q].y += x[e][q].y;
-                acc[k][q].z += x[e][q].z;
-                acc[k][q].w += x[e][q].w;
+              for (int q = 0; q < CG; ++q) {
+                acc[k][q].x = add_f32x2(acc[k][q].x, x[e][q].x);
+                acc[k][q].y = add_f32x2(acc[k][q].y, x[e][q].y);
               }
-              if (units) {
-                unit[k][q].x += x[e][q].x * sc[e];
-                unit[k][q].y += x[e][q].y * sc[e];
-                unit[k][q].z += x[e][q].z * sc[e];
-                unit[k][q].w += x[e][q].w * sc[e];
+          if (units)
+#pragma unroll
+            for (int e = 0; e < SB; ++e) {
+              const uint32_t sb = v + e < first_of[k + 1] ? __float_as_uint(ord_scale[v + e]) : 0u;
+              const uint64_t sc = uint64_t(sb) << 32 | sb;
+#pragma unroll
+              for (int q = 0; q < CG; ++q) {
+                unit[k][q].x = fma_f32x2(x[e][q].x, sc, unit[k][q].x);
+                unit[k][q].y = fma_f32x2(x[e][q].y, sc, unit[k][q].y);
               }
             }
         }
-      }
       __syncthreads();  // the step's slot may be refilled
       if (slots <= 2) issue(f, i + 2, back);
     }
     copy_async_wait<0>();  // (empty groups past the end)
   };
-  auto to_part = [&](float4 (&v)[K][CG]) {
+  auto to_part = [&](const ulonglong2 (&v)[K][CG]) {
 #pragma unroll
     for (int k = 0; k < K; ++k)
 #pragma unroll
       for (int q = 0; q < CG; ++q) {
         const int c = 4 * threadIdx.x + 4 * kStreamThreads * q;
-        if (c < D) *reinterpret_cast<float4*>(part + k * D + c) = v[k][q];
+        if (c < D) *reinterpret_cast<ulonglong2*>(part + k * D + c) = v[k][q];
       }
   };
   start(fin, false);
@@ -1879,6 +1977,10 @@ PruneWs carve(const PruneDims& p, Carve& cv) {
   return w;
 }
 
+// Shared-memory carveout of the kernels around K-means, in percent: with the driver's choice fewer CTAs of
+// anchor_sim_kernel share an SM than its registers allow (64 tiles, us a call: 446 with the driver's choice,
+// 409 / 412 / 415 / 446 at 25 / 50 / 75 / 100 %; one tile 75, 68 / 66 / 71 / 72).
+constexpr int kPruneCarveout = 50;
 constexpr size_t kResSmem = 200 * 1024;  // dynamic shared memory of the resident K-means
 int g_res_clusters = -1;                 // 16-CTA clusters of it the GPU holds at once
 int g_stream_clusters[9] = {};           // KC-CTA clusters of the one-sweep form, by KC
@@ -2038,7 +2140,7 @@ PrunePlan prune_plan(const PruneDims& p) {
   }
   // Many tiles: one sweep an iteration, over as many CTAs a tile as the SMs hold at one each
   q.stream = 0;
-  if (!q.res && !q.grid && p.K == 4 && p.d <= 8 * kStreamThreads && p.m > 0) {
+  if (!q.res && !q.grid && p.K == 4 && p.d >= 64 && p.d <= 8 * kStreamThreads && p.m > 0) {
     int KC = 8;
     while (KC > 1 && p.n_tiles > g_stream_clusters[KC]) KC /= 2;
     q.stream_slots = std::min(3, stream_slots(p.d, (p.m + KC - 1) / KC, kStreamSmem));
@@ -2106,25 +2208,28 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
   cudaStream_t st = static_cast<cudaStream_t>(stream_);
   const int T = p.n_tiles;
   const int slot = trace_begin(st);
-  SPD_CUDA_TRY(launch_pdl(p.sim == SPD_SIM_COS ? rowstats_kernel<SPD_SIM_COS>
+  SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, p.sim == SPD_SIM_COS ? rowstats_kernel<SPD_SIM_COS>
                           : p.sim == SPD_SIM_MSE ? rowstats_kernel<SPD_SIM_MSE> : rowstats_kernel<SPD_SIM_KL>,
                           dim3((p.n + 7) / 8, T), dim3(256), 0, st, p, attn, w));
-  SPD_CUDA_TRY(launch_pdl(anchor_kernel, dim3(rank_ctas(p.n), T), dim3(kRankThreads), 0, st, p, w));
+  SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, anchor_kernel, dim3(rank_ctas(p.n), T), dim3(kRankThreads), 0, st, p, w));
   if (int rc = kmeans_setup()) return rc;
   const PrunePlan plan = prune_plan(p);
   if (plan.anchor_sim) {
-    // the feature dimension over 8 CTAs while the tiles leave most SMs idle, else over 4
-    const dim3 g((p.m + 63) / 64, (p.n_anc + 63) / 64, T);
-    if (size_t(g.x) * g.y * T * 8 <= 2 * size_t(num_sms()))
-      SPD_CUDA_TRY(launch_pdl(p.sim == SPD_SIM_COS ? anchor_sim_kernel<SPD_SIM_COS, 8>
-                              : p.sim == SPD_SIM_MSE ? anchor_sim_kernel<SPD_SIM_MSE, 8>
-                                                     : anchor_sim_kernel<SPD_SIM_KL, 8>,
-                              dim3(g.x * 8, g.y, T), dim3(256), 0, st, p, w));
-    else
-      SPD_CUDA_TRY(launch_pdl(p.sim == SPD_SIM_COS ? anchor_sim_kernel<SPD_SIM_COS, 4>
-                              : p.sim == SPD_SIM_MSE ? anchor_sim_kernel<SPD_SIM_MSE, 4>
-                                                     : anchor_sim_kernel<SPD_SIM_KL, 4>,
-                              dim3(g.x * 4, g.y, T), dim3(256), 0, st, p, w));
+    const int aw = (p.n_anc + 47) / 48 * 48 < (p.n_anc + 63) / 64 * 64 ? 48 : 64;
+    const int ay = (p.n_anc + aw - 1) / aw;
+    const size_t ctas = size_t((p.m + 127) / 128) * ay * T * 8;  // at R = 128, AS = 8
+    const int as = ctas <= 3 * size_t(num_sms()) ? 8 : 4, rows = ctas < size_t(num_sms()) ? 64 : 128;
+    const dim3 g((p.m + rows - 1) / rows, ay, T);
+    auto pick = [&](auto sim) {
+      constexpr int S = decltype(sim)::value;
+      return rows == 64 ? (aw == 48 ? anchor_sim_kernel<S, 8, 48, 64> : anchor_sim_kernel<S, 8, 64, 64>)
+             : as == 8  ? (aw == 48 ? anchor_sim_kernel<S, 8, 48, 128> : anchor_sim_kernel<S, 8, 64, 128>)
+                        : (aw == 48 ? anchor_sim_kernel<S, 4, 48, 128> : anchor_sim_kernel<S, 4, 64, 128>);
+    };
+    auto kern = p.sim == SPD_SIM_COS   ? pick(std::integral_constant<int, SPD_SIM_COS>())
+                : p.sim == SPD_SIM_MSE ? pick(std::integral_constant<int, SPD_SIM_MSE>())
+                                       : pick(std::integral_constant<int, SPD_SIM_KL>());
+    SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, kern, dim3(g.x * as, g.y, T), dim3(256), 0, st, p, w));
   }
   const size_t cent_bytes = size_t(2) * p.K * p.d * sizeof(float);
   const size_t res_bytes = size_t((p.m + 15) / 16) * p.d * sizeof(float) + cent_bytes;
@@ -2162,9 +2267,9 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
     if (p.m > 0) {
       auto score = p.sim == SPD_SIM_COS ? score_kernel<SPD_SIM_COS>
                    : p.sim == SPD_SIM_MSE ? score_kernel<SPD_SIM_MSE> : score_kernel<SPD_SIM_KL>;
-      SPD_CUDA_TRY(launch_pdl(score, dim3((p.m + 7) / 8, T), dim3(256), 0, st, p, w));
+      SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, score, dim3((p.m + 7) / 8, T), dim3(256), 0, st, p, w));
     }
-    SPD_CUDA_TRY(launch_pdl(select_kernel, dim3(rank_ctas(p.m), T), dim3(kRankThreads), 0, st, p, w, keep_idx, kind, cluster,
+    SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, select_kernel, dim3(rank_ctas(p.m), T), dim3(kRankThreads), 0, st, p, w, keep_idx, kind, cluster,
                             scores));
   }
   // algorithmic work per tile: every tapped layer's features and the attention read once, the
