@@ -1273,19 +1273,18 @@ int make_operand_map(CUtensorMap* map, const void* ptr, int inner, int outer, in
 
 namespace {
 
-// ---- matrix-vector path (at most kGemvTok tokens, e.g. a decode step) ----------------------------
+// ---- matrix-vector path (one token, or up to eight: a decode step) --------------------------------
 // With a handful of tokens the contraction is a pure weight stream: no tensor-core tile can be
 // filled, and the tiled kernel's fixed costs (TMEM, barriers, a ring sized for wide tiles) and its
-// shared-memory traffic per weight byte cap it well below the HBM roof. Here each CTA owns 32
+// shared-memory traffic per weight byte cap it well below the HBM roof. At one token each CTA owns 32
 // weight rows (warp w: rows 4w .. 4w + 3) over a range of K; every lane streams 16-byte chunks
 // (eight bf16) so that one warp load covers 512 contiguous bytes of a row, with eight loads in
-// flight per lane, and multiplies them with the tokens' chunks staged in shared memory (fp32
+// flight per lane, and multiplies them with the token's chunks staged in shared memory (fp32
 // accumulation, fixed order). The first batch of weight loads is issued before the grid waits
 // on its predecessor (weights do not depend on it). The 32 row sums are then laid out as the
 // tcgen05 accumulator would hold them (lane = row within the 32-row group, eight token columns)
 // and go through the same fused epilogues. Residual (ADD) epilogues may split K over several CTAs
 // (red.add, as in the tiled kernel); the others own whole rows.
-constexpr int kGemvTok = 4;
 constexpr int kGemvThreads = 256;
 constexpr int kGemvChunk = 256;  // K elements per chunk column (32 lanes x 8 bf16)
 
@@ -1295,6 +1294,19 @@ __device__ __forceinline__ int4 ld_weights(const int4* p) {
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(p));
   return v;
+}
+// Requests the first bytes of weight row n's columns [k0, k0 + kn) into L2 (before the grid dependency wait:
+// weights depend on nothing). The predecessor's tail, the wait and the input's norm leave HBM idle for
+// several us a launch; what a CTA's registers can hold in flight covers about two of them. 2 KB a row
+// (64 KB a CTA) were as good as 4; whole rows of 8 KB took the bandwidth from the predecessor's own stream
+// (one token, 32 layers: 3084 us a step without, 2912 / 2914 / 3135 us with 2 / 4 / 8 KB a row).
+constexpr int kGemvAhead = 2048;  // bytes a row
+__device__ __forceinline__ void prefetch_rows(const uint16_t* w, const KArgs& a, int n, bool mine, int k0, int kn,
+                                              int ahead) {
+  if (mine && n < a.n_out && kn > 0) {
+    const uint32_t bytes = uint32_t(min(ahead, 2 * kn));
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(w + size_t(n) * a.k + k0), "r"(bytes) : "memory");
+  }
 }
 // acc + the dot product of eight bf16 pairs (w, x), element 2i in the low half of word i
 __device__ __forceinline__ float dot8_bf16(const int4& w, const int4& x, float acc) {
@@ -1308,17 +1320,17 @@ __device__ __forceinline__ float dot8_bf16(const int4& w, const int4& x, float a
   return acc;
 }
 
-// NT: tokens computed (>= n_tok); CPR: chunks of a row per batch. A warp's work is a sequence of
+// CPR: chunks of a row per batch. A warp's work is a sequence of
 // batches (row pair, block of CPR chunk columns). One register buffer per warp: latency is hidden
 // by the number of resident warps (measured faster than double-buffering registers, which lowers
 // occupancy).
-template <int EPI, int NT, int CPR>
-__global__ void __launch_bounds__(kGemvThreads)
+template <int EPI, int CPR>
+__global__ void __launch_bounds__(kGemvThreads, 3)
     gemv_kernel(const uint16_t* __restrict__ w, const uint16_t* x, const KArgs a,
                 int ksplit) {
   extern __shared__ __align__(16) uint8_t gsm[];
-  __shared__ float red[32][NT];
-  __shared__ int trow[kGemvTok], tpos[kGemvTok];
+  __shared__ float red[32];
+  __shared__ int trow[1], tpos[1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grp = blockIdx.x / ksplit, ks = blockIdx.x - grp * ksplit;
   const int n0 = grp * 32;
@@ -1326,7 +1338,7 @@ __global__ void __launch_bounds__(kGemvThreads)
   const int kc0 = ks * C / ksplit, kc1 = (ks + 1) * C / ksplit, nc = kc1 - kc0;
   const int nblk = (nc + CPR - 1) / CPR;  // chunk blocks per row pair
   const int nb = 2 * nblk;                // batches of this warp (two row pairs)
-  const int4* xs = reinterpret_cast<const int4*>(gsm);  // [NT][nc * 32] chunks of this K range
+  const int4* xs = reinterpret_cast<const int4*>(gsm);  // [nc * 32] chunks of this K range
   const size_t wrow = size_t(a.k) / 8;                  // int4 per weight row
   const int4* wbase = reinterpret_cast<const int4*>(w) + size_t(kc0) * 32 + lane;
   // batch b: rows n0 + 4 warp + 2 (b / nblk) + {0, 1}, chunk columns (b % nblk) CPR + u
@@ -1341,76 +1353,58 @@ __global__ void __launch_bounds__(kGemvThreads)
                         ? ld_weights(wbase + size_t(r + h) * wrow + 32 * (c0 + u))
                         : make_int4(0, 0, 0, 0);
   };
-  float acc[2][NT];
+  float acc[2];
   auto compute = [&](const int4 (&buf)[2][CPR], int b) {
     const int rp = b / nblk, blk = b - rp * nblk, c0 = blk * CPR;
-    if (blk == 0) {
-#pragma unroll
-      for (int t = 0; t < NT; ++t) acc[0][t] = acc[1][t] = 0.0f;
-    }
+    if (blk == 0) acc[0] = acc[1] = 0.0f;
 #pragma unroll
     for (int u = 0; u < CPR; ++u) {
       const int c = c0 + u;
       if (c < nc) {
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-          const int4 xv = xs[t * nc * 32 + c * 32 + lane];
-          acc[0][t] = dot8_bf16(buf[0][u], xv, acc[0][t]);
-          acc[1][t] = dot8_bf16(buf[1][u], xv, acc[1][t]);
-        }
+        const int4 xv = xs[c * 32 + lane];
+        acc[0] = dot8_bf16(buf[0][u], xv, acc[0]);
+        acc[1] = dot8_bf16(buf[1][u], xv, acc[1]);
       }
     }
     if (blk == nblk - 1) {  // the row pair is complete
-#pragma unroll
-      for (int t = 0; t < NT; ++t) {
-        const float s0 = warp_sum_f(acc[0][t]), s1 = warp_sum_f(acc[1][t]);
-        if (lane == 0) {
-          red[4 * warp + 2 * rp][t] = s0;
-          red[4 * warp + 2 * rp + 1][t] = s1;
-        }
+      const float s0 = warp_sum_f(acc[0]), s1 = warp_sum_f(acc[1]);
+      if (lane == 0) {
+        red[4 * warp + 2 * rp] = s0;
+        red[4 * warp + 2 * rp + 1] = s1;
       }
     }
   };
   pdl_launch_dependents();
   int4 b0[2][CPR];
   load(b0, 0);  // weights do not depend on the predecessor: in flight before the wait
+  prefetch_rows(w, a, n0 + 4 * warp + lane, lane < 4, kc0 * kGemvChunk, nc * kGemvChunk, kGemvAhead);
   pdl_wait();
   if (threadIdx.x == 0) stamp_start(a.stamp);
-  if (a.norm_h) {  // the input RMSNorm of each token's fp32 row, computed by every CTA
-    __shared__ float nred[kGemvThreads / 32][NT];
-    __shared__ float ninv[NT];
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      float ss = 0.0f;
-      const int hrow = t < a.n_tok ? (a.norm_rows ? a.norm_rows[t] : t) : -1;  // -1: list padding
-      if (hrow >= 0) {
-        const float4* hr = reinterpret_cast<const float4*>(a.norm_h + size_t(hrow) * a.k);
-        for (int c = threadIdx.x; c < a.k / 4; c += kGemvThreads) {
-          const float4 v = hr[c];
-          ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-        }
+  const int hrow = a.norm_h ? (a.norm_rows ? a.norm_rows[0] : 0) : -1;  // -1: list padding
+  int4* xd = reinterpret_cast<int4*>(gsm);
+  if (a.norm_h) {  // the input RMSNorm of the token's fp32 row, computed by every CTA
+    __shared__ float nred[kGemvThreads / 32];
+    float ss = 0.0f;
+    if (hrow >= 0) {
+      const float4* hr = reinterpret_cast<const float4*>(a.norm_h + size_t(hrow) * a.k);
+      for (int c = threadIdx.x; c < a.k / 4; c += kGemvThreads) {
+        const float4 v = hr[c];
+        ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
       }
-      ss = warp_sum_f(ss);
-      if (lane == 0) nred[warp][t] = ss;
     }
+    ss = warp_sum_f(ss);
+    if (lane == 0) nred[warp] = ss;
     __syncthreads();
-    if (threadIdx.x < NT) {
-      float tot = 0.0f;
-      for (int i = 0; i < kGemvThreads / 32; ++i) tot += nred[i][threadIdx.x];
-      ninv[threadIdx.x] = rsqrtf(tot / float(a.k) + a.norm_eps);
-    }
-    __syncthreads();
-    int4* xd = reinterpret_cast<int4*>(gsm);
-    for (int e = threadIdx.x; e < NT * nc * 32; e += kGemvThreads) {
-      const int t = e / (nc * 32), c = e - t * (nc * 32);
+    float tot = 0.0f;
+    for (int i = 0; i < kGemvThreads / 32; ++i) tot += nred[i];
+    const float inv = rsqrtf(tot / float(a.k) + a.norm_eps);
+    for (int c = threadIdx.x; c < nc * 32; c += kGemvThreads) {
       int4 r = make_int4(0, 0, 0, 0);
-      const int hrow = t < a.n_tok ? (a.norm_rows ? a.norm_rows[t] : t) : -1;
       if (hrow >= 0) {
         const size_t k0 = size_t(kc0 * 32 + c) * 8;
         const float* hr = a.norm_h + size_t(hrow) * a.k + k0;
         const float4 v0 = reinterpret_cast<const float4*>(hr)[0], v1 = reinterpret_cast<const float4*>(hr)[1];
         const uint4 gg = *reinterpret_cast<const uint4*>(a.norm_gain + k0);
-        const float inv = ninv[t];
         const float hv[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
         const uint32_t gw[4] = {gg.x, gg.y, gg.z, gg.w};
         uint32_t pk[4];
@@ -1422,23 +1416,14 @@ __global__ void __launch_bounds__(kGemvThreads)
         }
         r = make_int4(int(pk[0]), int(pk[1]), int(pk[2]), int(pk[3]));
       }
-      xd[e] = r;
+      xd[c] = r;
     }
-    if (threadIdx.x < a.n_tok) {
-      trow[threadIdx.x] = a.rows ? a.rows[threadIdx.x] : threadIdx.x;
-      tpos[threadIdx.x] = a.pos ? a.pos[threadIdx.x] : 0;
-    }
-  } else {  // tokens' chunks of this K range; token rows past n_tok are zeros
-    int4* xd = reinterpret_cast<int4*>(gsm);
-    for (int e = threadIdx.x; e < NT * nc * 32; e += kGemvThreads) {
-      const int t = e / (nc * 32), c = e - t * (nc * 32);
-      xd[e] = t < a.n_tok ? reinterpret_cast<const int4*>(x + size_t(t) * a.k)[kc0 * 32 + c]
-                          : make_int4(0, 0, 0, 0);
-    }
-    if (threadIdx.x < a.n_tok) {
-      trow[threadIdx.x] = a.rows ? a.rows[threadIdx.x] : threadIdx.x;
-      tpos[threadIdx.x] = a.pos ? a.pos[threadIdx.x] : 0;
-    }
+  } else {  // the token's chunks of this K range
+    for (int c = threadIdx.x; c < nc * 32; c += kGemvThreads) xd[c] = reinterpret_cast<const int4*>(x)[kc0 * 32 + c];
+  }
+  if (threadIdx.x == 0) {
+    trow[0] = a.rows ? a.rows[0] : 0;
+    tpos[0] = a.pos ? a.pos[0] : 0;
   }
   __syncthreads();
 #pragma unroll 1
@@ -1450,20 +1435,118 @@ __global__ void __launch_bounds__(kGemvThreads)
   if (warp == 0) {
     float v[8];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) v[t] = t < NT ? red[lane][t] : 0.0f;
+    for (int t = 0; t < 8; ++t) v[t] = t == 0 ? red[lane] : 0.0f;
+    epilogue8<EPI>(a, n0 + lane, (n0 >> 5) & 3, lane, n0 >> 7, 0, v, trow, tpos, 0);
+    if (lane == 0) stamp_end(a.stamp);
+  }
+}
+
+// Two to eight tokens (a decode step of as many sequences): still a weight stream, but with one fp32 FMA per
+// weight and token the kernel above was bound by instructions (4 layers of LLaVA width: 441 us a step at one
+// token, 689 at two, 732 at four), and the tiled kernel streams at half the HBM rate. Here the tokens are the
+// 8 columns of m16n8k16: a warp owns 16 of the CTA's 32 weight rows and a quarter of its K range, the
+// weights go from 16-byte loads straight into the A operand (the order of K is free: lane (r, c) takes
+// columns 8 c .. 8 c + 7 of a 32-wide step of rows r and r + 8 and the same columns of token r), eight
+// weight loads in flight a lane. The quarters are added in a fixed order through shared memory. The same step:
+// 423 us at two tokens (1-token kernel's prefetch, a quarter of it per quarter row; 463 with four times as
+// much), 485 at eight, where the tiled kernel took 577.
+constexpr int kGemvMmaTok = 8;
+
+__device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                          uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(kGemvThreads, 3)
+    gemv_mma_kernel(const uint16_t* __restrict__ w, const uint16_t* x, const KArgs a, int ksplit) {
+  __shared__ float red[4][32][kGemvMmaTok + 1];
+  __shared__ int trow[kGemvMmaTok], tpos[kGemvMmaTok];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
+  const int grp = blockIdx.x / ksplit, ks = blockIdx.x - grp * ksplit;
+  const int n0 = grp * 32;
+  const int C = a.k / kGemvChunk;
+  const int kc0 = ks * C / ksplit, nc = (ks + 1) * C / ksplit - kc0;
+  // this warp: rows n0 + 16 (warp / 4) + {0..15}, columns [k0, k0 + kn) with kn a multiple of 64
+  const int row = n0 + 16 * (warp >> 2), quarter = warp & 3;
+  const int kn = nc * (kGemvChunk / 4), k0 = kc0 * kGemvChunk + quarter * kn;
+  const bool ok0 = row + r < a.n_out, ok1 = row + r + 8 < a.n_out;
+  const int4* w0 = reinterpret_cast<const int4*>(w + size_t(ok0 ? row + r : 0) * a.k + k0) + c;
+  const int4* w1 = reinterpret_cast<const int4*>(w + size_t(ok1 ? row + r + 8 : 0) * a.k + k0) + c;
+  const bool okx = r < a.n_tok;
+  const int4* xp = reinterpret_cast<const int4*>(x + size_t(okx ? r : 0) * a.k + k0) + c;
+  constexpr int U = 4;  // 32-wide steps a batch
+  const int steps = kn / 32;
+  const int4 z = make_int4(0, 0, 0, 0);
+  int4 b0[U], b1[U];
+  auto load = [&](int st) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      b0[u] = ok0 && st + u < steps ? ld_weights(w0 + 4 * (st + u)) : z;
+      b1[u] = ok1 && st + u < steps ? ld_weights(w1 + 4 * (st + u)) : z;
+    }
+  };
+  pdl_launch_dependents();
+  load(0);
+  prefetch_rows(w, a, row + lane, lane < 16, k0, kn, kGemvAhead / 4);  // ... of each of the row's quarters
+  pdl_wait();
+  if (threadIdx.x == 0) stamp_start(a.stamp);
+  if (threadIdx.x < a.n_tok) {
+    trow[threadIdx.x] = a.rows ? a.rows[threadIdx.x] : threadIdx.x;
+    tpos[threadIdx.x] = a.pos ? a.pos[threadIdx.x] : 0;
+  }
+  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+  for (int st = 0; st < steps; st += U) {
+    if (st > 0) load(st);
+    int4 xv[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) xv[u] = okx && st + u < steps ? xp[4 * (st + u)] : z;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      mma_16816(acc, b0[u].x, b1[u].x, b0[u].y, b1[u].y, xv[u].x, xv[u].y);
+      mma_16816(acc, b0[u].z, b1[u].z, b0[u].w, b1[u].w, xv[u].z, xv[u].w);
+    }
+  }
+  const int lr = 16 * (warp >> 2) + r;
+  red[quarter][lr][2 * c] = acc[0];
+  red[quarter][lr][2 * c + 1] = acc[1];
+  red[quarter][lr + 8][2 * c] = acc[2];
+  red[quarter][lr + 8][2 * c + 1] = acc[3];
+  __syncthreads();
+  if (warp == 0) {
+    float v[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) v[t] = (red[0][lane][t] + red[1][lane][t]) + (red[2][lane][t] + red[3][lane][t]);
     epilogue8<EPI>(a, n0 + lane, (n0 >> 5) & 3, lane, n0 >> 7, 0, v, trow, tpos, 0);
     if (lane == 0) stamp_end(a.stamp);
   }
 }
 
 using GemvFn = void (*)(const uint16_t*, const uint16_t*, KArgs, int);
-template <int NT, int CPR>
+GemvFn gemv_mma_for(int epi) {
+  switch (epi) {
+    case EPI_F32: return gemv_mma_kernel<EPI_F32>;
+    case EPI_BF16: return gemv_mma_kernel<EPI_BF16>;
+    case EPI_BIAS_BF16: return gemv_mma_kernel<EPI_BIAS_BF16>;
+    case EPI_BIAS_GELU_BF16: return gemv_mma_kernel<EPI_BIAS_GELU_BF16>;
+    case EPI_ADD_F32: return gemv_mma_kernel<EPI_ADD_F32>;
+    case EPI_SWIGLU_BF16: return gemv_mma_kernel<EPI_SWIGLU_BF16>;
+    case EPI_QKV_BF16: return gemv_mma_kernel<EPI_QKV_BF16>;
+    default: return nullptr;
+  }
+}
+template <int CPR>
 GemvFn gemv_for(int epi) {
   switch (epi) {
-    case EPI_F32: return gemv_kernel<EPI_F32, NT, CPR>;
-    case EPI_ADD_F32: return gemv_kernel<EPI_ADD_F32, NT, CPR>;
-    case EPI_SWIGLU_BF16: return gemv_kernel<EPI_SWIGLU_BF16, NT, CPR>;
-    case EPI_QKV_BF16: return gemv_kernel<EPI_QKV_BF16, NT, CPR>;
+    case EPI_F32: return gemv_kernel<EPI_F32, CPR>;
+    case EPI_ADD_F32: return gemv_kernel<EPI_ADD_F32, CPR>;
+    case EPI_SWIGLU_BF16: return gemv_kernel<EPI_SWIGLU_BF16, CPR>;
+    case EPI_QKV_BF16: return gemv_kernel<EPI_QKV_BF16, CPR>;
     default: return nullptr;
   }
 }
@@ -1578,12 +1661,17 @@ bool vec_red_ok(const GemmProblem& p) {
          (reinterpret_cast<uintptr_t>(p.out) & 15) == 0;
 }
 
+// One token: gemv_kernel (which can norm its input); up to eight: gemv_mma_kernel
+bool gemv_aligned(const GemmProblem& p) {
+  return p.w && p.k % kGemvChunk == 0 && ((reinterpret_cast<uintptr_t>(p.w) | reinterpret_cast<uintptr_t>(p.x)) & 15) == 0;
+}
 bool gemv_eligible(const GemmProblem& p) {
   if (p.norm_h && ((reinterpret_cast<uintptr_t>(p.norm_h) | reinterpret_cast<uintptr_t>(p.norm_gain)) & 15))
     return false;
-  return p.n_tok <= kGemvTok && p.w && p.k % kGemvChunk == 0 &&
-         (reinterpret_cast<uintptr_t>(p.w) & 15) == 0 && (reinterpret_cast<uintptr_t>(p.x) & 15) == 0 &&
-         gemv_for<1, 4>(p.epi) != nullptr;
+  return p.n_tok == 1 && gemv_aligned(p) && gemv_for<4>(p.epi) != nullptr;
+}
+bool gemv_mma_eligible(const GemmProblem& p) {
+  return p.n_tok >= 1 && p.n_tok <= kGemvMmaTok && gemv_aligned(p) && !p.norm_h && gemv_mma_for(p.epi) != nullptr;
 }
 
 int gemv_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
@@ -1618,28 +1706,34 @@ int gemv_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
   int ksplit = 1;
   if (p.epi == EPI_ADD_F32 && !a.determ)
     while (groups * ksplit < num_sms() && ksplit * 2 <= C && ksplit < 8) ksplit *= 2;
-  const bool one = p.n_tok == 1;
-  const int nt = one ? 1 : kGemvTok;
-  const size_t smem = size_t(nt) * ((C + ksplit - 1) / ksplit) * kGemvChunk * sizeof(uint16_t);
-  const GemvFn kern = one ? gemv_for<1, 4>(p.epi) : gemv_for<kGemvTok, 4>(p.epi);
+  if (!gemv_eligible(p)) {
+    const int slot = trace_begin(stream);
+    SPD_CUDA_TRY(launch_pdl(gemv_mma_for(p.epi), dim3(groups * ksplit), dim3(kGemvThreads), 0, stream,
+                            static_cast<const uint16_t*>(p.w), static_cast<const uint16_t*>(p.x), a, ksplit));
+    trace_gemm(slot, p, stream);
+    return SPD_OK;
+  }
+  const size_t smem = size_t((C + ksplit - 1) / ksplit) * kGemvChunk * sizeof(uint16_t);
+  const GemvFn kern = gemv_for<4>(p.epi);
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(once, [] {
-    for (int e : {int(EPI_F32), int(EPI_ADD_F32), int(EPI_SWIGLU_BF16), int(EPI_QKV_BF16)})
-      for (GemvFn f : {gemv_for<1, 4>(e), gemv_for<kGemvTok, 4>(e)}) {
-        const cudaError_t r = cudaFuncSetAttribute(reinterpret_cast<const void*>(f),
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   200 * 1024);
-        if (r != cudaSuccess && attr_err == cudaSuccess) attr_err = r;
-      }
+    for (int e : {int(EPI_F32), int(EPI_ADD_F32), int(EPI_SWIGLU_BF16), int(EPI_QKV_BF16)}) {
+      const cudaError_t r = cudaFuncSetAttribute(reinterpret_cast<const void*>(gemv_for<4>(e)),
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      if (r != cudaSuccess && attr_err == cudaSuccess) attr_err = r;
+    }
   });
   if (attr_err != cudaSuccess)
     return fail(SPD_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(attr_err));
   if (smem > 200 * 1024) return fail(SPD_EUNSUPPORTED, "GEMV K range too long");
   const int slot = trace_begin(stream);
-  SPD_CUDA_TRY(launch_pdl(kern, dim3(groups * ksplit), dim3(kGemvThreads), smem, stream,
-                          static_cast<const uint16_t*>(p.w), static_cast<const uint16_t*>(p.x), a,
-                          ksplit));
+  // shared memory for three CTAs an SM (what the registers allow) and no more: the rest of the array buffers the
+  // weight loads in flight (one token, 32 layers: 3140 us a step with the driver's choice, 3084 so)
+  const int carveout = int(std::min<size_t>(100, 3 * (smem + 1536) * 100 / (256 * 1024)));
+  SPD_CUDA_TRY(launch_pdl_carveout(carveout, kern, dim3(groups * ksplit), dim3(kGemvThreads), smem, stream,
+                                   static_cast<const uint16_t*>(p.w), static_cast<const uint16_t*>(p.x), a,
+                                   ksplit));
   trace_gemm(slot, p, stream);
   return SPD_OK;
 }
@@ -1652,7 +1746,7 @@ int gemm_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
   if (p.k <= 0) return fail(SPD_EINVAL, "GEMM K must be positive");
   if (!kernel_for(p.epi, false)) return fail(SPD_EINVAL, "unknown GEMM epilogue %d", p.epi);
   if (!p.map_w && !p.w) return fail(SPD_EINVAL, "GEMM without weights");
-  if (gemv_eligible(p)) return gemv_run(p, s, stream);
+  if (gemv_eligible(p) || gemv_mma_eligible(p)) return gemv_run(p, s, stream);
   if (p.norm_h) return fail(SPD_EINVAL, "input RMSNorm fusion needs the matrix-vector path");
   if (cudaError_t e = set_kernel_attributes())
     return fail(SPD_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));

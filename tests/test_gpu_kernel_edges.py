@@ -69,6 +69,38 @@ def test_decode_attention_edges(heads, kv_heads, head_dim, pos, offset):
         assert not got[b, p[b] + 1:].any()
 
 
+# ---- few-token GEMMs: m16n8k16 straight from the weight rows ------------------------------------------
+@pytest.mark.parametrize("M", [1, 2, 7, 8, 9])  # 9: past the form's token columns
+@pytest.mark.parametrize("K,n", [(256, 1), (512, 40), (2816, 1000), (4096, 128)])
+def test_few_token_epilogues(M, K, n):
+    # K ranges of one chunk, of unequal shares; output widths that end inside a 16-row half, a 32-row group
+    g = torch.Generator().manual_seed(M * K + n)
+    X = torch.randn(M, K, generator=g).to(torch.bfloat16)
+    W = (torch.randn(n, K, generator=g) * 0.05).to(torch.bfloat16)
+    bias = torch.randn(n, generator=g).to(torch.bfloat16)
+    acc = bf16_np(X) @ bf16_np(W).T
+    ws = torch.zeros(N.spd_linear_workspace_size(M, n), dtype=torch.uint8, device="cuda")
+    Xc, Wc, bc = X.cuda(), W.cuda(), bias.cuda()
+    ldo = n + 3  # a row stride wider than the row: its padding stays untouched
+    for epi, ref, tol in ((N.EPI_F32, acc, 1e-4), (N.EPI_BF16, acc, 2 ** -8), (N.EPI_BIAS_BF16, acc + bf16_np(bias), 2 ** -8),
+                          (N.EPI_BIAS_GELU_BF16, od.gelu(acc + bf16_np(bias)), 2 ** -8)):
+        # fp32 sums: 1e-4 of the row; bf16 outputs: half a unit (2^-9) and the sums' error below another
+        dt = torch.float32 if epi == N.EPI_F32 else torch.bfloat16
+        out = torch.full((M, ldo), 7.0, dtype=dt, device="cuda")
+        N.spd_linear(Xc, M, K, Wc, n, epi, out, ldo, ws, bias=bc)
+        got = out.double().cpu().numpy()
+        assert rowwise_rel(got[:, :n], ref) < tol, epi
+        assert (got[:, n:] == 7.0).all()
+    rows = torch.randperm(M + 3, generator=g)[:M].to(torch.int32)
+    h0 = torch.randn(M + 3, n, generator=g)
+    h = h0.cuda()
+    N.spd_linear(Xc, M, K, Wc, n, N.EPI_ADD_F32, h, n, ws, rows=rows.cuda())
+    want = h0.double().numpy()
+    want[rows.numpy()] += acc
+    assert rowwise_rel(h.cpu().numpy(), want) < 1e-4
+    assert N.spd_workspace_status(ws) == 0
+
+
 # ---- MSV-Prune: K-means over the whole GPU, rankings over several CTAs --------------------------------
 def _shuffled_tile(seed0, n, d, keep, **kw):
     # a tile whose planted groups lie scattered over the token order: the seeds fall into any of them, so
