@@ -2,18 +2,25 @@
 // restricted to the attention-active tokens (VSkip-Attn, Sec. 3.2: a skipped token is not a
 // query, but it stays a key and a value for every other token of its sequence).
 //
-// One CTA = up to 128 active queries of one sequence x one head (the MMA's M = 128 rows):
-//   warp 4     TMA producer: the Q tile once, then blocks of 128 keys of K and V into a two-stage
-//              ring (128-byte swizzle, boxes of 64 head-dim columns)
-//   warp 5     MMA issuer: S = Q K^T into TMEM (kind::f16, fp32), then O += P V with P from shared
-//              memory and V read in place as an MN-major operand (the layout its TMA box has)
-//   warps 0-3  softmax: thread r owns query row r (TMEM lane r); online softmax in fp32 with exp2;
-//              P rounded to bf16 into shared memory as a K-major swizzled operand; O rescaled in
-//              TMEM when a row's running maximum grows; at the end O / l goes to HBM in bf16
-// S alternates between two TMEM buffers, so S of block j + 1 is computed while the softmax of
-// block j reads block j's (two passes: the maximum, then the exponentials, sum and P). A query at
-// position p sees keys 0..p of its own sequence. Every wait is bounded (status SPD_ETIMEOUT, no
-// hang).
+// One CTA = up to 128 active queries of one sequence x one head (the MMA's M = 128 rows), two CTAs an SM:
+//   warp 4     TMA producer: the Q tile once, then blocks of 64 keys of K and of V into two-stage rings
+//              (128-byte swizzle, boxes of 64 head-dim columns)
+//   warp 5     MMA issuer: S = Q K^T into TMEM (kind::f16, fp32), then O += P V with P read from TMEM and V
+//              read in place as an MN-major operand (the layout its TMA box has)
+//   warps 0-3  softmax: thread r owns query row r (TMEM lane r); one pass over the block's 64 scores in
+//              registers, online softmax in fp32 with exp2, P rounded to bf16 over S's own TMEM columns; O
+//              is rescaled in TMEM only when a row's maximum grew by more than a factor of two (until then
+//              P, l and O keep the older, smaller reference); at the end O / l goes to HBM in bf16
+// S alternates between two TMEM buffers, so S of block j + 1 is computed while the softmax of block j
+// runs. A query at position p sees keys 0..p of its own sequence; tiles run from the last to the first (in
+// causal order the longest first), all heads of a tile side by side. Every wait is bounded (status
+// SPD_ETIMEOUT, no hang).
+//
+// What bounds it: a 64-key block is 640 cycles of tensor work (the S products are limited by the operand reads
+// from shared memory), 512 of exponentials and about 300 instructions a softmax thread; the CTAs of an SM fill
+// each other's waits. With one CTA of 128-key blocks an SM (P through shared memory, two passes over S, a
+// rescale at every new maximum) the tensor pipe idled through each softmax: four requests of 1021-3302
+// tokens, 28 heads of 128, 492 us; so 243 us (0.47 of the burst bf16 rate, counting the causal half only).
 #include <cuda_bf16.h>
 #include <math.h>
 #include <stdint.h>
@@ -29,31 +36,42 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kTK = 128;              // keys per block (S columns, K of the PV product)
-constexpr uint32_t kBox = 128 * 128;  // one TMA box: 128 rows x 64 bf16
+constexpr int kTK = 64;                // keys per block (S columns, K of the PV product)
+constexpr uint32_t kQBox = 128 * 128;  // one TMA box of Q: 128 rows x 64 bf16
+constexpr uint32_t kKBox = kTK * 128;  // ... of K and V: 64 rows
 constexpr int kThreads = 192;
+constexpr uint32_t kTmemCols = 256;    // S: two buffers [0, 64) and [64, 128); O: [128, 128 + HD)
+// log2 growth of a row's maximum that rescales O. The largest weight of a row is 1, exact in bf16, only
+// relative to its own maximum: relative error against 64 bits 2.016e-3 / 2.019e-3 / 2.026e-3 / 2.049e-3 /
+// 2.072e-3 at 0 / 0.5 / 1 / 2 / 8 (2.037e-3 with the sum over unrounded weights and a rescale at every new
+// maximum, as before), 257 / 248 / 243 / 239 / 237 us for four requests of 1021-3302 tokens.
+constexpr float kRescale = 1.0f;
 
 template <int HD>
 struct AttnSmem {
   static constexpr int kChunks = HD / 64;                       // 64-column boxes per row
   static constexpr uint32_t q = 0;                              // Q tile
-  static constexpr uint32_t k = q + kChunks * kBox;             // K stages
-  static constexpr uint32_t v = k + 2 * kChunks * kBox;         // V stages
-  static constexpr uint32_t p = v + 2 * kChunks * kBox;         // P: two 64-key halves
-  static constexpr uint32_t bars = p + 2 * kBox;
+  static constexpr uint32_t k = q + kChunks * kQBox;            // K stages
+  static constexpr uint32_t v = k + 2 * kChunks * kKBox;        // V stages
+  static constexpr uint32_t bars = v + 2 * kChunks * kKBox;
   static constexpr uint32_t bytes = bars + 128 + 1024;          // + alignment slack
 };
 
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
 template <int HD>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, 2)
     attn_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                    const __grid_constant__ CUtensorMap map_kv, __nv_bfloat16* __restrict__ o,
-                   int ldo, const int4* tiles, const int32_t* q_pos, int n_heads, int n_kv_heads,
+                   int ldo, const int4* tiles, int n_tiles, const int32_t* q_pos, int n_heads, int n_kv_heads,
                    int v_off, float scale_log2, int* status, long long budget,
                    unsigned long long* stamp) {
   using L = AttnSmem<HD>;
@@ -61,30 +79,31 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
   uint64_t* q_full = reinterpret_cast<uint64_t*>(smem + L::bars);
-  uint64_t* kv_full = q_full + 1;   // [2] K and V block landed
-  uint64_t* kv_empty = q_full + 3;  // [2] its PV product has completed
-  uint64_t* s_full = q_full + 5;    // [2] S of block j is in TMEM buffer j % 2
-  uint64_t* s_free = q_full + 7;    // [2] the softmax warps have read S buffer j % 2
-  uint64_t* p_full = q_full + 9;    // P written and O rescaled
-  uint64_t* o_done = q_full + 10;   // PV product of the current block completed
-  uint64_t* drain = q_full + 11;    // every MMA completed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(q_full + 12);
+  uint64_t* k_full = q_full + 1;   // [2] K block landed
+  uint64_t* k_empty = q_full + 3;  // [2] its S product has completed
+  uint64_t* v_full = q_full + 5;   // [2] V block landed
+  uint64_t* v_empty = q_full + 7;  // [2] its PV product has completed
+  uint64_t* s_full = q_full + 9;   // [2] S of block j is in TMEM buffer j % 2
+  uint64_t* p_full = q_full + 11;  // [2] P of block j written (S read) and O rescaled; two, since a softmax
+                                   // warp may finish block j + 1 before another has finished block j
+  uint64_t* o_done = q_full + 13;  // PV product of the current block completed
+  uint64_t* drain = q_full + 14;   // every MMA completed: O is final
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(q_full + 15);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = blockIdx.y;
+  const int h = blockIdx.x % n_heads, tile = n_tiles - 1 - int(blockIdx.x) / n_heads;
   const int hk = h / (n_heads / n_kv_heads);
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
     for (int s = 0; s < 2; ++s) {
-      mbar_init(&kv_full[s], 1);
-      mbar_init(&kv_empty[s], 1);
+      mbar_init(&k_full[s], 1);
+      mbar_init(&k_empty[s], 1);
+      mbar_init(&v_full[s], 1);
+      mbar_init(&v_empty[s], 1);
+      mbar_init(&s_full[s], 1);
+      mbar_init(&p_full[s], 4);  // one arrival per softmax warp
     }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&s_full[b], 1);
-      mbar_init(&s_free[b], 4);  // one arrival per softmax warp
-    }
-    mbar_init(p_full, 4);
     mbar_init(o_done, 1);
     mbar_init(drain, 1);
     *abort_flag = 0;
@@ -93,14 +112,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     prefetch_tmap(&map_kv);
   }
   if (warp == 4) {
-    tmem_alloc(tmem_slot, 512);  // S: two buffers, columns [0, 128) and [128, 256); O: [256, 256 + HD)
+    tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const uint32_t t_o = tmem + 256;  // S buffer b at tmem + 128 b
+  const uint32_t t_o = tmem + 2 * kTK;  // S buffer b at tmem + 64 b
 
   // Nothing written by an earlier kernel of the stream is read before the grid dependency wait:
   // under programmatic overlap this kernel's prologue may run while several earlier kernels are
@@ -109,35 +128,38 @@ __global__ void __launch_bounds__(kThreads, 1)
   pdl_launch_dependents();
   pdl_wait();
   if (threadIdx.x == 0) stamp_start(stamp);
-  const int4 tl = tiles[blockIdx.x];
+  const int4 tl = tiles[tile];
   const int q0 = tl.x, nq = tl.y, kv0 = tl.z, len = tl.w;
   const int p_last = q_pos[q0 + nq - 1];  // positions ascend within a tile
   const int nkb = max(1, min((p_last + kTK) / kTK, (len + kTK - 1) / kTK));
   const int my_pos = threadIdx.x < 128 ? q_pos[q0 + min(int(threadIdx.x), nq - 1)] : 0;
 
-  int issued = 0;  // K/V blocks whose loads the producer issued
+  int issued_k = 0, issued_v = 0;  // blocks whose loads the producer issued
   if (warp == 4) {
     if (lane == 0) {
       // ---- TMA producer ----
       const uint64_t pol_q = policy_evict_first(), pol_kv = policy_evict_last();
-      mbar_arrive_expect_tx(q_full, L::kChunks * kBox);
+      mbar_arrive_expect_tx(q_full, L::kChunks * kQBox);
       for (int c = 0; c < L::kChunks; ++c)
-        tma_load_2d(smem + L::q + c * kBox, &map_q, q_full, h * HD + c * 64, q0, pol_q);
-      for (int j = 0; j < nkb; ++j) {
+        tma_load_2d(smem + L::q + c * kQBox, &map_q, q_full, h * HD + c * 64, q0, pol_q);
+      auto load = [&](int j, uint64_t* full, uint64_t* empty, uint32_t at, int x0) -> bool {
         const int s = j & 1;
-        if (j >= 2 && !mbar_wait(&kv_empty[s], ((j >> 1) - 1) & 1, abort_flag, budget)) {
+        if (j >= 2 && !mbar_wait(&empty[s], ((j >> 1) - 1) & 1, abort_flag, budget)) {
           *abort_flag = 1;
           set_status(status, SPD_ETIMEOUT);
-          break;
+          return false;
         }
-        mbar_arrive_expect_tx(&kv_full[s], 2 * L::kChunks * kBox);
-        for (int c = 0; c < L::kChunks; ++c) {
-          const int x = hk * HD + c * 64, y = kv0 + j * kTK;
-          tma_load_2d(smem + L::k + (s * L::kChunks + c) * kBox, &map_kv, &kv_full[s], x, y, pol_kv);
-          tma_load_2d(smem + L::v + (s * L::kChunks + c) * kBox, &map_kv, &kv_full[s], v_off + x, y,
-                      pol_kv);
-        }
-        issued = j + 1;
+        mbar_arrive_expect_tx(&full[s], L::kChunks * kKBox);
+        for (int c = 0; c < L::kChunks; ++c)
+          tma_load_2d(smem + at + (s * L::kChunks + c) * kKBox, &map_kv, &full[s], x0 + hk * HD + c * 64,
+                      kv0 + j * kTK, pol_kv);
+        return true;
+      };
+      for (int j = 0; j < nkb; ++j) {
+        if (!load(j, k_full, k_empty, L::k, 0)) break;
+        issued_k = j + 1;
+        if (!load(j, v_full, v_empty, L::v, v_off)) break;
+        issued_v = j + 1;
       }
     }
   } else if (warp == 5) {
@@ -145,37 +167,37 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ---- MMA issuer ----
       const uint32_t id_s = idesc_bf16_f32(128, kTK);
       const uint32_t id_o = idesc_bf16_f32(128, HD) | (1u << 16);  // V is MN-major
-      const uint32_t sq = smem_u32(smem + L::q), sp = smem_u32(smem + L::p);
+      const uint32_t sq = smem_u32(smem + L::q);
       bool ok = mbar_wait(q_full, 0, abort_flag, budget);
       auto issue_s = [&](int j) -> bool {
         const int s = j & 1;
-        if (!mbar_wait(&kv_full[s], (j >> 1) & 1, abort_flag, budget)) return false;
-        // S buffer s was last read by the softmax of block j - 2
-        if (j > 1 && !mbar_wait(&s_free[s], ((j >> 1) - 1) & 1, abort_flag, budget)) return false;
+        if (!mbar_wait(&k_full[s], (j >> 1) & 1, abort_flag, budget)) return false;
+        // S buffer s holds P of block j - 2 until its PV product has completed
+        if (j > 1 && !mbar_wait(o_done, j & 1, abort_flag, budget)) return false;
         tc_fence_after();
-        const uint32_t sk = smem_u32(smem + L::k + s * L::kChunks * kBox);
+        const uint32_t sk = smem_u32(smem + L::k + s * L::kChunks * kKBox);
 #pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * kBox + (kk & 3) * 32;
-          mma_bf16(tmem + 128 * s, sdesc_k128(sq + off), sdesc_k128(sk + off), id_s, kk > 0 ? 1u : 0u);
-        }
+        for (int kk = 0; kk < HD / 16; ++kk)
+          mma_bf16(tmem + kTK * s, sdesc_k128(sq + (kk >> 2) * kQBox + (kk & 3) * 32),
+                   sdesc_k128(sk + (kk >> 2) * kKBox + (kk & 3) * 32), id_s, kk > 0 ? 1u : 0u);
         mma_commit(&s_full[s]);
+        mma_commit(&k_empty[s]);
         return true;
       };
       if (ok) ok = issue_s(0);
       for (int j = 0; j < nkb && ok; ++j) {
+        const int s = j & 1;
         if (j + 1 < nkb && !(ok = issue_s(j + 1))) break;
-        if (!(ok = mbar_wait(p_full, j & 1, abort_flag, budget))) break;
+        if (!(ok = mbar_wait(&v_full[s], (j >> 1) & 1, abort_flag, budget))) break;
+        if (!(ok = mbar_wait(&p_full[s], (j >> 1) & 1, abort_flag, budget))) break;
         tc_fence_after();
-        const uint32_t sv = smem_u32(smem + L::v + (j & 1) * L::kChunks * kBox);
+        const uint32_t sv = smem_u32(smem + L::v + s * L::kChunks * kKBox);
 #pragma unroll
-        for (int kk = 0; kk < kTK / 16; ++kk) {
-          const uint64_t ad = sdesc_k128(sp + (kk >> 2) * kBox + (kk & 3) * 32);
-          const uint64_t bd = sdesc_mn128(sv + kk * 2048, kBox);
-          mma_bf16(t_o, ad, bd, id_o, (j > 0 || kk > 0) ? 1u : 0u);
-        }
+        for (int kk = 0; kk < kTK / 16; ++kk)
+          mma_bf16_ts(t_o, tmem + kTK * s + 8 * kk, sdesc_mn128(sv + kk * 2048, kKBox), id_o,
+                      (j > 0 || kk > 0) ? 1u : 0u);
         mma_commit(o_done);
-        mma_commit(&kv_empty[j & 1]);
+        mma_commit(&v_empty[s]);
       }
       if (!ok) {
         *abort_flag = 1;
@@ -189,86 +211,70 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ---- softmax and epilogue: warp w reads TMEM lanes [32 w, 32 w + 32) ----
     const int r = warp * 32 + lane;  // query row of the tile
     const uint32_t lanes = static_cast<uint32_t>(warp * 32) << 16;
-    uint8_t* prow = smem + L::p + r * 128;
-    float m_run = -INFINITY, l_run = 0.0f;
+    const float grow = kRescale / scale_log2;
+    float m_run = -INFINITY, l_run = 0.0f;  // the row's reference maximum (raw scores) and sum
+    const int pos_min = __shfl_sync(0xffffffffu, my_pos, 0);  // the warp's first row sees the fewest keys
     bool ok = true;
     for (int j = 0; j < nkb; ++j) {
-      const int sb = j & 1;
-      if (!(ok = __all_sync(0xffffffffu, mbar_wait(&s_full[sb], (j >> 1) & 1, abort_flag, budget))))
+      const uint32_t t_s = tmem + kTK * (j & 1) + lanes;
+      if (!(ok = __all_sync(0xffffffffu, mbar_wait(&s_full[j & 1], (j >> 1) & 1, abort_flag, budget))))
         break;
       tc_fence_after();
-      const uint32_t t_s = tmem + 128 * sb + lanes;
+      float v[kTK];
+      tmem_ld64(t_s, v);
       const int kb = j * kTK;
-      // Two passes over the block's S row, 32 columns at a time in rolled loops (small code; the
-      // fully unrolled single pass held all 128 values in 254 registers and its first run cost
-      // 3 us against 1.4 for the second block): the row maximum, then 2^(s - m), the row sum and
-      // P. The next block's S goes to the other TMEM buffer meanwhile.
-      float mx = -INFINITY;
-#pragma unroll 1
-      for (int c = 0; c < kTK / 32; ++c) {
-        float v[32];
-        tmem_ld32(t_s + c * 32, v);
-        float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+      if (pos_min < kb + kTK - 1) {  // some row of the warp does not see the whole block (warp-uniform)
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float x = (kb + c * 32 + i <= my_pos) ? v[i] * scale_log2 : -INFINITY;
-          m4[i & 3] = fmaxf(m4[i & 3], x);
-        }
-        mx = fmaxf(mx, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
+        for (int i = 0; i < kTK; ++i)
+          if (kb + i > my_pos) v[i] = -INFINITY;
       }
-      const float m_new = fmaxf(m_run, mx);  // finite: block 0 holds key 0 <= every position
-      const float corr = exp2f(m_run - m_new);  // 0 on the first block
-      if (j > 0) {
-        // the previous PV product has completed: P's buffer is free and O can be rescaled
+      float m4[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+      for (int i = 4; i < kTK; ++i) m4[i & 3] = fmaxf(m4[i & 3], v[i]);
+      const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+      if (j == 0) {
+        m_run = mx;  // finite: block 0 holds key 0 <= every position
+      } else if (__any_sync(0xffffffffu, mx > m_run + grow)) {
+        // the previous PV product has completed (the one before it had when these scores came): O can be
+        // rescaled
         if (!(ok = __all_sync(0xffffffffu, mbar_wait(o_done, (j - 1) & 1, abort_flag, budget))))
           break;
         tc_fence_after();
-        if (__any_sync(0xffffffffu, corr != 1.0f)) {
+        const float m_new = fmaxf(m_run, mx);
+        const float corr = ex2((m_run - m_new) * scale_log2);
+        m_run = m_new;
+        l_run *= corr;
 #pragma unroll 1
-          for (int c = 0; c < HD / 32; ++c) {
-            float v[32];
-            tmem_ld32(t_o + lanes + c * 32, v);
+        for (int c = 0; c < HD / 32; ++c) {
+          float ov[32];
+          tmem_ld32(t_o + lanes + c * 32, ov);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] *= corr;
-            tmem_st32(t_o + lanes + c * 32, v);
-          }
+          for (int i = 0; i < 32; ++i) ov[i] *= corr;
+          tmem_st32(t_o + lanes + c * 32, ov);
         }
       }
-      // P in bf16: row r of a K-major operand in the 128-byte swizzle layout (16-byte unit u of
-      // the row at position u ^ (r % 8)), keys [0, 64) and [64, 128) in two boxes
-      float rs = 0.0f;
-#pragma unroll 1
-      for (int c = 0; c < kTK / 32; ++c) {
-        float v[32];
-        tmem_ld32(t_s + c * 32, v);
-        float r4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      const float off = m_run * scale_log2;
+      float r4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      uint32_t pk[kTK / 2];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float x = (kb + c * 32 + i <= my_pos) ? v[i] * scale_log2 : -INFINITY;
-          v[i] = exp2f(x - m_new);
-          r4[i & 3] += v[i];
-        }
-        rs += (r4[0] + r4[1]) + (r4[2] + r4[3]);
-#pragma unroll
-        for (int uu = 0; uu < 4; ++uu) {
-          const int u = 4 * c + uu;
-          const uint4 w = make_uint4(pack_bf16(v[8 * uu], v[8 * uu + 1]), pack_bf16(v[8 * uu + 2], v[8 * uu + 3]),
-                                     pack_bf16(v[8 * uu + 4], v[8 * uu + 5]),
-                                     pack_bf16(v[8 * uu + 6], v[8 * uu + 7]));
-          *reinterpret_cast<uint4*>(prow + (u >> 3) * kBox + (((u & 7) ^ (r & 7)) << 4)) = w;
-        }
+      for (int i = 0; i < kTK; i += 2) {
+        const float p0 = ex2(fmaf(v[i], scale_log2, -off)), p1 = ex2(fmaf(v[i + 1], scale_log2, -off));
+        const uint32_t pr = pack_bf16(p0, p1);
+        r4[i & 2] += __uint_as_float(pr << 16);  // the sum of the weights as the product sees them
+        r4[(i & 2) + 1] += __uint_as_float(pr & 0xffff0000u);
+        pk[i >> 1] = pr;
       }
-      l_run = l_run * corr + rs;
-      m_run = m_new;
+      l_run += (r4[0] + r4[1]) + (r4[2] + r4[3]);
+      float pf[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) pf[i] = __uint_as_float(pk[i]);
+      tmem_st32(t_s, pf);  // over the scores: keys 2 i and 2 i + 1 in column i
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&s_free[sb]);  // S buffer sb read (both passes)
-      fence_proxy_async_smem();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(p_full);
+      if (lane == 0) mbar_arrive(&p_full[j & 1]);
     }
-    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_done, (nkb - 1) & 1, abort_flag, budget));
+    // (not o_done: here its phase may be any of the last two, which a parity cannot tell apart)
+    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(drain, 0, abort_flag, budget));
     if (!ok) {
       *abort_flag = 1;
       set_status(status, SPD_ETIMEOUT);
@@ -295,16 +301,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 128 && *abort_flag) {
-    // loads issued but never consumed land before the CTA exits (without an abort the last PV
-    // product consumed every issued block)
+    // loads issued but never consumed land before the CTA exits (without an abort the last products
+    // consumed every issued block)
     volatile int no_abort = 0;
     mbar_wait(q_full, 0, &no_abort, budget);
-    for (int j = max(0, issued - 2); j < issued; ++j)
-      mbar_wait(&kv_full[j & 1], (j >> 1) & 1, &no_abort, budget);
+    for (int j = max(0, issued_k - 2); j < issued_k; ++j) mbar_wait(&k_full[j & 1], (j >> 1) & 1, &no_abort, budget);
+    for (int j = max(0, issued_v - 2); j < issued_v; ++j) mbar_wait(&v_full[j & 1], (j >> 1) & 1, &no_abort, budget);
   }
   __syncwarp();
   tc_fence_after();
-  if (warp == 4) tmem_dealloc(tmem, 512);
+  if (warp == 4) tmem_dealloc(tmem, kTmemCols);
   if (threadIdx.x == 0) stamp_end(stamp);
 }
 
@@ -320,8 +326,8 @@ int launch(const CUtensorMap& mq, const CUtensorMap& mkv, void* o, int ldo, cons
     attr = true;
   }
   const float scale_log2 = 1.4426950408889634f / sqrtf(float(HD));
-  SPD_CUDA_TRY(launch_pdl(attn_tc_kernel<HD>, dim3(n_tiles, n_heads), dim3(kThreads), L::bytes,
-                          stream, mq, mkv, static_cast<__nv_bfloat16*>(o), ldo, tiles, q_pos,
+  SPD_CUDA_TRY(launch_pdl(attn_tc_kernel<HD>, dim3(n_tiles * n_heads), dim3(kThreads), L::bytes,
+                          stream, mq, mkv, static_cast<__nv_bfloat16*>(o), ldo, tiles, n_tiles, q_pos,
                           n_heads, n_kv_heads, v_off, scale_log2, status, kWaitBudget, stamp));
   return SPD_OK;
 }

@@ -166,3 +166,21 @@ def test_anchor_ranking_with_ties(n):
     v["attn"][:] = np.random.default_rng(n).integers(0, 7, v["attn"].shape).astype(np.float32)
     g = gpu_prune(v, n // 2, 0, has_cls=False, attn_form=1, n_clusters=1, anchor_ratio=1.0)
     np.testing.assert_array_equal(g["keep_idx"][0], op.select_anchors(v["attn"][0, 0].astype(np.float64), n // 2))
+
+
+# ---- prefill attention: 64-key blocks, P in TMEM, rescales only where a maximum doubled ----------------
+@pytest.mark.parametrize("lens,H,Hkv,hd,frac,ramp", [
+    ([63, 64, 65, 1, 191, 193], 4, 2, 128, 1.0, 0.0),  # lengths at the edges of key blocks
+    ([127, 128, 129, 257], 4, 4, 64, 0.6, 0.0),        # ... and of query tiles
+    ([700], 7, 1, 128, 0.9, 2.0),                      # maxima that grow by less than the threshold a block
+    ([700], 2, 2, 64, 0.9, 40.0),                      # ... by more at every block
+    ([1500, 40], 2, 1, 128, 0.05, 8.0),                # few queries far down a long sequence
+    ([2996, 1021], 14, 2, 128, 1.0, 0.0),              # many blocks and CTAs: warps of a CTA run ahead of others
+])
+def test_attention_edges(lens, H, Hkv, hd, frac, ramp):
+    from tests import test_gpu_attention as A
+    q, q_pos, q_cu, kv, cu = A.case(lens, H, Hkv, hd, frac, seed=sum(lens) + H, ramp=ramp)
+    got = A.run(q, q_pos, q_cu, kv, cu, H, Hkv, hd)
+    ref = A.oracle_attention(q, q_pos, q_cu, kv, cu, H, Hkv, hd)
+    assert np.isfinite(got).all()
+    assert rowwise_rel(got, ref) < A.TOL
