@@ -315,6 +315,7 @@ static GemmScratch scratch_from(Carve& cv) {
   s.acc = nullptr;
   s.acc_floats = 0;
   s.status = cv.status();
+  s.cleared = nullptr;
   return s;
 }
 // The accumulation buffers, carved last in a workspace (after the activation buffers).
@@ -336,7 +337,8 @@ extern "C" int spd_linear(const uint16_t* X, int M, int K, const uint16_t* W, in
   take_acc(cv, s);
   if (!cv.fits()) return fail(SPD_ENOSPC, "linear workspace too small");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (int rc = gemm_scratch_clear(s, st)) return rc;
+  GemmCleared cleared;
+  s.cleared = &cleared;
   GemmProblem p{};
   p.w = W;
   p.x = X;
@@ -406,7 +408,8 @@ extern "C" int spd_linear_noalloc(const uint16_t* X, int M, int K, const uint16_
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the status word and the counters start at zero (a failed earlier call may have left them set)
   SPD_CUDA_TRY(cudaMemsetAsync(base, 0, 256, st));
-  if (int rc = gemm_scratch_clear(s, st)) return rc;
+  SPD_CUDA_TRY(cudaMemsetAsync(s.counters, 0, s.n_counters * sizeof(int), st));
+  s.cleared = nullptr;
   GemmProblem p{};
   p.w = W;
   p.x = X;
@@ -444,7 +447,8 @@ extern "C" int spd_project(const spd_model* m, const uint16_t* vis, int rows, co
   take_acc(cv, s);
   if (!cv.fits()) return fail(SPD_ENOSPC, "project workspace too small");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (int rc = gemm_scratch_clear(s, st)) return rc;
+  GemmCleared cleared;
+  s.cleared = &cleared;
   GemmProblem p{};
   p.map_w = &m->m_p1;
   p.w = m->pw1;
@@ -828,7 +832,8 @@ extern "C" int spd_prefill(const spd_model* m, const uint16_t* x, int T, const i
   for (int l = 0; l < c.n_layers; ++l) plan_layer(P, l, mask ? mask + size_t(l) * T : nullptr, cu, B, T);
   int32_t* dl = bf.lists;
   SPD_CUDA_TRY(cudaMemcpyAsync(dl, P.hl.data(), P.end * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-  if (int rc = gemm_scratch_clear(bf.gs, st)) return rc;
+  GemmCleared cleared;
+  bf.gs.cleared = &cleared;
   if (int rc = bf16_to_f32_run(x, h, size_t(T) * c.d_model, st)) return rc;
   for (int l = 0; l < c.n_layers; ++l)
     if (int rc = run_layer(m, l, P.ll[l], P, bf, dl, h, T, st)) return rc;
@@ -923,7 +928,8 @@ extern "C" int spd_prefill_adaptive(const spd_model* m, const uint16_t* x, int T
     SPD_CUDA_TRY(cudaMemcpyAsync(ab.text, text.data(), text.size() * sizeof(int32_t),
                                  cudaMemcpyHostToDevice, st));
   SPD_CUDA_TRY(cudaMemsetAsync(ab.s_skip, 0, T * sizeof(float), st));
-  if (int rc = gemm_scratch_clear(bf.gs, st)) return rc;
+  GemmCleared cleared;
+  bf.gs.cleared = &cleared;
   if (int rc = bf16_to_f32_run(x, h, size_t(T) * D, st)) return rc;
 
   // logit lens of nc candidate tokens (device list): final RMSNorm, then the unembedding with the
@@ -1068,7 +1074,8 @@ extern "C" int spd_prefill_kv(const spd_model* m, const uint16_t* x, int T, cons
   for (int l = 0; l < c.n_layers; ++l) plan_layer(P, l, mask ? mask + size_t(l) * T : nullptr, cu, B, T);
   int32_t* dl = bf.lists;
   SPD_CUDA_TRY(cudaMemcpyAsync(dl, P.hl.data(), P.end * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-  if (int rc = gemm_scratch_clear(bf.gs, st)) return rc;
+  GemmCleared cleared;
+  bf.gs.cleared = &cleared;
   if (int rc = bf16_to_f32_run(x, h, size_t(T) * c.d_model, st)) return rc;
   const size_t layer_rows = size_t(B) * max_len, row = 2 * size_t(c.n_kv_heads) * c.head_dim;
   for (int l = 0; l < c.n_layers; ++l) {
@@ -1116,7 +1123,8 @@ extern "C" int spd_decode(const spd_model* m, const uint16_t* x, int B, const in
   for (int l = 0; l < c.n_layers; ++l) plan_layer(P, l, nullptr, cu.data(), B, B);
   int32_t* dl = bf.lists;
   SPD_CUDA_TRY(cudaMemcpyAsync(dl, P.hl.data(), P.end * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-  if (int rc = gemm_scratch_clear(bf.gs, st)) return rc;
+  GemmCleared cleared;
+  bf.gs.cleared = &cleared;
   if (int rc = bf16_to_f32_run(x, h, size_t(B) * c.d_model, st)) return rc;
   const size_t layer_rows = size_t(B) * max_len, row = 2 * size_t(c.n_kv_heads) * c.head_dim;
   for (int l = 0; l < c.n_layers; ++l) {

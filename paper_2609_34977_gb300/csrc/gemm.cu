@@ -1247,12 +1247,6 @@ int make_map(CUtensorMap* map, const void* ptr, int inner, int outer, int box_ou
 
 }  // namespace
 
-int gemm_scratch_clear(const GemmScratch& s, cudaStream_t stream) {
-  SPD_CUDA_TRY(cudaMemsetAsync(s.counters, 0, s.n_counters * sizeof(int), stream));
-  if (s.acc_floats) SPD_CUDA_TRY(cudaMemsetAsync(s.acc, 0, s.acc_floats * sizeof(float), stream));
-  return SPD_OK;
-}
-
 namespace {
 std::atomic<int> g_deterministic{0};
 }
@@ -1273,7 +1267,7 @@ int make_operand_map(CUtensorMap* map, const void* ptr, int inner, int outer, in
 
 namespace {
 
-// ---- matrix-vector path (one token, or up to eight: a decode step) --------------------------------
+// ---- matrix-vector path (one token, or up to 16: a decode step) -----------------------------------
 // With a handful of tokens the contraction is a pure weight stream: no tensor-core tile can be
 // filled, and the tiled kernel's fixed costs (TMEM, barriers, a ring sized for wide tiles) and its
 // shared-memory traffic per weight byte cap it well below the HBM roof. At one token each CTA owns 32
@@ -1441,16 +1435,16 @@ __global__ void __launch_bounds__(kGemvThreads, 3)
   }
 }
 
-// Two to eight tokens (a decode step of as many sequences): still a weight stream, but with one fp32 FMA per
+// Two to 16 tokens (a decode step of as many sequences): still a weight stream, but with one fp32 FMA per
 // weight and token the kernel above was bound by instructions (4 layers of LLaVA width: 441 us a step at one
 // token, 689 at two, 732 at four), and the tiled kernel streams at half the HBM rate. Here the tokens are the
-// 8 columns of m16n8k16: a warp owns 16 of the CTA's 32 weight rows and a quarter of its K range, the
+// 8 columns of m16n8k16 (NT = 2: two sets of them): a warp owns 16 of the CTA's 32 weight rows and a quarter of its K range, the
 // weights go from 16-byte loads straight into the A operand (the order of K is free: lane (r, c) takes
 // columns 8 c .. 8 c + 7 of a 32-wide step of rows r and r + 8 and the same columns of token r), eight
 // weight loads in flight a lane. The quarters are added in a fixed order through shared memory. The same step:
 // 423 us at two tokens (1-token kernel's prefetch, a quarter of it per quarter row; 463 with four times as
-// much), 485 at eight, where the tiled kernel took 577.
-constexpr int kGemvMmaTok = 8;
+// much), 480 at eight and 585 at 16, where the tiled kernel took 577 and 662.
+constexpr int kGemvMmaTok = 16;  // 20 tokens: 787 us against 715 with the tiled kernel
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                           uint32_t b0, uint32_t b1) {
@@ -1461,11 +1455,11 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-template <int EPI>
-__global__ void __launch_bounds__(kGemvThreads, 3)
+template <int EPI, int NT>
+__global__ void __launch_bounds__(kGemvThreads, NT == 1 ? 3 : 2)
     gemv_mma_kernel(const uint16_t* __restrict__ w, const uint16_t* x, const KArgs a, int ksplit) {
-  __shared__ float red[4][32][kGemvMmaTok + 1];
-  __shared__ int trow[kGemvMmaTok], tpos[kGemvMmaTok];
+  __shared__ float red[4][32][8 * NT + 1];
+  __shared__ int trow[8 * NT], tpos[8 * NT];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
   const int grp = blockIdx.x / ksplit, ks = blockIdx.x - grp * ksplit;
   const int n0 = grp * 32;
@@ -1477,8 +1471,7 @@ __global__ void __launch_bounds__(kGemvThreads, 3)
   const bool ok0 = row + r < a.n_out, ok1 = row + r + 8 < a.n_out;
   const int4* w0 = reinterpret_cast<const int4*>(w + size_t(ok0 ? row + r : 0) * a.k + k0) + c;
   const int4* w1 = reinterpret_cast<const int4*>(w + size_t(ok1 ? row + r + 8 : 0) * a.k + k0) + c;
-  const bool okx = r < a.n_tok;
-  const int4* xp = reinterpret_cast<const int4*>(x + size_t(okx ? r : 0) * a.k + k0) + c;
+  const int4* xp = reinterpret_cast<const int4*>(x + size_t(min(r, a.n_tok - 1)) * a.k + k0) + c;
   constexpr int U = 4;  // 32-wide steps a batch
   const int steps = kn / 32;
   const int4 z = make_int4(0, 0, 0, 0);
@@ -1499,46 +1492,62 @@ __global__ void __launch_bounds__(kGemvThreads, 3)
     trow[threadIdx.x] = a.rows ? a.rows[threadIdx.x] : threadIdx.x;
     tpos[threadIdx.x] = a.pos ? a.pos[threadIdx.x] : 0;
   }
-  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  float acc[NT][4];
+#pragma unroll
+  for (int q = 0; q < NT; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.0f;
 #pragma unroll 1
   for (int st = 0; st < steps; st += U) {
     if (st > 0) load(st);
-    int4 xv[U];
+    int4 xv[U][NT];
 #pragma unroll
-    for (int u = 0; u < U; ++u) xv[u] = okx && st + u < steps ? xp[4 * (st + u)] : z;
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      mma_16816(acc, b0[u].x, b1[u].x, b0[u].y, b1[u].y, xv[u].x, xv[u].y);
-      mma_16816(acc, b0[u].z, b1[u].z, b0[u].w, b1[u].w, xv[u].z, xv[u].w);
-    }
+      for (int q = 0; q < NT; ++q)
+        xv[u][q] = r + 8 * q < a.n_tok && st + u < steps ? xp[size_t(q) * a.k + 4 * (st + u)] : z;  // 8 rows of k / 8 int4
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int q = 0; q < NT; ++q) {
+        mma_16816(acc[q], b0[u].x, b1[u].x, b0[u].y, b1[u].y, xv[u][q].x, xv[u][q].y);
+        mma_16816(acc[q], b0[u].z, b1[u].z, b0[u].w, b1[u].w, xv[u][q].z, xv[u][q].w);
+      }
   }
   const int lr = 16 * (warp >> 2) + r;
-  red[quarter][lr][2 * c] = acc[0];
-  red[quarter][lr][2 * c + 1] = acc[1];
-  red[quarter][lr + 8][2 * c] = acc[2];
-  red[quarter][lr + 8][2 * c + 1] = acc[3];
+#pragma unroll
+  for (int q = 0; q < NT; ++q) {
+    red[quarter][lr][8 * q + 2 * c] = acc[q][0];
+    red[quarter][lr][8 * q + 2 * c + 1] = acc[q][1];
+    red[quarter][lr + 8][8 * q + 2 * c] = acc[q][2];
+    red[quarter][lr + 8][8 * q + 2 * c + 1] = acc[q][3];
+  }
   __syncthreads();
-  if (warp == 0) {
+  if (warp < NT && 8 * warp < a.n_tok) {
+    const int t0 = 8 * warp;
     float v[8];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) v[t] = (red[0][lane][t] + red[1][lane][t]) + (red[2][lane][t] + red[3][lane][t]);
-    epilogue8<EPI>(a, n0 + lane, (n0 >> 5) & 3, lane, n0 >> 7, 0, v, trow, tpos, 0);
+    for (int t = 0; t < 8; ++t)
+      v[t] = (red[0][lane][t0 + t] + red[1][lane][t0 + t]) + (red[2][lane][t0 + t] + red[3][lane][t0 + t]);
+    epilogue8<EPI>(a, n0 + lane, (n0 >> 5) & 3, lane, n0 >> 7, t0, v, trow, tpos, 0);
     if (lane == 0) stamp_end(a.stamp);
   }
 }
 
 using GemvFn = void (*)(const uint16_t*, const uint16_t*, KArgs, int);
+template <int NT>
 GemvFn gemv_mma_for(int epi) {
   switch (epi) {
-    case EPI_F32: return gemv_mma_kernel<EPI_F32>;
-    case EPI_BF16: return gemv_mma_kernel<EPI_BF16>;
-    case EPI_BIAS_BF16: return gemv_mma_kernel<EPI_BIAS_BF16>;
-    case EPI_BIAS_GELU_BF16: return gemv_mma_kernel<EPI_BIAS_GELU_BF16>;
-    case EPI_ADD_F32: return gemv_mma_kernel<EPI_ADD_F32>;
-    case EPI_SWIGLU_BF16: return gemv_mma_kernel<EPI_SWIGLU_BF16>;
-    case EPI_QKV_BF16: return gemv_mma_kernel<EPI_QKV_BF16>;
+    case EPI_F32: return gemv_mma_kernel<EPI_F32, NT>;
+    case EPI_BF16: return gemv_mma_kernel<EPI_BF16, NT>;
+    case EPI_BIAS_BF16: return gemv_mma_kernel<EPI_BIAS_BF16, NT>;
+    case EPI_BIAS_GELU_BF16: return gemv_mma_kernel<EPI_BIAS_GELU_BF16, NT>;
+    case EPI_ADD_F32: return gemv_mma_kernel<EPI_ADD_F32, NT>;
+    case EPI_SWIGLU_BF16: return gemv_mma_kernel<EPI_SWIGLU_BF16, NT>;
+    case EPI_QKV_BF16: return gemv_mma_kernel<EPI_QKV_BF16, NT>;
     default: return nullptr;
   }
+}
+GemvFn gemv_mma_for(int epi, int n_tok) {
+  return n_tok <= 8 ? gemv_mma_for<1>(epi) : gemv_mma_for<2>(epi);
 }
 template <int CPR>
 GemvFn gemv_for(int epi) {
@@ -1661,7 +1670,7 @@ bool vec_red_ok(const GemmProblem& p) {
          (reinterpret_cast<uintptr_t>(p.out) & 15) == 0;
 }
 
-// One token: gemv_kernel (which can norm its input); up to eight: gemv_mma_kernel
+// One token: gemv_kernel (which can norm its input); up to 16: gemv_mma_kernel
 bool gemv_aligned(const GemmProblem& p) {
   return p.w && p.k % kGemvChunk == 0 && ((reinterpret_cast<uintptr_t>(p.w) | reinterpret_cast<uintptr_t>(p.x)) & 15) == 0;
 }
@@ -1671,7 +1680,7 @@ bool gemv_eligible(const GemmProblem& p) {
   return p.n_tok == 1 && gemv_aligned(p) && gemv_for<4>(p.epi) != nullptr;
 }
 bool gemv_mma_eligible(const GemmProblem& p) {
-  return p.n_tok >= 1 && p.n_tok <= kGemvMmaTok && gemv_aligned(p) && !p.norm_h && gemv_mma_for(p.epi) != nullptr;
+  return p.n_tok >= 1 && p.n_tok <= kGemvMmaTok && gemv_aligned(p) && !p.norm_h && gemv_mma_for(p.epi, p.n_tok) != nullptr;
 }
 
 int gemv_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
@@ -1708,7 +1717,7 @@ int gemv_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
     while (groups * ksplit < num_sms() && ksplit * 2 <= C && ksplit < 8) ksplit *= 2;
   if (!gemv_eligible(p)) {
     const int slot = trace_begin(stream);
-    SPD_CUDA_TRY(launch_pdl(gemv_mma_for(p.epi), dim3(groups * ksplit), dim3(kGemvThreads), 0, stream,
+    SPD_CUDA_TRY(launch_pdl(gemv_mma_for(p.epi, p.n_tok), dim3(groups * ksplit), dim3(kGemvThreads), 0, stream,
                             static_cast<const uint16_t*>(p.w), static_cast<const uint16_t*>(p.x), a, ksplit));
     trace_gemm(slot, p, stream);
     return SPD_OK;
@@ -1770,6 +1779,9 @@ int gemm_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
   // 256-row tiles in one CTA for token tiles of at most 64: their stages are mostly weights, and
   // two MMAs per token box double the weight bytes per stage (needs the row-major pointer)
   a.nh = (!pair && a.tt <= 64 && p.w) ? 2 : 1;
+  // ... but 128-row tiles where those leave at most half of the SMs a tile: the cluster split of K then fills
+  // them, with twice the CTAs (32 tokens, 4608 x 3584: 72 -> 144 CTAs; a decode step of four layers 807 -> 779 us)
+  if (a.nh == 2 && p.epi != EPI_ADD_F32 && (p.n_out + kBM - 1) / kBM * 2 <= sms) a.nh = 1;
   const int tile_rows = pair ? 2 * kBM : a.nh * kBM;  // weight rows per work item
   const int cta_rows = pair ? kBM : tile_rows;          // ... per CTA
   const int wbox = (pair ? 1 : a.nh) * kHalfW;
@@ -1810,16 +1822,16 @@ int gemm_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
   a.units = int(units);
   const int work_slots = pair ? slots : sms;  // work items the GPU holds at once
   // split-K when the tiles fill at most half the work slots. ADD epilogues: the most work items
-  // per tile (a power of two, at least two k-blocks each) that still fit. Others (single CTA):
+  // per tile (at least two k-blocks each) that still fit (powers of two alone left a quarter of the SMs idle:
+  // 14 tiles x 8 CTAs; a decode step of 32 sequences and four layers 829 -> 807 us). Others (single CTA):
   // the largest C in {2, 4, 8} with at least one k-block per CTA whose clusters all fit on the
   // GPU at once.
   a.csplit = 1;
   a.cluster = 0;
   a.determ = deterministic();
   if (tiles * 2 <= work_slots && p.epi == EPI_ADD_F32 && !a.determ) {
-    int C = 2;
-    while (tiles * C * 2 <= work_slots && C * 4 <= a.n_kb) C *= 2;
-    if (C * 2 <= a.n_kb) a.csplit = C;
+    const int C = int(std::min<long long>(work_slots / tiles, a.n_kb / 2));
+    if (C >= 2) a.csplit = C;
   } else if (!pair && tiles * 2 <= sms) {
     for (int C = 8; C >= 2; C /= 2) {
       // the ring receives C copies of each CTA's share of 32-column chunks ([128][36] fp32 each)
@@ -1864,13 +1876,30 @@ int gemm_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
     grid = tiles * a.csplit;
   } else if (a.dpr) {
     // grid set above
-  } else if (tiles <= work_slots && tiles * 2 > work_slots && a.tt >= 128) {
+  } else if (tiles <= work_slots && tiles * 2 > work_slots && a.tt >= 128 && 
+             (p.epi != EPI_ADD_F32 || a.determ || tiles * 4 > work_slots * 3)) {
     // between half and all of the work slots' worth of wide tiles: one whole tile per work item.
     // Stream-K's balance would split most tiles two or three ways, and the fixups of wide token
-    // tiles cost more than the idle SMs do.
+    // tiles cost more than the idle SMs do. Residual tiles need no fixup (each part adds itself), so they take
+    // it up to three quarters: 640 tokens (48 tiles for 76 pairs), two layers 647 -> 627 us; 1000 tokens (64
+    // tiles) 795 -> 817 with it.
     grid = tiles;
   }
   a.grid = int(grid);
+  // tile counters: the schedules with fixups (stream-K, which residual tiles run without, and dpr)
+  if (s.cleared) {
+    const bool adds = p.epi == EPI_ADD_F32 && !a.determ;
+    const bool whole_tiles = !a.dpr && a.grid == tiles;
+    auto clear = [&](auto* buf, size_t need, size_t* done) {
+      const size_t from = *done;
+      if (need <= from) return cudaSuccess;
+      *done = need;
+      return cudaMemsetAsync(buf + from, 0, (need - from) * sizeof(*buf), stream);
+    };
+    if (a.csplit == 1 && !adds && !whole_tiles)
+      SPD_CUDA_TRY(clear(s.counters, size_t(a.dpr ? a.rem_tiles : tiles) * (pair ? 2 : 1), &s.cleared->counters));
+    if (a.dpr) SPD_CUDA_TRY(clear(s.acc, size_t(a.rem_tiles) * tile_rows * a.tt, &s.cleared->acc));
+  }
   const KernelFn kern = kernel_for(p.epi, pair, a.determ);
   a.out = p.out;
   a.ldo = p.ldo;

@@ -136,6 +136,9 @@ constexpr size_t kGemmSlotFloats = size_t(10) << 20;
 // Accumulation buffers of the data-parallel + remainder schedule: zero when a GEMM starts, left
 // zero by every GEMM.
 constexpr size_t kGemmAccFloats = size_t(4) << 20;
+struct GemmCleared {
+  size_t counters = 0, acc = 0;  // the first ints / floats
+};
 struct GemmScratch {
   float* partial;     // stream-K partial slots
   size_t partial_floats;
@@ -144,10 +147,12 @@ struct GemmScratch {
   int* counters;
   int n_counters;
   int* status;
+  // What one entry-point call has cleared so far (null: the scratch is clear): a GEMM of the call whose schedule
+  // uses the counters or the accumulation buffers clears what it needs of them on its stream, unless an
+  // earlier one did (every GEMM leaves them zero). Most calls on few tokens use neither, and the 16 MB of
+  // buffers take about 5 us to clear.
+  GemmCleared* cleared;
 };
-// Clears the tile counters and the accumulation buffers of a workspace scratch on `stream` (done
-// once per entry-point call, before its first GEMM).
-int gemm_scratch_clear(const GemmScratch& s, cudaStream_t stream);
 // Deterministic mode (process-wide): GEMMs sum every output element in a fixed order (split tiles
 // through per-CTA partial slots summed in CTA order, residual updates as one read-modify-write per
 // element) instead of fire-and-forget L2 reductions; repeated runs are then bit-identical.

@@ -70,7 +70,7 @@ def test_decode_attention_edges(heads, kv_heads, head_dim, pos, offset):
 
 
 # ---- few-token GEMMs: m16n8k16 straight from the weight rows ------------------------------------------
-@pytest.mark.parametrize("M", [1, 2, 7, 8, 9])  # 9: past the form's token columns
+@pytest.mark.parametrize("M", [1, 2, 7, 8, 9, 16, 17])  # one and two sets of token columns, and past them
 @pytest.mark.parametrize("K,n", [(256, 1), (512, 40), (2816, 1000), (4096, 128)])
 def test_few_token_epilogues(M, K, n):
     # K ranges of one chunk, of unequal shares; output widths that end inside a 16-row half, a 32-row group
