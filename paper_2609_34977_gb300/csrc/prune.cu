@@ -2282,7 +2282,10 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
 namespace {
 int received_splits(int n_maps, int n_q, int n_k) {
   const int blocks = (n_k / 4 + 255) / 256;
-  int sp = (2 * num_sms() + blocks * n_maps - 1) / (blocks * n_maps);  // about two CTAs per SM
+  // About four CTAs an SM (32 KB of loads in flight each): with two, 2.1 a SM at 16 maps of 3840 x 3840 left
+  // half of the SMs at two thirds of the others' share, 183 us against 138 (6.8 TB/s); eight were slower at
+  // 32 maps of 4096 x 4096 (350 us, 303 at four).
+  int sp = (4 * num_sms() + blocks * n_maps - 1) / (blocks * n_maps);
   sp = std::max(1, std::min(sp, (n_q + 63) / 64));                    // at least 64 rows each
   return sp;
 }
