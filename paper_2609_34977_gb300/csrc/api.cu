@@ -904,7 +904,7 @@ extern "C" int spd_prefill_adaptive(const spd_model* m, const uint16_t* x, int T
   const bool no_slc = pol->ablate & SPD_SKIP_NO_SLC;
   const int mode = ((pol->w1 != 0.0f && !(pol->ablate & SPD_SKIP_NO_ENTROPY)) ? kSkipEntropy : 0) |
                    ((pol->w1 != 0.0f && !(pol->ablate & SPD_SKIP_NO_ITC)) ? kSkipItc : 0) |
-                   ((pol->ablate & SPD_SKIP_NO_ACCUM) ? 0 : kSkipAccumulate) | kSkipLse;
+                   ((pol->ablate & SPD_SKIP_NO_ACCUM) ? 0 : kSkipAccumulate);
   Carve cv(ws, ws_bytes);
   PrefillBufs bf = carve_prefill(c, T, B, cv);
   AdaptiveBufs ab = carve_adaptive(c, T, B, cv);

@@ -126,18 +126,50 @@ __global__ void scatter_rows_kernel(const uint16_t* src, int D, const int32_t* r
 }
 
 // q_t of sequence b (ASL-Skip's text context, Sec. 4.2.1): the mean of h over the text tokens
-// text[ts[b] .. ts[b+1]), one thread per column, tokens in order (zero when there are none).
+// text[ts[b] .. ts[b+1]) (zero when there are none). A CTA takes 128 columns (four a lane), its warps every
+// eighth token each, eight rows in flight, and adds the warps' sums in order: the kernel is a chain of
+// dependent loads, 10 us for 64 tokens with one thread a column walking them all, 5.1 so.
+constexpr int kMeanCols = 128;
 __global__ void __launch_bounds__(kThreads) text_mean_kernel(const float* h, int D, const int32_t* ts,
                                                              const int32_t* text,
                                                              float* __restrict__ tmean) {
   pdl_launch_dependents();
   pdl_wait();
-  const int c = blockIdx.x * kThreads + threadIdx.x, b = blockIdx.y;
-  if (c >= D) return;
+  __shared__ float4 part[kThreads / 32][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, b = blockIdx.y;
+  constexpr int NW = kThreads / 32;
+  const int c = blockIdx.x * kMeanCols + 4 * lane;  // D is a multiple of 8: a group of four is in or out
   const int t0 = ts[b], t1 = ts[b + 1];
-  float s = 0.0f;
-  for (int e = t0; e < t1; ++e) s += h[size_t(text[e]) * D + c];
-  tmean[size_t(b) * D + c] = t1 > t0 ? s / float(t1 - t0) : 0.0f;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int e = t0 + warp; e < t1; e += 8 * NW) {
+    float4 x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      x[u] = e + u * NW < t1 && c < D ? *reinterpret_cast<const float4*>(h + size_t(text[e + u * NW]) * D + c)
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      s.x += x[u].x;
+      s.y += x[u].y;
+      s.z += x[u].z;
+      s.w += x[u].w;
+    }
+  }
+  part[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && c < D) {
+    float4 t = part[0][lane];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) {
+      t.x += part[w][lane].x;
+      t.y += part[w][lane].y;
+      t.z += part[w][lane].z;
+      t.w += part[w][lane].w;
+    }
+    const float n = float(t1 - t0);
+    *reinterpret_cast<float4*>(tmean + size_t(b) * D + c) =
+        t1 > t0 ? make_float4(t.x / n, t.y / n, t.z / n, t.w / n) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
 }
 
 __device__ __forceinline__ float block_max(float v, float* red) {
@@ -154,10 +186,10 @@ __device__ __forceinline__ float block_max(float v, float* red) {
 }
 
 // One candidate visual token per CTA (Sec. 4.2.1 and Eq. 6): E_ii = entropy of softmax(logits
-// row) / log V, F_itc = (cos(h_i, q_t) + 1) / 2 (0.5 without text), S_sa = ReLU(1 - E - F);
+// row) / log V from the statistics of EPI_LSE_F32, F_itc = (cos(h_i, q_t) + 1) / 2 (0.5 without text), S_sa = ReLU(1 - E - F);
 // s_skip[i] += w1 S_sa + w2 SLC^Norm(l), flag[n] = s_skip[i] >= T_skip.
 __global__ void __launch_bounds__(kThreads)
-    skip_score_kernel(const float* logits, int V, const float* h, int D, const int32_t* cand,
+    skip_score_kernel(const float* lse, int V, const float* h, int D, const int32_t* cand,
                       const int32_t* ts, const int32_t* seq_of, const float* tmean, float inv_log_v,
                       float w1, float add_slc, float t_skip, int mode, float* s_skip, uint8_t* flag,
                       int32_t* admit, uint8_t* target, int layer, int tgt) {
@@ -166,66 +198,60 @@ __global__ void __launch_bounds__(kThreads)
   pdl_wait();
   const int n = blockIdx.x, i = cand[n], b = seq_of[i];
   if ((mode & kSkipDevice) && admit[i] >= 0) return;  // already in skip mode (block-uniform)
-  float ent = 0.0f;
-  if ((mode & kSkipEntropy) && (mode & kSkipLse)) {
+  // every sum of the score in one block reduction, behind the maximum's: the kernel is a chain of loads and
+  // barriers (six reductions in a row: 10.3 us for 192 candidates of 1000 groups and 4096 columns, 8.5 so)
+  float sums[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};  // e^(m - max) terms s and u of the entropy; h.q, h.h, q.q
+  if (mode & kSkipItc) {
+    const float4* h4 = reinterpret_cast<const float4*>(h + size_t(i) * D);
+    const float4* q4 = reinterpret_cast<const float4*>(tmean + size_t(b) * D);
+#pragma unroll 4
+    for (int c = threadIdx.x; c < D / 4; c += kThreads) {
+      const float4 x = h4[c], q = q4[c];
+      sums[2] += x.x * q.x + x.y * q.y + x.z * q.z + x.w * q.w;
+      sums[3] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+      sums[4] += q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w;
+    }
+  }
+  if (mode & kSkipEntropy) {
     // merge of the per-32-word statistics (m_g, s_g, u_g): with m = max m_g,
     // S = sum_g e^(m_g - m) s_g and U = sum_g e^(m_g - m) (u_g + (m_g - m) s_g), H = log S - U / S
     const int G = lse_groups(V);
-    const float4* st = reinterpret_cast<const float4*>(logits) + size_t(n) * G;
+    const float4* st = reinterpret_cast<const float4*>(lse) + size_t(n) * G;
     float mx = -INFINITY;
+#pragma unroll 4
     for (int g = threadIdx.x; g < G; g += kThreads) mx = fmaxf(mx, st[g].x);
     mx = block_max(mx, red);
-    float se = 0.0f, te = 0.0f;
+#pragma unroll 4
     for (int g = threadIdx.x; g < G; g += kThreads) {
       const float4 q = st[g];
       if (q.y > 0.0f) {
         const float dm = q.x - mx, f = expf(dm);
-        se += f * q.y;
-        te += f * (q.z + dm * q.y);
+        sums[0] += f * q.y;
+        sums[1] += f * (q.z + dm * q.y);
       }
     }
-    __syncthreads();
-    se = block_sum(se, red);
-    __syncthreads();
-    te = block_sum(te, red);
-    ent = (logf(se) - te / se) * inv_log_v;
-  } else if (mode & kSkipEntropy) {
-    const float* z = logits + size_t(n) * V;
-    float mx = -INFINITY;
-    for (int v = threadIdx.x; v < V; v += kThreads) mx = fmaxf(mx, z[v]);
-    mx = block_max(mx, red);
-    float se = 0.0f, te = 0.0f;  // sum e^(z - m) and sum e^(z - m) (z - m)
-    for (int v = threadIdx.x; v < V; v += kThreads) {
-      const float d = z[v] - mx, e = expf(d);
-      se += e;
-      te += e * d;
-    }
-    __syncthreads();
-    se = block_sum(se, red);
-    __syncthreads();
-    te = block_sum(te, red);
-    ent = (logf(se) - te / se) * inv_log_v;
   }
-  const float* hi = h + size_t(i) * D;
-  const float* q = tmean + size_t(b) * D;
+  __shared__ float all[5][kThreads / 32];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+#pragma unroll
+    for (int off = 16; off; off >>= 1) sums[k] += __shfl_xor_sync(0xffffffffu, sums[k], off);
+    if ((threadIdx.x & 31) == 0) all[k][threadIdx.x >> 5] = sums[k];
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    sums[k] = 0.0f;
+    for (int w = 0; w < kThreads / 32; ++w) sums[k] += all[k][w];
+  }
+  const float ent = (mode & kSkipEntropy) ? (logf(sums[0]) - sums[1] / sums[0]) * inv_log_v : 0.0f;
   float f = 0.0f;
   if (mode & kSkipItc) {
-    float dot = 0.0f, hh = 0.0f, qq = 0.0f;
-    for (int c = threadIdx.x; c < D; c += kThreads) {
-      dot += hi[c] * q[c];
-      hh += hi[c] * hi[c];
-      qq += q[c] * q[c];
-    }
-    __syncthreads();
-    dot = block_sum(dot, red);
-    __syncthreads();
-    hh = block_sum(hh, red);
-    __syncthreads();
-    qq = block_sum(qq, red);
-    const bool has_text = ts[b + 1] > ts[b] && hh > 0.0f && qq > 0.0f;
-    f = has_text ? 0.5f + 0.5f * dot / (sqrtf(hh) * sqrtf(qq)) : 0.5f;
+    const bool has_text = ts[b + 1] > ts[b] && sums[3] > 0.0f && sums[4] > 0.0f;
+    f = has_text ? 0.5f + 0.5f * sums[2] / (sqrtf(sums[3]) * sqrtf(sums[4])) : 0.5f;
   }
-  if (threadIdx.x == 0) {
+  {
     const float s_sa = fmaxf(0.0f, 1.0f - ent - f);
     const float fuse = w1 * s_sa + add_slc;
     const float acc = (mode & kSkipAccumulate) ? s_skip[i] + fuse : fuse;
@@ -341,15 +367,15 @@ __global__ void __launch_bounds__(1024)
 
 }  // namespace
 
-int skip_scores_run(const float* logits, int V, int n_cand, const float* h, int D, const int32_t* cand,
+int skip_scores_run(const float* lse, int V, int n_cand, const float* h, int D, const int32_t* cand,
                     const int32_t* ts, const int32_t* text, const int32_t* seq_of, int B, float* tmean,
                     float w1, float add_slc, float t_skip, int mode, float* s_skip, uint8_t* flag,
                     cudaStream_t stream, int32_t* admit, uint8_t* target, int layer, int tgt) {
   if (mode & kSkipItc)
-    SPD_CUDA_TRY(launch_pdl(text_mean_kernel, dim3((D + kThreads - 1) / kThreads, B), dim3(kThreads),
+    SPD_CUDA_TRY(launch_pdl(text_mean_kernel, dim3((D + kMeanCols - 1) / kMeanCols, B), dim3(kThreads),
                             0, stream, h, D, ts, text, tmean));
   SPD_CUDA_TRY(launch_pdl(skip_score_kernel, dim3(n_cand), dim3(kThreads), 0, stream,
-                          logits, V, h, D, cand, ts, seq_of, static_cast<const float*>(tmean),
+                          lse, V, h, D, cand, ts, seq_of, static_cast<const float*>(tmean),
                           float(1.0 / log(double(V))), w1, add_slc, t_skip, mode, s_skip, flag,
                           admit, target, layer, tgt));
   return SPD_OK;
