@@ -137,6 +137,22 @@ __device__ __forceinline__ void quad_transpose8(const float (&v)[8], float (&w)[
   }
 }
 
+// Reduces eight values over the 32 lanes; lanes 4 j .. 4 j + 3 receive value j's result in x[0].
+template <typename Op>
+__device__ __forceinline__ void reduce8(float (&x)[8], int lane, Op op) {
+#pragma unroll
+  for (int h = 4, off = 16; h >= 1; h >>= 1, off >>= 1) {
+    const bool up = lane & off;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const float recv = __shfl_xor_sync(0xffffffffu, up ? x[i] : x[i + h], off);
+      x[i] = op(up ? x[i + h] : x[i], recv);
+    }
+  }
+  x[0] = op(x[0], __shfl_xor_sync(0xffffffffu, x[0], 2));
+  x[0] = op(x[0], __shfl_xor_sync(0xffffffffu, x[0], 1));
+}
+
 __device__ __forceinline__ float gelu_erf(float x) {
   return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f));
 }
@@ -473,33 +489,27 @@ __device__ __forceinline__ void epilogue8(const KArgs& a, int n, int q, int lane
     }
   } else if constexpr (EPI == EPI_LSE_F32) {
     // the statistics of this warp's 32 weight rows (vocabulary words) for each of the 8 tokens:
-    // warp max, then the sums of e^(z - m) and e^(z - m) (z - m); lane j stores token t0 + j's
-    float m8[8], s8[8], u8[8];
+    // warp max, then the sums of e^(z - m) and e^(z - m) (z - m); lane 4 j stores token t0 + j's. Each
+    // reduction over the 32 lanes halves the tokens a lane still carries: 35 exchanges in all for the 8
+    // tokens, where a butterfly each took 120 and held the epilogue back; the pairs added are the same.
     const bool live = n < a.n_out;
+    float m8[8], s8[8], u8[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) m8[j] = live ? v[j] : -INFINITY;
+    reduce8(m8, lane, [](float x, float y) { return fmaxf(x, y); });
+    const float m = m8[0];  // of token t0 + lane / 4
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      float m = live ? v[j] : -INFINITY;
-#pragma unroll
-      for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-      const float d = live ? v[j] - m : 0.0f;
-      const float e = live ? __expf(d) : 0.0f;
-      float sj = e, uj = e * d;
-#pragma unroll
-      for (int off = 16; off; off >>= 1) {
-        sj += __shfl_xor_sync(0xffffffffu, sj, off);
-        uj += __shfl_xor_sync(0xffffffffu, uj, off);
-      }
-      m8[j] = m;
-      s8[j] = sj;
-      u8[j] = uj;
+      const float mj = __shfl_sync(0xffffffffu, m, 4 * j);
+      const float d = live ? v[j] - mj : 0.0f;
+      s8[j] = live ? __expf(d) : 0.0f;
+      u8[j] = s8[j] * d;
     }
-    float4* o = static_cast<float4*>(a.out);
-    const int g = n >> 5;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int t = t0 + j;
-      if (lane == j && t < nt) o[size_t(t) * a.ldo + g] = make_float4(m8[j], s8[j], u8[j], 0.0f);
-    }
+    reduce8(s8, lane, [](float x, float y) { return x + y; });
+    reduce8(u8, lane, [](float x, float y) { return x + y; });
+    const int t = t0 + (lane >> 2);
+    if ((lane & 3) == 0 && t < nt)
+      static_cast<float4*>(a.out)[size_t(t) * a.ldo + (n >> 5)] = make_float4(m, s8[0], u8[0], 0.0f);
   } else if constexpr (EPI == EPI_SWIGLU_BF16) {
     // lanes l and l + 16 hold gate and up of the same FFN channel f: after one exchange lane l
     // finishes the even tokens of the group and lane l + 16 the odd ones
