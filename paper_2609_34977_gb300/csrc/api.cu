@@ -580,6 +580,7 @@ struct HostPlan {
   std::vector<LayerLists> ll;
   size_t pos_off = 0, kvrow_off = 0, last_off = 0, end = 0;
   bool decode = false;  // one query per sequence at its last position (attention_decode_run)
+  std::vector<int> by_length;  // decode: the sequences, longest first
 };
 
 // Token t of sequence b = seq_of at position pos_all; its K/V row is kvrow (cache modes) or t.
@@ -640,6 +641,16 @@ void plan_layer(HostPlan& P, int l, const uint8_t* mk, const int32_t* cu, int B,
       hl[q.amap + t] = -1;
     }
     if (!(bits & 2)) hl[q.frows + q.nf++] = t;
+  }
+  if (P.decode) {  // one query a sequence, the longest first: its CTAs are the launch's last otherwise
+    for (int b : P.by_length) {
+      int32_t* tl = &hl[q.tiles + 4 * size_t(q.ntiles++)];
+      tl[0] = b;
+      tl[1] = 1;
+      tl[2] = P.kv0[b];
+      tl[3] = P.kvlen[b];
+    }
+    return;
   }
   // attention tiles: up to kAttnTileQ active queries of one sequence each
   int a = 0;
@@ -1120,6 +1131,9 @@ extern "C" int spd_decode(const spd_model* m, const uint16_t* x, int B, const in
   static thread_local HostPlan P;
   plan_init(P, c, cu.data(), B, B, bf.list_ints, pos, max_len);
   P.decode = true;
+  P.by_length.resize(B);
+  for (int b = 0; b < B; ++b) P.by_length[b] = b;
+  std::stable_sort(P.by_length.begin(), P.by_length.end(), [&](int x, int y) { return P.kvlen[x] > P.kvlen[y]; });
   for (int l = 0; l < c.n_layers; ++l) plan_layer(P, l, nullptr, cu.data(), B, B);
   int32_t* dl = bf.lists;
   SPD_CUDA_TRY(cudaMemcpyAsync(dl, P.hl.data(), P.end * sizeof(int32_t), cudaMemcpyHostToDevice, st));

@@ -393,9 +393,11 @@ __global__ void __launch_bounds__(kDecWarps * 32, 1)
   pdl_wait();
   if (threadIdx.x == 0) stamp_start(stamp);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
-  const int G = n_heads / n_kv_heads, g = blockIdx.y / chunks, hc = (blockIdx.y - g * chunks) * kDecHeads;
+  // all heads of a sequence side by side, the sequences in the list's order
+  const int groups = n_kv_heads * chunks, seq = blockIdx.x / groups, grp = blockIdx.x - seq * groups;
+  const int G = n_heads / n_kv_heads, g = grp / chunks, hc = (grp - g * chunks) * kDecHeads;
   const int h0 = g * G + hc, ng = min(kDecHeads, G - hc);
-  const int4 tl = tiles[blockIdx.x];  // (query row, query count = 1, first key row, key count)
+  const int4 tl = tiles[seq];  // (query row, query count = 1, first key row, key count)
   const int j_lo = int((long long)rank * tl.w / S), j_hi = int((long long)(rank + 1) * tl.w / S);
   const __nv_bfloat16* kbase = kv + size_t(tl.z) * ldkv + g * HD;
   uint4 qf[KB];
@@ -607,7 +609,7 @@ int attention_decode_run(const void* q, const void* kv, int ldkv, int v_off, voi
   int S = 1;
   while (S < kDecMaxSplit && groups * 2 * S <= 2LL * num_sms() && ctx_sum >= 128.0 * S * n_tiles) S *= 2;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n_tiles, n_kv_heads * chunks, S);
+  cfg.gridDim = dim3(n_tiles * n_kv_heads * chunks, 1, S);
   cfg.blockDim = dim3(kDecWarps * 32);
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
