@@ -27,6 +27,8 @@
 
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "internal.h"
 #include "ptx.cuh"
 #include "trace.h"
@@ -340,11 +342,11 @@ int launch(const CUtensorMap& mq, const CUtensorMap& mkv, void* o, int ldo, cons
 // eight warps takes groups of 16 keys, 16 bytes a lane and load, and multiplies them with the legacy
 // m16n8k16 tensor instruction straight from registers (at most 8 of a tile's 128 rows would be
 // queries on the tcgen05 path, which would also have to stage K and V in shared memory).
-// Eight warps of 184 registers, one CTA an SM, were faster than four CTAs of four warps (a whole step of
+// For few CTAs, eight warps of 184 registers, one CTA an SM, were faster than four CTAs of four warps (a whole step of
 // 32 sequences 829 against 828 us, of one sequence 3142 against 3167) or 128 registers a thread (3199).
 // One layer's attention of 32 sequences (28 query heads on 4 K/V heads of 128, 1122 keys on average,
-// 73 MB, serialised): 143 us with one warp a key and one CTA a query head, 35.5 us here; the step of four
-// layers 1256 -> 829 us. One sequence of 257 keys, 32 heads: 10.4 -> 7.2 us.
+// 73 MB, serialised): 143 us with one warp a key and one CTA a query head, 35.5 us here and 29 with the
+// longest sequences first; the step of four layers 1256 -> 829 us. One sequence of 257 keys, 32 heads: 10.4 -> 7.2 us.
 //  * S = Q K^T: heads are the 16 rows of A (rows 8..15 stay zero), keys the 8 columns of B. The
 //    order of the contraction index is free, so lane (r = lane / 4, c = lane % 4) feeds the two
 //    MMAs of a 32-dim block from one 16-byte load of key r, dims 8 c .. 8 c + 7, of K and of Q alike.
@@ -378,8 +380,8 @@ __device__ __forceinline__ uint4 load8(const __nv_bfloat16* p) {
   }
 }
 
-template <int HD, bool A16>
-__global__ void __launch_bounds__(kDecWarps * 32, 1)
+template <int HD, bool A16, int MINB>
+__global__ void __launch_bounds__(kDecWarps * 32, MINB)
     attn_decode_kernel(const __nv_bfloat16* q, const __nv_bfloat16* kv, int ldkv, int v_off,
                        __nv_bfloat16* __restrict__ o, int ldo, const int4* tiles, int n_heads,
                        int n_kv_heads, int chunks, float scale_log2, unsigned long long* stamp) {
@@ -622,8 +624,16 @@ int attention_decode_run(const void* q, const void* kv, int ldkv, int v_off, voi
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   const bool a16 = (reinterpret_cast<uintptr_t>(kv) & 15) == 0 && (ldkv | v_off) % 8 == 0;
-  auto kern = head_dim == 128 ? (a16 ? attn_decode_kernel<128, true> : attn_decode_kernel<128, false>)
-                              : (a16 ? attn_decode_kernel<64, true> : attn_decode_kernel<64, false>);
+  // Two CTAs an SM (128 registers, a few spilled) where there are more than that of them: 16 / 64 sequences of 500
+  // keys, 32 K/V heads, four layers 582 / 1114 -> 557 / 1021 us a step; but 256 CTAs of seven heads each (32
+  // sequences) 755 -> 781, one sequence and 32 layers 2829 -> 2887.
+  const bool two = groups * S > 2LL * num_sms();
+  auto pick = [&](auto minb) {
+    constexpr int M = decltype(minb)::value;
+    return head_dim == 128 ? (a16 ? attn_decode_kernel<128, true, M> : attn_decode_kernel<128, false, M>)
+                           : (a16 ? attn_decode_kernel<64, true, M> : attn_decode_kernel<64, false, M>);
+  };
+  auto kern = two ? pick(std::integral_constant<int, 2>()) : pick(std::integral_constant<int, 1>());
   SPD_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, qb, kb, ldkv, v_off, ob, ldo, tiles, n_heads, n_kv_heads, chunks,
                                   scale_log2, stamp));
   trace_end(slot, stream, TR_ATTN, fl, by);

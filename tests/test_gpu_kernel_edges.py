@@ -25,6 +25,7 @@ def _bf16(seed, *shape):
     (28, 4, 128, [65, 127, 128, 129, 500, 7], 0),   # seven heads a K/V head, shares of unequal length
     (18, 2, 64, [31, 260, 511], 0),                 # nine heads a K/V head: a second chunk of one head
     (16, 1, 128, [0, 1, 300, 511, 48, 47, 33, 2], 0),  # two full chunks; clusters of eight CTAs
+    (32, 32, 64, list(range(0, 500, 50)), 0),          # more CTAs than two an SM hold
 ])
 def test_decode_attention_edges(heads, kv_heads, head_dim, pos, offset):
     # one decoder layer over a given cache: logits and the appended K/V rows. Tolerance: every rounding of
