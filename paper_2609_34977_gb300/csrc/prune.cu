@@ -3,20 +3,20 @@
 //   rowstats     a_v = head-mean of the attention (Sec. 4.1.1); 1/||F_l,i|| for every tapped layer
 //                (and ||F_l,i||^2, or the log-sum-exp and negentropy of softmax(F_l,i), for the
 //                MSE and KL ablations of sim)
-//   anchors      top-N_anc of a_v by ranking (a_v desc, index asc) keys (Eq. 1); stable lists of
-//                anchor and non-anchor tokens by block prefix sums
+//   anchors      top-N_anc of a_v by rank counting of (a_v desc, index asc) keys (Eq. 1), over several
+//                CTAs for a long tile; stable lists of anchor and non-anchor tokens by one block scan
 //   anchor_sim   a_i = max_p cos(F^L_i, F^L_p) over anchors: 128 x 64 (or 48) register-tiled fp32 products,
 //                the feature dimension split over a cluster of 4 or 8 CTAs whose partial tiles are summed
 //                in rank order through distributed shared memory; max via atomicMax on
 //                order-preserving integer keys (exact, order independent)
-//   kmeans       one thread-block cluster of 16 CTAs per tile, each owning a contiguous slice of the
-//                non-anchor tokens whose F^L rows it keeps in shared memory for every iteration (8
-//                CTAs re-reading them from L2 where they do not fit, 4 beyond one wave of such
-//                clusters): Lloyd on raw F^L (assignment
-//                in each CTA, per-CTA sums in token order, cross-CTA sums in rank order through
-//                distributed shared memory), then the
-//                per-cluster, per-layer sums of unit feature rows, the sums of a_j, sizes and Eq. 2
-//                quotas
+//   kmeans       Lloyd on raw F^L of the non-anchor tokens, then the per-cluster, per-layer sums of unit
+//                feature rows, the sums of a_j, sizes and Eq. 2 quotas. One thread-block cluster of
+//                16 CTAs per tile, each with its slice of the rows in shared memory for every
+//                iteration, where they fit and all tiles run at once (kmeans_kernel); the whole GPU,
+//                launched cooperatively, for a few larger tiles (kmeans_grid_kernel); one sweep over
+//                the rows an iteration for many tiles (kmeans_stream_kernel); clusters of 8 CTAs that
+//                re-read the rows from L2 for the shapes none of these takes. Sums across CTAs run in
+//                a fixed order
 //   scores       s_i = [sum_l w_l f_i . (S_l,k - f_i)] / (|C_k| - 1) + a_i + (A_k - a_i) / (|C_k| - 1),
 //                the per-token mean of Eq. 3's S_ij over the other members of its cluster (for
 //                the MSE and KL ablations the same cluster-sum identity with raw rows, plus the
@@ -2114,9 +2114,8 @@ PrunePlan prune_plan(const PruneDims& p) {
   const size_t cent_bytes = size_t(2) * p.K * p.d * sizeof(float);
   const size_t res_bytes = size_t((p.m + 15) / 16) * p.d * sizeof(float) + cent_bytes;
   // K-means: the rows resident in shared memory over 16 CTAs per tile where they fit and all tiles
-  // run in one wave of such clusters (latency); else re-read from L2 each pass by 8 CTAs per tile,
-  // twice as many tiles at once (throughput), or by 4 where 8-CTA clusters would take more than one
-  // wave at two CTAs an SM (the paper's K = 4)
+  // run in one wave of such clusters (latency); else the whole GPU or the one-sweep form below; else
+  // (K other than 4, or rows too wide for the one-sweep ring) re-read from L2 each pass by 8 CTAs
   q.res = p.m > 0 && res_bytes <= kResSmem && g_res_clusters > 0 && p.n_tiles <= g_res_clusters;
   // resident rows and the cosine kind: scores, selection and compaction in the same kernel (CTA 0's
   // row buffer holds the m sort keys and the n kept flags by then)
