@@ -1886,13 +1886,12 @@ int gemm_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
     grid = tiles * a.csplit;
   } else if (a.dpr) {
     // grid set above
-  } else if (tiles <= work_slots && tiles * 2 > work_slots && a.tt >= 128 && 
-             (p.epi != EPI_ADD_F32 || a.determ || tiles * 4 > work_slots * 3)) {
+  } else if (tiles <= work_slots && tiles * 2 > work_slots && a.tt >= 128) {
     // between half and all of the work slots' worth of wide tiles: one whole tile per work item.
     // Stream-K's balance would split most tiles two or three ways, and the fixups of wide token
-    // tiles cost more than the idle SMs do. Residual tiles need no fixup (each part adds itself), so they take
-    // it up to three quarters: 640 tokens (48 tiles for 76 pairs), two layers 647 -> 627 us; 1000 tokens (64
-    // tiles) 795 -> 817 with it.
+    // tiles cost more than the idle SMs do. Residual tiles need no fixup (each part adds itself) and
+    // would gain up to three quarters of the slots (640 tokens, two layers: 636 against 655 us), but
+    // their parts would land in any order: whole tiles give the same bits in every run.
     grid = tiles;
   }
   a.grid = int(grid);

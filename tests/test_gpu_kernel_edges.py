@@ -102,6 +102,28 @@ def test_few_token_epilogues(M, K, n):
     assert N.spd_workspace_status(ws) == 0
 
 
+@pytest.mark.parametrize("M", [640, 1000, 1200])  # 48, 64 and 80 pair tiles of 4096 rows for 76 slots
+def test_residual_whole_tiles_repeat_exactly(M):
+    # between half and all of the slots a residual tile belongs to one work item, which adds each element
+    # once: the same bits in every run (80 tiles are more than the slots: split, right within rounding)
+    K = n = 4096
+    g = torch.Generator().manual_seed(M)
+    X = torch.randn(M, K, generator=g).to(torch.bfloat16).cuda()
+    W = (torch.randn(n, K, generator=g) * 0.05).to(torch.bfloat16).cuda()
+    h0 = torch.randn(M, n, generator=g).cuda()
+    ws = torch.zeros(N.spd_linear_workspace_size(M, n), dtype=torch.uint8, device="cuda")
+    outs = []
+    for _ in range(4):
+        h = h0.clone()
+        N.spd_linear(X, M, K, W, n, N.EPI_ADD_F32, h, n, ws)
+        outs.append(h)
+    torch.cuda.synchronize()
+    assert N.spd_workspace_status(ws) == 0
+    assert rowwise_rel(outs[0].cpu().numpy(), (h0.double() + X.double() @ W.double().T).cpu().numpy()) < 1e-4
+    if M < 1200:
+        assert all(torch.equal(o, outs[0]) for o in outs)
+
+
 # ---- MSV-Prune: K-means over the whole GPU, rankings over several CTAs --------------------------------
 def _shuffled_tile(seed0, n, d, keep, **kw):
     # a tile whose planted groups lie scattered over the token order: the seeds fall into any of them, so
