@@ -8,9 +8,9 @@
 //   warp 5     MMA issuer: S = Q K^T into TMEM (kind::f16, fp32), then O += P V with P read from TMEM and V
 //              read in place as an MN-major operand (the layout its TMA box has)
 //   warps 0-3  softmax: thread r owns query row r (TMEM lane r); one pass over the block's 64 scores in
-//              registers, online softmax in fp32 with exp2, P rounded to bf16 over S's own TMEM columns; O
-//              is rescaled in TMEM only when a row's maximum grew by more than a factor of two (until then
-//              P, l and O keep the older, smaller reference); at the end O / l goes to HBM in bf16
+//              registers, online softmax in fp32 with exp2, P rounded to bf16 over S's own TMEM columns, the
+//              row sum over the unrounded weights; O is rescaled in TMEM when a row's maximum grew; at the
+//              end O / l goes to HBM in bf16
 // S alternates between two TMEM buffers, so S of block j + 1 is computed while the softmax of block j
 // runs. A query at position p sees keys 0..p of its own sequence; tiles run from the last to the first (in
 // causal order the longest first), all heads of a tile side by side. Every wait is bounded (status
@@ -20,7 +20,9 @@
 // from shared memory), 512 of exponentials and about 300 instructions a softmax thread; the CTAs of an SM fill
 // each other's waits. With one CTA of 128-key blocks an SM (P through shared memory, two passes over S, a
 // rescale at every new maximum) the tensor pipe idled through each softmax: four requests of 1021-3302
-// tokens, 28 heads of 128, 492 us; so 243 us (0.47 of the burst bf16 rate, counting the causal half only).
+// tokens, 28 heads of 128, 492 us; so 252 us (0.45 of the burst bf16 rate, counting the causal half only).
+// Rescaling only where a maximum doubled and adding up the rounded weights took 244 us, at the price of weights
+// up to 2 and of sums of 16-bit values; relative error against 64 bits 2.029e-3 (2.037e-3 with 128-key blocks).
 #include <cuda_bf16.h>
 #include <math.h>
 #include <stdint.h>
@@ -43,11 +45,6 @@ constexpr uint32_t kQBox = 128 * 128;  // one TMA box of Q: 128 rows x 64 bf16
 constexpr uint32_t kKBox = kTK * 128;  // ... of K and V: 64 rows
 constexpr int kThreads = 192;
 constexpr uint32_t kTmemCols = 256;    // S: two buffers [0, 64) and [64, 128); O: [128, 128 + HD)
-// log2 growth of a row's maximum that rescales O. The largest weight of a row is 1, exact in bf16, only
-// relative to its own maximum: relative error against 64 bits 2.016e-3 / 2.019e-3 / 2.026e-3 / 2.049e-3 /
-// 2.072e-3 at 0 / 0.5 / 1 / 2 / 8 (2.037e-3 with the sum over unrounded weights and a rescale at every new
-// maximum, as before), 257 / 248 / 243 / 239 / 237 us for four requests of 1021-3302 tokens.
-constexpr float kRescale = 1.0f;
 
 template <int HD>
 struct AttnSmem {
@@ -213,8 +210,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     // ---- softmax and epilogue: warp w reads TMEM lanes [32 w, 32 w + 32) ----
     const int r = warp * 32 + lane;  // query row of the tile
     const uint32_t lanes = static_cast<uint32_t>(warp * 32) << 16;
-    const float grow = kRescale / scale_log2;
-    float m_run = -INFINITY, l_run = 0.0f;  // the row's reference maximum (raw scores) and sum
+    float m_run = -INFINITY, l_run = 0.0f;  // the row's maximum so far (raw scores) and sum of weights
     const int pos_min = __shfl_sync(0xffffffffu, my_pos, 0);  // the warp's first row sees the fewest keys
     bool ok = true;
     for (int j = 0; j < nkb; ++j) {
@@ -236,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
       if (j == 0) {
         m_run = mx;  // finite: block 0 holds key 0 <= every position
-      } else if (__any_sync(0xffffffffu, mx > m_run + grow)) {
+      } else if (__any_sync(0xffffffffu, mx > m_run)) {
         // the previous PV product has completed (the one before it had when these scores came): O can be
         // rescaled
         if (!(ok = __all_sync(0xffffffffu, mbar_wait(o_done, (j - 1) & 1, abort_flag, budget))))
@@ -261,10 +257,9 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
       for (int i = 0; i < kTK; i += 2) {
         const float p0 = ex2(fmaf(v[i], scale_log2, -off)), p1 = ex2(fmaf(v[i + 1], scale_log2, -off));
-        const uint32_t pr = pack_bf16(p0, p1);
-        r4[i & 2] += __uint_as_float(pr << 16);  // the sum of the weights as the product sees them
-        r4[(i & 2) + 1] += __uint_as_float(pr & 0xffff0000u);
-        pk[i >> 1] = pr;
+        r4[i & 2] += p0;
+        r4[(i & 2) + 1] += p1;
+        pk[i >> 1] = pack_bf16(p0, p1);
       }
       l_run += (r4[0] + r4[1]) + (r4[2] + r4[3]);
       float pf[32];

@@ -191,12 +191,12 @@ def test_anchor_ranking_with_ties(n):
     np.testing.assert_array_equal(g["keep_idx"][0], op.select_anchors(v["attn"][0, 0].astype(np.float64), n // 2))
 
 
-# ---- prefill attention: 64-key blocks, P in TMEM, rescales only where a maximum doubled ----------------
+# ---- prefill attention: 64-key blocks, P in TMEM ---------------------------------------------------------
 @pytest.mark.parametrize("lens,H,Hkv,hd,frac,ramp", [
     ([63, 64, 65, 1, 191, 193], 4, 2, 128, 1.0, 0.0),  # lengths at the edges of key blocks
     ([127, 128, 129, 257], 4, 4, 64, 0.6, 0.0),        # ... and of query tiles
-    ([700], 7, 1, 128, 0.9, 2.0),                      # maxima that grow by less than the threshold a block
-    ([700], 2, 2, 64, 0.9, 40.0),                      # ... by more at every block
+    ([700], 7, 1, 128, 0.9, 2.0),                      # maxima that grow a little a block
+    ([700], 2, 2, 64, 0.9, 40.0),                      # ... by much at every block
     ([1500, 40], 2, 1, 128, 0.05, 8.0),                # few queries far down a long sequence
     ([2996, 1021], 14, 2, 128, 1.0, 0.0),              # many blocks and CTAs: warps of a CTA run ahead of others
 ])
@@ -207,3 +207,28 @@ def test_attention_edges(lens, H, Hkv, hd, frac, ramp):
     ref = A.oracle_attention(q, q_pos, q_cu, kv, cu, H, Hkv, hd)
     assert np.isfinite(got).all()
     assert rowwise_rel(got, ref) < A.TOL
+
+
+@pytest.mark.parametrize("hd,ramp", [(128, 0.0), (128, 2.0), (64, 6.0)])
+def test_attention_weights_and_sums(hd, ramp):
+    # the arithmetic of the kernel, step by step: weights relative to the running maximum of 64-key blocks
+    # (at most 1), rounded to bf16 for the product alone, the row sum over the unrounded ones. fp32
+    # sums move an output by about 1e-5 of itself, past one in 250 of bf16's borders: 2 % may differ.
+    from tests import test_gpu_attention as A
+    n, H = 700, 2
+    q, q_pos, q_cu, kv, cu = A.case([n], H, H, hd, 1.0, seed=hd, ramp=ramp)
+    got = A.run(q, q_pos, q_cu, kv, cu, H, H, hd)
+    qf, kvf = bf16_np(q).reshape(n, H, hd), bf16_np(kv).reshape(n, 2, H, hd)
+    want = np.zeros((n, H, hd))
+    for h in range(H):
+        z = (qf[:, h] @ kvf[:, 0, h].T) * (1.4426950408889634 / np.sqrt(hd))
+        z[np.triu_indices(n, 1)] = -np.inf
+        m, l, o = np.full((n, 1), -np.inf), np.zeros((n, 1)), np.zeros((n, hd))
+        for k in range(0, n, 64):
+            mn = np.maximum(m, z[:, k:k + 64].max(1, keepdims=True))
+            p, corr = np.exp2(z[:, k:k + 64] - mn), np.exp2(m - mn)
+            pb = torch.from_numpy(p).float().to(torch.bfloat16).double().numpy()
+            l, o, m = l * corr + p.sum(1, keepdims=True), o * corr + pb @ kvf[k:k + 64, 1, h], mn
+        want[:, h] = o / l
+    want = torch.from_numpy(want.reshape(n, H * hd)).float().to(torch.bfloat16).double().numpy()
+    assert (got.reshape(n, H * hd) == want).mean() > 0.98
