@@ -1448,12 +1448,18 @@ __global__ void __launch_bounds__(kGemvThreads, 3)
 // Two to 16 tokens (a decode step of as many sequences): still a weight stream, but with one fp32 FMA per
 // weight and token the kernel above was bound by instructions (4 layers of LLaVA width: 441 us a step at one
 // token, 689 at two, 732 at four), and the tiled kernel streams at half the HBM rate. Here the tokens are the
-// 8 columns of m16n8k16 (NT = 2: two sets of them): a warp owns 16 of the CTA's 32 weight rows and a quarter of its K range, the
-// weights go from 16-byte loads straight into the A operand (the order of K is free: lane (r, c) takes
-// columns 8 c .. 8 c + 7 of a 32-wide step of rows r and r + 8 and the same columns of token r), eight
-// weight loads in flight a lane. The quarters are added in a fixed order through shared memory. The same step:
-// 423 us at two tokens (1-token kernel's prefetch, a quarter of it per quarter row; 463 with four times as
-// much), 480 at eight and 585 at 16, where the tiled kernel took 577 and 662.
+// 8 columns of m16n8k16 (NT = 2: two sets of them): a warp owns 16 of the CTA's 32 weight rows and a quarter
+// of its K range, the weights go from 16-byte loads straight into the A operand (the order of K is free: lane
+// (r, c) takes columns 8 c .. 8 c + 7 of a 32-wide step of rows r and r + 8 and the same columns of token r),
+// eight weight loads in flight a lane. The quarters are added in a fixed order through shared memory. The same
+// step: 429 us at two tokens (1-token kernel's prefetch, a quarter of it per quarter row; 463 with four times
+// as much), 480 at eight and 561 at 16, where the tiled kernel took 577 and 662.
+// Sums: the tensor cores cut a product's low bits off at its accumulator's, so a chain over K is 2 to 27 times
+// further from 64 bits than fp32 FMAs (K 1024 to 18944: 2.3e-7 to 5.1e-6, FMAs 6.9e-8 to 1.9e-7). Up to
+// eight tokens every product of 16 columns starts from zero, a batch's eight are added as an fp32 tree and
+// the quarters with their rounding errors: 5.0e-8 / 6.3e-8 / 8.0e-8 / 1.3e-7 at K 256 / 1024 / 4096 / 18944 where
+// FMAs have 5.5e-8 / 6.9e-8 / 9.4e-8 / 1.9e-7. (Two CTAs an SM instead of three hold the tree without spills.)
+// Nine to 16 tokens keep the chain, whose error is the tiled kernel's that they would take otherwise.
 constexpr int kGemvMmaTok = 16;  // 20 tokens: 787 us against 715 with the tiled kernel
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
@@ -1465,8 +1471,20 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// (a + b) + (c + d) with the rounding errors of the three additions added back (Knuth's two-sum).
+__device__ __forceinline__ float sum4_compensated(float a, float b, float c, float d) {
+  float err = 0.0f;
+  auto two_sum = [&](float x, float y) {
+    const float s = __fadd_rn(x, y), t = __fsub_rn(s, x);
+    err += __fadd_rn(__fsub_rn(x, __fsub_rn(s, t)), __fsub_rn(y, t));
+    return s;
+  };
+  const float s = two_sum(two_sum(a, b), two_sum(c, d));
+  return isfinite(s) ? s + err : s;  // infinities and NaN have no error term
+}
+
 template <int EPI, int NT>
-__global__ void __launch_bounds__(kGemvThreads, NT == 1 ? 3 : 2)
+__global__ void __launch_bounds__(kGemvThreads, 2)
     gemv_mma_kernel(const uint16_t* __restrict__ w, const uint16_t* x, const KArgs a, int ksplit) {
   __shared__ float red[4][32][8 * NT + 1];
   __shared__ int trow[8 * NT], tpos[8 * NT];
@@ -1514,13 +1532,27 @@ __global__ void __launch_bounds__(kGemvThreads, NT == 1 ? 3 : 2)
 #pragma unroll
       for (int q = 0; q < NT; ++q)
         xv[u][q] = r + 8 * q < a.n_tok && st + u < steps ? xp[size_t(q) * a.k + 4 * (st + u)] : z;  // 8 rows of k / 8 int4
+    if constexpr (NT == 1) {
+      float p[2 * U][4];
 #pragma unroll
-    for (int u = 0; u < U; ++u)
+      for (int u = 0; u < U; ++u) {
 #pragma unroll
-      for (int q = 0; q < NT; ++q) {
-        mma_16816(acc[q], b0[u].x, b1[u].x, b0[u].y, b1[u].y, xv[u][q].x, xv[u][q].y);
-        mma_16816(acc[q], b0[u].z, b1[u].z, b0[u].w, b1[u].w, xv[u][q].z, xv[u][q].w);
+        for (int e = 0; e < 4; ++e) p[2 * u][e] = p[2 * u + 1][e] = 0.0f;
+        mma_16816(p[2 * u], b0[u].x, b1[u].x, b0[u].y, b1[u].y, xv[u][0].x, xv[u][0].y);
+        mma_16816(p[2 * u + 1], b0[u].z, b1[u].z, b0[u].w, b1[u].w, xv[u][0].z, xv[u][0].w);
       }
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        acc[0][e] += ((p[0][e] + p[1][e]) + (p[2][e] + p[3][e])) + ((p[4][e] + p[5][e]) + (p[6][e] + p[7][e]));
+    } else {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int q = 0; q < NT; ++q) {
+          mma_16816(acc[q], b0[u].x, b1[u].x, b0[u].y, b1[u].y, xv[u][q].x, xv[u][q].y);
+          mma_16816(acc[q], b0[u].z, b1[u].z, b0[u].w, b1[u].w, xv[u][q].z, xv[u][q].w);
+        }
+    }
   }
   const int lr = 16 * (warp >> 2) + r;
 #pragma unroll
@@ -1535,8 +1567,10 @@ __global__ void __launch_bounds__(kGemvThreads, NT == 1 ? 3 : 2)
     const int t0 = 8 * warp;
     float v[8];
 #pragma unroll
-    for (int t = 0; t < 8; ++t)
-      v[t] = (red[0][lane][t0 + t] + red[1][lane][t0 + t]) + (red[2][lane][t0 + t] + red[3][lane][t0 + t]);
+    for (int t = 0; t < 8; ++t) {
+      const float q0 = red[0][lane][t0 + t], q1 = red[1][lane][t0 + t], q2 = red[2][lane][t0 + t], q3 = red[3][lane][t0 + t];
+      v[t] = NT == 1 ? sum4_compensated(q0, q1, q2, q3) : (q0 + q1) + (q2 + q3);
+    }
     epilogue8<EPI>(a, n0 + lane, (n0 >> 5) & 3, lane, n0 >> 7, t0, v, trow, tpos, 0);
     if (lane == 0) stamp_end(a.stamp);
   }

@@ -102,6 +102,27 @@ def test_few_token_epilogues(M, K, n):
     assert N.spd_workspace_status(ws) == 0
 
 
+@pytest.mark.parametrize("M", [2, 4, 8])
+@pytest.mark.parametrize("K", [256, 1024, 4096, 18944])
+def test_few_token_sums_are_fp32(M, K):
+    # sums of up to eight tokens round like fp32: an output passes about 8 additions and K / 512 more, each
+    # half a unit (2^-24) of its sum off at most and, adding up at random, their root of it in all.
+    n = 4096
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    X = torch.randn(M, K, generator=g, device="cuda").to(torch.bfloat16)
+    W = (torch.randn(n, K, generator=g, device="cuda") * K ** -0.5).to(torch.bfloat16)
+    ws = torch.zeros(N.spd_linear_workspace_size(M, n), dtype=torch.uint8, device="cuda")
+    out = torch.empty(M, n, device="cuda")
+    N.spd_linear(X, M, K, W, n, N.EPI_F32, out, n, ws)
+    ref = X.double() @ W.double().T
+    assert ((out.double() - ref).norm() / ref.norm()).item() < 2.0 ** -24 * (8 + K / 512) ** 0.5
+    # infinities stay infinities: one infinite weight
+    W[:, 0] = float("inf")
+    X[:, 0] = 1.0
+    N.spd_linear(X, M, K, W, n, N.EPI_F32, out, n, ws)
+    assert torch.isposinf(out).all()
+
+
 @pytest.mark.parametrize("M", [640, 1000, 1200])  # 48, 64 and 80 pair tiles of 4096 rows for 76 slots
 def test_residual_whole_tiles_repeat_exactly(M):
     # between half and all of the slots a residual tile belongs to one work item, which adds each element
