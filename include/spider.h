@@ -396,6 +396,7 @@ typedef enum {
 size_t spd_linear_workspace_size(int M, int N);
 
 /* out = epilogue(X W^T) on the tcgen05 tensor cores, fp32 accumulation.
+ * Every input, W too, may be the output of the work enqueued on `stream` just before.
  * X (dev) bf16 [M][K]; W (dev) bf16 [N][K]; K a multiple of 8; N a multiple of 128 (or equal to
  * a padded weight count whose extra rows are never written); bias (dev) bf16 [N] or NULL; rows (dev)
  * int32 [M] or NULL; out (dev) as described by the epilogue, row stride ldo elements. */

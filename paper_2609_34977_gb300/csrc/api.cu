@@ -351,6 +351,7 @@ extern "C" int spd_linear(const uint16_t* X, int M, int K, const uint16_t* W, in
   p.rows = rows;
   p.bias = bias;
   p.out_cols = N;
+  p.w_new = true;
   return gemm_run(p, s, st);
 }
 
@@ -422,6 +423,7 @@ extern "C" int spd_linear_noalloc(const uint16_t* X, int M, int K, const uint16_
   p.rows = rows;
   p.bias = bias;
   p.out_cols = N;
+  p.w_new = true;
   if (int rc = gemm_run(p, s, st)) return rc;
   if (status) SPD_CUDA_TRY(cudaMemcpyAsync(status, s.status, sizeof(int), cudaMemcpyDeviceToDevice, st));
   return SPD_OK;

@@ -78,8 +78,9 @@ constexpr int kCounters = 1 << 16;
 constexpr int kRecvPitch = 36;      // fp32 per row of a received 32-column chunk (conflict-free)
 
 struct KArgs {
-  int n_out, n_tok, k, tt, n_kb, n_ttiles, units, grid, stages, ldo, rope_rows, head_dim,
+  int n_out, n_tok, k, w_new, tt, n_kb, n_ttiles, units, grid, stages, ldo, rope_rows, head_dim,
       out_cols, kbox, csplit, cluster, nbuf, hoff, nh, ldo2, split, accs;
+  // w_new: the weights may be the output of the launch before (see GemmProblem; tiled kernel)
   // kbox: 64-wide boxes per stage (1 or 2); a k-block is kbox * 64 wide
   // csplit: CTAs per output tile in split-K (1 = stream-K); cluster: split-K CTAs reduce through
   // distributed shared memory (0: ADD epilogue, every CTA adds its own partial)
@@ -654,6 +655,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ---- TMA producer ----
       // The first stages' weight boxes do not depend on the previous kernel: they are issued
       // before griddepcontrol.wait, so the weight stream starts while that kernel drains.
+      if (a.w_new) pdl_wait();
       const uint64_t pol_w = policy_evict_first(), pol_x = policy_evict_last();
       int pre_tile[kMaxStages], pre_kb[kMaxStages];
       int n_pre = 0;
@@ -1761,8 +1763,8 @@ int gemv_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
     while (groups * ksplit < num_sms() && ksplit * 2 <= C && ksplit < 8) ksplit *= 2;
   if (!gemv_eligible(p)) {
     const int slot = trace_begin(stream);
-    SPD_CUDA_TRY(launch_pdl(gemv_mma_for(p.epi, p.n_tok), dim3(groups * ksplit), dim3(kGemvThreads), 0, stream,
-                            static_cast<const uint16_t*>(p.w), static_cast<const uint16_t*>(p.x), a, ksplit));
+    SPD_CUDA_TRY(launch_with(!p.w_new, 0, gemv_mma_for(p.epi, p.n_tok), dim3(groups * ksplit), dim3(kGemvThreads), 0,
+                             stream, static_cast<const uint16_t*>(p.w), static_cast<const uint16_t*>(p.x), a, ksplit));
     trace_gemm(slot, p, stream);
     return SPD_OK;
   }
@@ -1784,9 +1786,8 @@ int gemv_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
   // shared memory for three CTAs an SM (what the registers allow) and no more: the rest of the array buffers the
   // weight loads in flight (one token, 32 layers: 3140 us a step with the driver's choice, 3084 so)
   const int carveout = int(std::min<size_t>(100, 3 * (smem + 1536) * 100 / (256 * 1024)));
-  SPD_CUDA_TRY(launch_pdl_carveout(carveout, kern, dim3(groups * ksplit), dim3(kGemvThreads), smem, stream,
-                                   static_cast<const uint16_t*>(p.w), static_cast<const uint16_t*>(p.x), a,
-                                   ksplit));
+  SPD_CUDA_TRY(launch_with(!p.w_new, carveout, kern, dim3(groups * ksplit), dim3(kGemvThreads), smem, stream,
+                           static_cast<const uint16_t*>(p.w), static_cast<const uint16_t*>(p.x), a, ksplit));
   trace_gemm(slot, p, stream);
   return SPD_OK;
 }
@@ -1961,6 +1962,7 @@ int gemm_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {
   a.counters = s.counters;
   a.status = s.status;
   a.budget = kWaitBudget;
+  a.w_new = p.w_new;
   a.stamp = gemm_stamp(p);
   a.vec_red = vec_red_ok(p);
   {

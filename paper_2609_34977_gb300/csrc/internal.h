@@ -33,7 +33,7 @@ int num_sms();  // SM count of the current device
 // Rules every kernel of the library keeps under this overlap (the chain of launches in a stream
 // can have several kernels resident at once, each waiting on its predecessor):
 //  * before griddepcontrol.wait a kernel reads only data that no launch of the library writes
-//    (weights, tensor maps, its own arguments) and writes nothing but its own shared memory;
+//    (weights of a model handle, tensor maps, its own arguments) and writes nothing but its own shared memory;
 //  * data that an earlier kernel of the stream wrote is read after the wait, and never through
 //    the non-coherent path (no const __restrict__ pointers or ld.global.nc on it: PTX allows that
 //    path only for data that stays unchanged while the kernel runs, and here the predecessor
@@ -43,9 +43,10 @@ int num_sms();  // SM count of the current device
 //    stream has completed.
 // carveout: the share of an SM's 256 KB that is set aside as shared memory, in percent (0: the driver's choice,
 // which can hold a kernel of several CTAs an SM below the number that its registers allow).
+// overlap: false starts the kernel only when everything before it in the stream has completed.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl_carveout(int carveout, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                cudaStream_t stream, Args&&... args) {
+cudaError_t launch_with(bool overlap, int carveout, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                        cudaStream_t stream, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -53,12 +54,17 @@ cudaError_t launch_pdl_carveout(int carveout, void (*kernel)(KArgs...), dim3 gri
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = overlap;
   attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
   attr[1].val.sharedMemCarveout = unsigned(carveout);
   cfg.attrs = attr;
   cfg.numAttrs = carveout > 0 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_carveout(int carveout, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                cudaStream_t stream, Args&&... args) {
+  return launch_with(true, carveout, kernel, grid, block, smem, stream, std::forward<Args>(args)...);
 }
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
@@ -126,6 +132,11 @@ struct GemmProblem {
   const uint16_t* norm_gain;
   const int32_t* norm_rows;
   float norm_eps;
+  // The weights are a buffer of the caller's, which earlier work of the stream may write: the tiled kernel loads
+  // them after the grid dependency wait, and the matrix-vector kernels, which read them through the
+  // non-coherent path, are launched without overlap. Otherwise (weights of a model handle, which nothing
+  // writes after its creation) the first of them are loaded under several unfinished launches.
+  bool w_new;
 };
 // True when gemm_run will run p on the matrix-vector path, which can apply the input RMSNorm itself.
 bool gemm_fuses_norm(const GemmProblem& p);

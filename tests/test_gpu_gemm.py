@@ -110,11 +110,53 @@ def test_linear_cta_pairs(M, K, N_, epi, determ):
         assert torch.equal(outs[0], outs[1])
 
 
+@pytest.mark.parametrize("M,N_,epi", [
+    (1, 4096, N.EPI_F32),       # the matrix-vector kernel
+    (8, 4096, N.EPI_BF16),      # a few tokens on m16n8k16, one set of token columns
+    (16, 4096, N.EPI_F32),      # ... two sets
+    (77, 1024, N.EPI_F32),      # few tiles: K split over clusters
+    (640, 4096, N.EPI_BF16),    # one whole tile per work item
+    (64, 4096, N.EPI_ADD_F32),  # residual tiles, K split
+])
+def test_linear_weights_written_by_the_launch_before(M, N_, epi):
+    # W is the output of the spd_linear call right before on the stream (which writes its last rows late): every
+    # repeat has to read the new W, not the zeros that lay there
+    K, M0 = 4096, 4096
+    X0, W0 = operands(M0, 1024, K, seed=1)
+    X, _ = operands(M, K, 8, seed=2)
+    X0, W0, X = X0.cuda(), (W0 * 0.05).cuda(), X.cuda()
+    ws = [torch.zeros(N.spd_linear_workspace_size(M0, K), dtype=torch.uint8, device="cuda") for _ in range(2)]
+    W = torch.empty(M0, K, dtype=torch.bfloat16, device="cuda")
+    dt = torch.bfloat16 if epi == N.EPI_BF16 else torch.float32
+
+    def chain(sync=False):
+        W.zero_()
+        out = torch.zeros(M, N_, dtype=dt, device="cuda")
+        N.spd_linear(X0, M0, 1024, W0, K, N.EPI_BF16, W, K, ws[0])
+        if sync:
+            torch.cuda.synchronize()
+        N.spd_linear(X, M, K, W[M0 - N_:], N_, epi, out, N_, ws[1])
+        return out
+
+    want = chain(sync=True)
+    torch.cuda.synchronize()
+    ref = X.double() @ W[M0 - N_:].double().T
+    tol = 2 ** -8 if epi == N.EPI_BF16 else 1e-4
+    assert rowwise_rel(want.double().cpu().numpy(), ref.cpu().numpy()) < tol
+    for _ in range(30):
+        got = chain()
+        if epi == N.EPI_ADD_F32:  # parts of K land in any order
+            assert rowwise_rel(got.double().cpu().numpy(), ref.cpu().numpy()) < tol
+        else:
+            assert torch.equal(got, want)
+    assert all(N.spd_workspace_status(w) == 0 for w in ws)
+
+
 @pytest.mark.parametrize("M", [1, 2, 3, 4])
 @pytest.mark.parametrize("K,N_", [(256, 1000), (4096, 4096), (11008, 640)])
 def test_linear_few_tokens_matrix_vector_path(M, K, N_):
-    # at most four tokens with K a multiple of 256: the matrix-vector kernel (F32 output, and the
-    # residual scatter-add, whose K range is split over several CTAs)
+    # one token with K a multiple of 256: the matrix-vector kernel, more (up to 16): the few-token kernel
+    # (F32 output, and the residual scatter-add, whose K range is split over several CTAs)
     X, W = operands(M, K, N_, seed=M + K)
     ref = bf16_np(X) @ bf16_np(W).T
     ws = torch.zeros(N.spd_linear_workspace_size(M, N_), dtype=torch.uint8, device="cuda")
