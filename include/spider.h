@@ -55,6 +55,12 @@ int spd_workspace_status(void* ws, void* stream, int* status);
  * context stays usable. Asynchronous; read the result with spd_workspace_status. */
 int spd_selftest_bounded_wait(void* ws, long long budget_cycles, void* stream);
 
+/* The same for the barrier between CTAs of the whole-GPU K-means: 16 CTAs go through `barriers` barriers
+ * that a 17th would have to reach. The first one expires after `budget_cycles` in every CTA, records
+ * SPD_ETIMEOUT in the status word of `ws` (at least 8 bytes of device memory) and ends the wait of all
+ * that follow. Asynchronous; read the result with spd_workspace_status. Errors: SPD_EINVAL, SPD_ECUDA. */
+int spd_selftest_tile_barrier(void* ws, int barriers, long long budget_cycles, void* stream);
+
 /* Deterministic mode (library-wide; no counterpart in the paper). With on != 0, every GEMM sums
  * each output element in a fixed order: K-split tiles store per-CTA fp32 partials that the tile's
  * last CTA adds in CTA order, and residual updates of the fp32 stream are one read-modify-write per

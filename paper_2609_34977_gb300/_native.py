@@ -19,7 +19,7 @@ SPD_MAX_FEAT_LAYERS = 4
 EPI_F32, EPI_BF16, EPI_BIAS_BF16, EPI_BIAS_GELU_BF16, EPI_ADD_F32 = 0, 1, 2, 3, 4
 
 # every symbol include/spider.h declares
-EXPORTS = ("spd_last_error", "spd_workspace_status", "spd_selftest_bounded_wait",
+EXPORTS = ("spd_last_error", "spd_workspace_status", "spd_selftest_bounded_wait", "spd_selftest_tile_barrier",
            "spd_prune_workspace_size", "spd_prune_launches", "spd_prune", "spd_received_attention_workspace_size",
            "spd_received_attention", "spd_gather_rows_bf16", "spd_model_create",
            "spd_model_destroy", "spd_plan_adaptive", "spd_plan_static", "spd_project_workspace_size",
@@ -99,6 +99,7 @@ def lib():
             "spd_last_error": (C.c_char_p, []),
             "spd_workspace_status": (i, [vp, vp, C.POINTER(i)]),
             "spd_selftest_bounded_wait": (i, [vp, ll, vp]),
+            "spd_selftest_tile_barrier": (i, [vp, i, ll, vp]),
             "spd_prune_workspace_size": (sz, [C.POINTER(PruneCfg)]),
             "spd_prune_launches": (i, [C.POINTER(PruneCfg)]),
             "spd_prune": (i, [C.POINTER(PruneCfg), C.POINTER(vp), vp, vp, vp, vp, vp, vp, sz, vp]),
@@ -233,6 +234,10 @@ def spd_workspace_status(ws, stream=None) -> int:
 
 def spd_selftest_bounded_wait(ws, budget_cycles: int, stream=None):
     _check(lib().spd_selftest_bounded_wait(_p(ws), int(budget_cycles), _stream(stream)))
+
+
+def spd_selftest_tile_barrier(ws, barriers: int, budget_cycles: int, stream=None):
+    _check(lib().spd_selftest_tile_barrier(_p(ws), int(barriers), int(budget_cycles), _stream(stream)))
 
 
 def prune_cfg(n_tiles, n_tok, d_feat, n_layers, final_layer, n_heads, keep, *, has_cls=True,

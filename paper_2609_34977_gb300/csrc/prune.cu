@@ -1167,9 +1167,11 @@ constexpr int kGridMaxRows = 512;  // a CTA
 constexpr int kGridMeta = 2 * SPD_MAX_CLUSTERS;  // ints a CTA: sizes, [15 + 1]: changed flag; then a_j sums
 
 // Barrier number `phase` (1, 2, ...) of the G CTAs sharing *counter (zero at the start of the call). The
-// wait is bounded: on expiry the status is set and the counter raised past every later target, so that
-// every CTA of the tile runs on to its end.
-__device__ __forceinline__ void tile_barrier(int* counter, int G, int phase, int* status) {
+// wait is bounded: on expiry the status is set and the counter raised past every target, whichever CTAs
+// expire with this one, so that no later barrier of the call waits. False from then on.
+constexpr int kBarrierGone = 1 << 30;
+__device__ __forceinline__ bool tile_barrier(int* counter, int G, int phase, int* status, long long budget) {
+  bool gone = false;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -1178,15 +1180,24 @@ __device__ __forceinline__ void tile_barrier(int* counter, int G, int phase, int
     while (true) {
       int v;
       asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
-      if (v >= G * phase) break;
-      if (clock64() - t0 > kWaitBudget) {
+      if (v >= G * phase) {
+        gone = v >= kBarrierGone;
+        break;
+      }
+      if (clock64() - t0 > budget) {
         set_status(status, SPD_ETIMEOUT);
-        atomicAdd(counter, 1 << 28);
+        atomicMax(counter, kBarrierGone);
+        gone = true;
         break;
       }
     }
   }
-  __syncthreads();
+  return !__syncthreads_or(gone);
+}
+
+// CTAs at `barriers` barriers in a row that one more CTA would have to reach (spd_selftest_tile_barrier).
+__global__ void tile_barrier_probe_kernel(int* ws, int barriers, long long budget) {
+  for (int i = 1; i <= barriers; ++i) tile_barrier(ws + 1, int(gridDim.x) + 1, i, ws, budget);
 }
 
 template <int KN, bool COS>
@@ -1217,6 +1228,7 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
   float* gcent = w.gcent + size_t(t) * KD;                  // [K][D]
   int* bar = &w.arrive[4 * t + 2];
   int phase = 0;
+  bool ok = true;  // no barrier has expired
   pdl_wait();
   for (int jj = threadIdx.x; jj < nl; jj += blockDim.x) {
     idx[jj] = ul[j0 + jj];
@@ -1279,7 +1291,7 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
     __syncthreads();
     // sizes of K <= 16 clusters and the flag in the first 16 ints of the CTA's block (a flag bit on size 0)
     if (threadIdx.x < K) meta[r * kGridMeta + threadIdx.x] = cnt[threadIdx.x] | (changed ? 1 << 30 : 0);
-    tile_barrier(bar, G, ++phase, w.status);
+    if (!(ok = tile_barrier(bar, G, ++phase, w.status, kWaitBudget))) break;
     if (threadIdx.x == 0) any_changed = 0;
     __syncthreads();
     if (warp < K) {
@@ -1306,7 +1318,7 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
       const int n = ncl[e / D];
       gcent[e] = n > 0 ? sum / float(n) : cent[e];
     });
-    tile_barrier(bar, G, ++phase, w.status);
+    if (!(ok = tile_barrier(bar, G, ++phase, w.status, kWaitBudget))) break;
     for (int e = 4 * threadIdx.x; e < KD; e += 4 * blockDim.x)
       *reinterpret_cast<float4*>(cent + e) = __ldcg(reinterpret_cast<const float4*>(gcent + e));
     __syncthreads();
@@ -1335,10 +1347,14 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
     column_sums(part + (size_t(r) * p.L + l) * KD, K, D, nl, ord, start,
                 RowAccess{res && l == p.fin ? rows : nullptr, p.feat[l], row0, idx, D, COS ? rinv : static_cast<float*>(nullptr)});
   }
-  tile_barrier(bar, G, ++phase, w.status);
+  ok = tile_barrier(bar, G, ++phase, w.status, kWaitBudget) && ok;
   pdl_launch_dependents();
   reduce(part, size_t(p.L) * KD, p.L * KD, [&](int e, float sum) { w.csum[size_t(t) * p.L * KD + e] = sum; });
   if (r != 0) return;
+  if (!ok) {  // an expired barrier (the status tells): the sizes may be anything, and nothing is selected by them
+    if (threadIdx.x < SPD_MAX_CLUSTERS) ncl[threadIdx.x] = 0;
+    __syncthreads();
+  }
   if (warp < K) {  // lane sums over CTAs lane, lane + 32, ..., then a butterfly: a fixed order
     float a = 0.0f;
     for (int cc = lane; cc < G; cc += 32) a += __int_as_float(__ldcg(meta + cc * kGridMeta + SPD_MAX_CLUSTERS + warp));
@@ -2174,6 +2190,15 @@ cudaError_t launch_stream(const PruneDims& p, const PruneWs& w, const PrunePlan&
 }  // namespace spd
 
 using namespace spd;
+
+extern "C" int spd_selftest_tile_barrier(void* ws, int barriers, long long budget_cycles, void* stream) {
+  if (!ws || barriers < 1) return fail(SPD_EINVAL, "null workspace or no barriers");
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  SPD_CUDA_TRY(cudaMemsetAsync(static_cast<int*>(ws) + 1, 0, sizeof(int), st));
+  tile_barrier_probe_kernel<<<16, 32, 0, st>>>(static_cast<int*>(ws), barriers, budget_cycles);
+  SPD_CUDA_TRY(cudaGetLastError());
+  return SPD_OK;
+}
 
 extern "C" int spd_prune_launches(const spd_prune_cfg* cfg) {
   PruneDims p;

@@ -23,6 +23,22 @@ def test_bounded_wait_times_out_and_context_survives():
     assert torch.all(out == 128.0)
 
 
+def test_expired_barrier_between_ctas_ends_the_later_ones():
+    # 16 CTAs expire together at a barrier that a 17th never reaches: the 199 barriers behind it must not wait
+    ws = torch.zeros(64, dtype=torch.int32, device="cuda")
+    N.spd_selftest_tile_barrier(ws, 1, 20_000)
+    torch.cuda.synchronize()
+    assert N.spd_workspace_status(ws) == N.SPD_ETIMEOUT
+    budget = 4_000_000  # 2 ms at 2 GHz
+    t = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    t[0].record()
+    N.spd_selftest_tile_barrier(ws, 200, budget)
+    t[1].record()
+    torch.cuda.synchronize()
+    assert N.spd_workspace_status(ws) == N.SPD_ETIMEOUT
+    assert t[0].elapsed_time(t[1]) < 20.0  # one limit and 200 round trips, not 200 limits (400 ms)
+
+
 def test_host_side_rejections_touch_nothing():
     ws = torch.zeros(16, dtype=torch.uint8, device="cuda")
     X = torch.ones(4, 128, dtype=torch.bfloat16, device="cuda")
