@@ -2000,6 +2000,7 @@ constexpr int kPruneCarveout = 50;
 constexpr size_t kResSmem = 200 * 1024;  // dynamic shared memory of the resident K-means
 int g_res_clusters = -1;                 // 16-CTA clusters of it the GPU holds at once
 int g_stream_clusters[9] = {};           // KC-CTA clusters of the one-sweep form, by KC
+bool g_grid_fits = false;                // one CTA an SM of the whole-GPU form can be resident
 
 template <int KC, bool RES, int KN, bool FUSED = false>
 cudaError_t launch_kmeans(const PruneDims& p, const PruneWs& w, const PruneOut& out, size_t smem,
@@ -2108,6 +2109,15 @@ int kmeans_setup() {
         n = 0;
       }
       g_res_clusters = n;
+      g_grid_fits = true;
+      for (const void* kern : {(const void*)kmeans_grid_kernel<4, true>, (const void*)kmeans_grid_kernel<4, false>,
+                               (const void*)kmeans_grid_kernel<SPD_MAX_CLUSTERS, true>,
+                               (const void*)kmeans_grid_kernel<SPD_MAX_CLUSTERS, false>}) {
+        int blocks = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, kGridThreads, kResSmem) != cudaSuccess)
+          cudaGetLastError();
+        if (blocks < 1) g_grid_fits = false;
+      }
     }
   });
   if (err != cudaSuccess) return fail(SPD_ECUDA, "K-means attributes: %s", cudaGetErrorString(err));
@@ -2124,7 +2134,8 @@ struct PrunePlan {
   int stream_slots;
   int launches;
 };
-PrunePlan prune_plan(const PruneDims& p) {
+// whole_gpu: false where a cooperative launch over every SM is not to be had.
+PrunePlan prune_plan(const PruneDims& p, bool whole_gpu = g_grid_fits) {
   PrunePlan q;
   q.anchor_sim = p.n_anc > 0 && p.m > 0 && p.wa != 0.0f;
   const size_t cent_bytes = size_t(2) * p.K * p.d * sizeof(float);
@@ -2143,7 +2154,7 @@ PrunePlan prune_plan(const PruneDims& p) {
   // 104 / 135 / 204 / 330 us a call; 9 / 10 tiles of 576 x 1024: 170 / 176 -> 149 / 160 us, but 12 of
   // them 183 -> 187 us.
   q.grid = 0;
-  if (!q.res && grid_tile(p)) {
+  if (!q.res && whole_gpu && grid_tile(p)) {
     const int G = std::min({num_sms() / p.n_tiles, kGridMaxCtas / p.n_tiles, (p.m + 3) / 4});
     const size_t nl = (p.m + G - 1) / std::max(G, 1);
     if (G >= 15 && nl <= size_t(kGridMaxRows)) {
@@ -2237,7 +2248,7 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
                           dim3((p.n + 7) / 8, T), dim3(256), 0, st, p, attn, w));
   SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, anchor_kernel, dim3(rank_ctas(p.n), T), dim3(kRankThreads), 0, st, p, w));
   if (int rc = kmeans_setup()) return rc;
-  const PrunePlan plan = prune_plan(p);
+  PrunePlan plan = prune_plan(p);
   if (plan.anchor_sim) {
     const int aw = (p.n_anc + 47) / 48 * 48 < (p.n_anc + 63) / 64 * 64 ? 48 : 64;
     const int ay = (p.n_anc + aw - 1) / aw;
@@ -2272,7 +2283,16 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    SPD_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, p, w, plan.grid, int(plan.grid_res)));
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p, w, plan.grid, int(plan.grid_res));
+    if (e == cudaErrorCooperativeLaunchTooLarge) {  // the stream's context has fewer SMs than the device
+      cudaGetLastError();
+      plan = prune_plan(p, false);
+    } else {
+      SPD_CUDA_TRY(e);
+    }
+  }
+  if (plan.grid) {
+    // launched above
   } else if (plan.fused && p.K == 4)
     SPD_CUDA_TRY((launch_kmeans<16, true, 4, true>(p, w, out, res_bytes, st)));
   else if (plan.fused)

@@ -192,6 +192,34 @@ def test_many_tiles_kmeans(tiles, n, d, keep, kw):
     test_whole_gpu_kmeans(tiles, n, d, keep, kw)
 
 
+def _stream_of_few_sms(n_sms):
+    # a stream of a green context (a part of the device's SMs) through the driver's interface
+    import ctypes as C
+    cu = C.CDLL("libcuda.so.1")
+    everything, part = (C.c_byte * 144)(), (C.c_byte * 144)()  # CUdevResource
+    groups, desc, ctx, stream = C.c_uint(1), C.c_void_p(), C.c_void_p(), C.c_void_p()
+    torch.cuda.init()
+    torch.zeros(1, device="cuda")  # the primary context is current
+    for rc in (lambda: cu.cuDeviceGetDevResource(0, everything, 1),  # 1: SMs
+               lambda: cu.cuDevSmResourceSplitByCount(part, C.byref(groups), everything, None, 0, n_sms),
+               lambda: cu.cuDevResourceGenerateDesc(C.byref(desc), part, 1),
+               lambda: cu.cuGreenCtxCreate(C.byref(ctx), desc, 0, 1),  # 1: default stream, required
+               lambda: cu.cuGreenCtxStreamCreate(C.byref(stream), ctx, 1, 0)):  # 1: non-blocking, required
+        code = rc()
+        if code != 0:
+            pytest.skip(f"no green context here (driver error {code})")
+    return torch.cuda.ExternalStream(stream.value)
+
+
+def test_large_tile_in_a_context_of_few_sms():
+    # a context that holds a part of the SMs cannot run the cooperative launch over all of them: the shape goes
+    # through the clusters instead, with the same result
+    _, v, res = conditioned_vision(20265001, 1, 1100, 1024, 2, 4, 150, 1, has_cls=False, attn_form=1)
+    with torch.cuda.stream(_stream_of_few_sms(32)):
+        assert_prune_parity(gpu_prune(v, 150, 1, has_cls=False, attn_form=1), res)
+    assert_prune_parity(gpu_prune(v, 150, 1, has_cls=False, attn_form=1), res)
+
+
 def test_whole_gpu_kmeans_iterations():
     v, res = _shuffled_tile(20264001, 900, 1280, 180)
     a = gpu_prune(v, 180, 1, has_cls=False, attn_form=1)
