@@ -1959,9 +1959,20 @@ int validate(const spd_prune_cfg* c, PruneDims* p) {
   return SPD_OK;
 }
 
-// Whether a call is of the few, large tiles that K-means spreads over the whole GPU (grid_plan below
-// decides with the device's SM count): workspace is set aside for them.
-bool grid_tile(const PruneDims& p) { return p.n_tiles <= 10 && p.m > 0; }
+// Dynamic shared memory of the resident K-means: its limit, and what p takes (a CTA's rows, centroids and sums).
+constexpr size_t kResSmem = 200 * 1024;
+size_t res_bytes(const PruneDims& p) {
+  return (size_t((p.m + 15) / 16) + 2 * size_t(p.K)) * p.d * sizeof(float);
+}
+// Whether a call may be one of the few, large tiles that K-means spreads over the whole GPU (prune_plan
+// decides with what the device holds): workspace is set aside for these alone. The others' rows are resident in
+// clusters, of which 152 SMs hold kResTiles at once.
+constexpr int kResTiles = 7;
+bool grid_tile(const PruneDims& p) {
+  return p.n_tiles <= 10 && p.m > 0 && (res_bytes(p) > kResSmem || p.n_tiles > kResTiles);
+}
+// Most CTAs a tile of that form.
+int grid_ctas(const PruneDims& p) { return std::min(kGridMaxCtas / p.n_tiles, (p.m + 3) / 4); }
 
 PruneWs carve(const PruneDims& p, Carve& cv) {
   PruneWs w;
@@ -1985,7 +1996,7 @@ PruneWs carve(const PruneDims& p, Carve& cv) {
   w.ssum = cv.take<double>(T * p.L * 16);
   w.score = cv.take<float>(T * (p.m + 1));
   w.arrive = cv.take<int>(T * 4);
-  const size_t gc = grid_tile(p) ? kGridMaxCtas : 0;  // CTAs of all tiles
+  const size_t gc = grid_tile(p) ? T * grid_ctas(p) : 0;  // CTAs of all tiles
   w.gpart = cv.take<float>(gc * p.L * p.K * p.d);
   w.gcent = cv.take<float>(gc ? T * p.K * p.d : 0);
   w.gdsum = cv.take<double>(gc * p.L * 16);
@@ -1997,7 +2008,6 @@ PruneWs carve(const PruneDims& p, Carve& cv) {
 // anchor_sim_kernel share an SM than its registers allow (64 tiles, us a call: 446 with the driver's choice,
 // 409 / 412 / 415 / 446 at 25 / 50 / 75 / 100 %; one tile 75, 68 / 66 / 71 / 72).
 constexpr int kPruneCarveout = 50;
-constexpr size_t kResSmem = 200 * 1024;  // dynamic shared memory of the resident K-means
 int g_res_clusters = -1;                 // 16-CTA clusters of it the GPU holds at once
 int g_stream_clusters[9] = {};           // KC-CTA clusters of the one-sweep form, by KC
 bool g_grid_fits = false;                // one CTA an SM of the whole-GPU form can be resident
@@ -2138,12 +2148,10 @@ struct PrunePlan {
 PrunePlan prune_plan(const PruneDims& p, bool whole_gpu = g_grid_fits) {
   PrunePlan q;
   q.anchor_sim = p.n_anc > 0 && p.m > 0 && p.wa != 0.0f;
-  const size_t cent_bytes = size_t(2) * p.K * p.d * sizeof(float);
-  const size_t res_bytes = size_t((p.m + 15) / 16) * p.d * sizeof(float) + cent_bytes;
   // K-means: the rows resident in shared memory over 16 CTAs per tile where they fit and all tiles
   // run in one wave of such clusters (latency); else the whole GPU or the one-sweep form below; else
   // (K other than 4, or rows too wide for the one-sweep ring) re-read from L2 each pass by 8 CTAs
-  q.res = p.m > 0 && res_bytes <= kResSmem && g_res_clusters > 0 && p.n_tiles <= g_res_clusters;
+  q.res = p.m > 0 && res_bytes(p) <= kResSmem && g_res_clusters > 0 && p.n_tiles <= g_res_clusters;
   // resident rows and the cosine kind: scores, selection and compaction in the same kernel (CTA 0's
   // row buffer holds the m sort keys and the n kept flags by then)
   const size_t row_bytes = size_t((p.m + 15) / 16) * p.d * sizeof(float);
@@ -2155,7 +2163,7 @@ PrunePlan prune_plan(const PruneDims& p, bool whole_gpu = g_grid_fits) {
   // them 183 -> 187 us.
   q.grid = 0;
   if (!q.res && whole_gpu && grid_tile(p)) {
-    const int G = std::min({num_sms() / p.n_tiles, kGridMaxCtas / p.n_tiles, (p.m + 3) / 4});
+    const int G = std::min(num_sms() / p.n_tiles, grid_ctas(p));
     const size_t nl = (p.m + G - 1) / std::max(G, 1);
     if (G >= 15 && nl <= size_t(kGridMaxRows)) {
       q.grid = G;
@@ -2267,7 +2275,6 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
     SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, kern, dim3(g.x * as, g.y, T), dim3(256), 0, st, p, w));
   }
   const size_t cent_bytes = size_t(2) * p.K * p.d * sizeof(float);
-  const size_t res_bytes = size_t((p.m + 15) / 16) * p.d * sizeof(float) + cent_bytes;
   const PruneOut out{keep_idx, kind, cluster, scores};
   if (plan.grid) {
     auto kern = p.K == 4 ? (p.sim == SPD_SIM_COS ? kmeans_grid_kernel<4, true> : kmeans_grid_kernel<4, false>)
@@ -2294,13 +2301,13 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
   if (plan.grid) {
     // launched above
   } else if (plan.fused && p.K == 4)
-    SPD_CUDA_TRY((launch_kmeans<16, true, 4, true>(p, w, out, res_bytes, st)));
+    SPD_CUDA_TRY((launch_kmeans<16, true, 4, true>(p, w, out, res_bytes(p), st)));
   else if (plan.fused)
-    SPD_CUDA_TRY((launch_kmeans<16, true, SPD_MAX_CLUSTERS, true>(p, w, out, res_bytes, st)));
+    SPD_CUDA_TRY((launch_kmeans<16, true, SPD_MAX_CLUSTERS, true>(p, w, out, res_bytes(p), st)));
   else if (plan.res && p.K == 4)
-    SPD_CUDA_TRY((launch_kmeans<16, true, 4>(p, w, out, res_bytes, st)));
+    SPD_CUDA_TRY((launch_kmeans<16, true, 4>(p, w, out, res_bytes(p), st)));
   else if (plan.res)
-    SPD_CUDA_TRY((launch_kmeans<16, true, SPD_MAX_CLUSTERS>(p, w, out, res_bytes, st)));
+    SPD_CUDA_TRY((launch_kmeans<16, true, SPD_MAX_CLUSTERS>(p, w, out, res_bytes(p), st)));
   else if (plan.stream)
     SPD_CUDA_TRY(launch_stream(p, w, plan, st));
   else if (p.K == 4)

@@ -70,6 +70,16 @@ def test_prune_config_validation(lib):
         assert N.spd_prune_workspace_size(bad) == 0
 
 
+def test_prune_workspace_of_resident_tiles_is_small(lib):
+    # up to seven LLaVA tiles are clustered from shared memory: 32 KB of cluster sums a tile, a few values a token and
+    # no block for the K-means over the whole GPU (152 to 160 CTAs x 2 layers x 4 clusters x 1024 floats, 5 MB),
+    # which one tile of 2739 tokens and eight small ones have
+    for tiles in (1, 7):
+        assert N.spd_prune_workspace_size(N.prune_cfg(tiles, 577, 1024, 2, 1, 16, 192)) < 100_000 * tiles + 10_000
+    assert N.spd_prune_workspace_size(N.prune_cfg(8, 577, 1024, 2, 1, 16, 192)) > 5_000_000
+    assert N.spd_prune_workspace_size(N.prune_cfg(1, 2739, 1280, 2, 1, 16, 685, has_cls=False, attn_form=1)) > 6_000_000
+
+
 def test_workspace_sizes_grow_with_problem(lib):
     a = N.spd_prune_workspace_size(N.prune_cfg(1, 577, 1024, 2, 1, 16, 192))
     b = N.spd_prune_workspace_size(N.prune_cfg(5, 577, 1024, 2, 1, 16, 64))
