@@ -129,6 +129,11 @@ __global__ void __launch_bounds__(kThreads, 2)
   if (threadIdx.x == 0) stamp_start(stamp);
   const int4 tl = tiles[tile];
   const int q0 = tl.x, nq = tl.y, kv0 = tl.z, len = tl.w;
+  if (nq == 0) {  // padding of a list made on the device: nothing to do
+    if (warp == 4) tmem_dealloc(tmem, kTmemCols);
+    if (threadIdx.x == 0) stamp_end(stamp);
+    return;
+  }
   const int p_last = q_pos[q0 + nq - 1];  // positions ascend within a tile
   const int nkb = max(1, min((p_last + kTK) / kTK, (len + kTK - 1) / kTK));
   const int my_pos = threadIdx.x < 128 ? q_pos[q0 + min(int(threadIdx.x), nq - 1)] : 0;

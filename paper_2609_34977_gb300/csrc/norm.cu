@@ -300,8 +300,8 @@ __device__ int block_scan_excl(int v, int* tmp, int* total) {
 // layer l when 0 <= admit[t] <= l. Outputs in the executor's layout: arows (attention-active
 // tokens, ascending; padded to T with -1), amap (token -> its query row or -1), apos (positions of
 // the query rows), frows (FFN-active tokens; padded with -1), tiles (up to 128 queries of one
-// sequence each; padded to max_tiles with copies of the last tile, whose recomputation writes the
-// same values, or a one-query tile when no token is a query). One CTA.
+// sequence each, behind empty tiles that make them up to max_tiles: the attention kernel walks the list
+// from its end, so the empty ones come last). One CTA.
 __global__ void __launch_bounds__(1024)
     plan_lists_kernel(int T, int B, const int32_t* cu, const int32_t* pos, const int32_t* admit,
                       const uint8_t* target, int l, const int32_t* kv0, const int32_t* kvlen,
@@ -348,20 +348,14 @@ __global__ void __launch_bounds__(1024)
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    int a = 0, k = 0;
+    int a = 0, k = max_tiles;
+    for (int b = 0; b < B; ++b) k -= (seq_cnt[b] + 127) / 128;
+    for (int e = 0; e < k; ++e) tiles[e] = make_int4(0, 0, 0, 0);
     for (int b = 0; b < B; ++b) {
       const int n = seq_cnt[b];
       for (int s0 = 0; s0 < n; s0 += 128) tiles[k++] = make_int4(a + s0, min(128, n - s0), kv0[b], kvlen[b]);
       a += n;
     }
-    int4 pad;
-    if (k > 0) {
-      pad = tiles[k - 1];
-    } else {
-      pad = make_int4(0, 1, kv0[0], kvlen[0]);
-      apos[0] = pos[0];
-    }
-    for (; k < max_tiles; ++k) tiles[k] = pad;
   }
 }
 

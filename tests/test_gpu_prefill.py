@@ -329,6 +329,28 @@ def test_adaptive_device_plan_small_and_textless_sequences(seed, lens, n_text):
     assert rowwise_rel(logits.cpu().numpy(), lg0) < TOL
 
 
+@pytest.mark.parametrize("lens,n_text", [
+    ([300, 200, 129], [10, 4, 1]),  # 15 of 629 tokens stay queries: four of seven tiles of the list are empty
+    ([140, 20], [0, 0]),            # nobody does: every tile is
+])
+def test_adaptive_device_plan_of_skipped_queries(lens, n_text):
+    # every visual token is admitted at layer 0 and passes the attention by from then on
+    model, om, x, vis, cu = _adaptive_inputs(43, lens, n_text)
+    slc, tgt = np.full(6, 0.5), np.full(6, 1, np.uint8)
+    h0, lg0, admit0, _, _ = od.prefill_adaptive(om, bf16_np(x), cu, vis, slc, tgt, -1.0, 3.0, 1.0, 2)
+    assert (admit0[vis] == 0).all()
+    T, B = x.shape[0], len(lens)
+    ws = torch.zeros(N.spd_prefill_adaptive_workspace_size(model, T, B), dtype=torch.uint8, device="cuda")
+    h = torch.full((T, 256), float("nan"), device="cuda")
+    logits = torch.full((B, 512), float("nan"), device="cuda")
+    admit = N.spd_prefill_adaptive(model, x.cuda(), T, cu, vis, slc, tgt, -1.0, 3.0, 1.0, 2, h, logits, ws, device_plan=1)
+    torch.cuda.synchronize()
+    assert N.spd_workspace_status(ws) == 0
+    np.testing.assert_array_equal(admit.astype(np.int64), admit0)
+    assert rowwise_rel(h.cpu().numpy(), h0) < TOL
+    assert rowwise_rel(logits.cpu().numpy(), lg0) < TOL
+
+
 def test_adaptive_plan_with_given_plan_is_the_plain_prefill():
     # the same tokens, the plan the online rule chose, run through spd_prefill: the same result up
     # to the order of the residual adds (split-K red.add) and the bf16 roundings that order decides
