@@ -41,8 +41,8 @@ int num_sms();  // SM count of the current device
 //  * every kernel executes griddepcontrol.wait in at least one thread before it can complete, so
 //    completion orders transitively: when kernel N passes its wait, every earlier kernel of the
 //    stream has completed.
-// carveout: the share of an SM's 256 KB that is set aside as shared memory, in percent (0: the driver's choice,
-// which can hold a kernel of several CTAs an SM below the number that its registers allow).
+// carveout: how much of the shared memory that an SM can hold (228 KB) is set aside for it, in percent (0: the
+// driver's choice, which can hold a kernel of several CTAs an SM below the number that its registers allow).
 // overlap: false starts the kernel only when everything before it in the stream has completed.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_with(bool overlap, int carveout, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
