@@ -145,6 +145,29 @@ def test_residual_whole_tiles_repeat_exactly(M):
         assert all(torch.equal(o, outs[0]) for o in outs)
 
 
+def test_scratch_cleared_as_a_call_needs_more_of_it():
+    # 1250 tokens on 152 SMs: the QKV GEMM leaves 12 tiles over (their sums and counters are cleared), the gate-up
+    # GEMM needs more counters, the other layer's GEMMs find all of it clear. The workspace holds garbage before.
+    cfg = dict(synth.TINY_DECODER, n_layers=2, d_model=2048, n_heads=32, n_kv_heads=32, head_dim=128, d_ffn=11008)
+    w = synth.decoder_weights(4, cfg, device="cuda")
+    model = N.SpdModel(cfg, w)
+    T = 1250
+    x = _bf16(8, T, 2048).cuda()
+    cu = np.array([0, 700, T], np.int32)
+    got = []
+    for fill in (0, 0x7f):
+        ws = torch.full((N.spd_prefill_workspace_size(model, T, 2),), fill, dtype=torch.uint8, device="cuda")
+        ws[:256] = 0  # the status word
+        h, logits = torch.empty(T, 2048, device="cuda"), torch.empty(2, cfg["vocab"], device="cuda")
+        N.spd_prefill(model, x, T, cu, None, h, logits, ws)
+        torch.cuda.synchronize()
+        assert N.spd_workspace_status(ws) == 0
+        got.append((h, logits))
+    for a, b in zip(*got):  # the same kernels twice: bf16 units that the order of residual sums decides
+        assert torch.isfinite(b).all()
+        assert rowwise_rel(b.double().cpu().numpy(), a.double().cpu().numpy()) < 2.0 ** -6
+
+
 # ---- MSV-Prune: K-means over the whole GPU, rankings over several CTAs --------------------------------
 def _shuffled_tile(seed0, n, d, keep, **kw):
     # a tile whose planted groups lie scattered over the token order: the seeds fall into any of them, so
@@ -178,6 +201,40 @@ def test_whole_gpu_kmeans(tiles, n, d, keep, kw):
     v = {"feats": [np.concatenate([x["feats"][l] for x in vs]) for l in range(2)],
          "attn": np.concatenate([x["attn"] for x in vs])}
     assert_prune_parity(gpu_prune(v, keep, 1, has_cls=False, attn_form=1, **kw), res)
+
+
+@pytest.mark.parametrize("tiles,n,d,keep,layers,final,kw", [
+    (12, 200, 2052, 40, 2, 1, {}),                  # rows too wide for the one-sweep ring: re-read from L2
+    (12, 200, 32, 40, 2, 1, {}),                    # ... too short for it
+    (12, 200, 32, 40, 2, 0, dict(sim="mse")),
+    (12, 200, 2052, 40, 1, 0, dict(sim="kl")),
+    (11, 333, 512, 50, 1, 0, {}),                   # one sweep: the final layer alone, first, between the others
+    (11, 333, 512, 50, 3, 0, {}),
+    (11, 333, 512, 50, 3, 1, {}),
+    (11, 333, 512, 50, 3, 1, dict(sim="mse")),
+    (1, 1100, 1024, 150, 1, 0, {}),                 # the whole GPU: the same
+    (1, 1100, 1024, 150, 3, 0, {}),
+    (1, 1100, 1024, 150, 3, 1, {}),
+])
+def test_kmeans_forms_and_layers(tiles, n, d, keep, layers, final, kw):
+    vs, res = [], []
+    for i in range(tiles):
+        _, v1, r1 = conditioned_vision(20266001 + 307 * i, 1, n, d, layers, 4, keep, final, has_cls=False, attn_form=1,
+                                       tries=256, **kw)
+        vs.append(v1)
+        res += r1
+    v = {"feats": [np.concatenate([x["feats"][l] for x in vs]) for l in range(layers)],
+         "attn": np.concatenate([x["attn"] for x in vs])}
+    assert_prune_parity(gpu_prune(v, keep, final, has_cls=False, attn_form=1, **kw), res)
+
+
+@pytest.mark.parametrize("tiles", [1, 12])
+def test_prune_without_other_tokens(tiles):
+    # every token is an anchor: nothing to cluster, score or select
+    v = synth.vision_tiles(9, tiles, 70, 128, 2, 4, has_cls=False, attn_form=1)
+    g = gpu_prune(v, 70, 1, has_cls=False, attn_form=1, anchor_ratio=1.0)
+    np.testing.assert_array_equal(g["keep_idx"], np.tile(np.arange(70), (tiles, 1)))
+    assert (g["kind"] == 1).all() and (g["cluster"] == -1).all() and np.isposinf(g["scores"]).all()
 
 
 @pytest.mark.parametrize("tiles,n,d,keep,kw", [

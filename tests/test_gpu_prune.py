@@ -39,9 +39,9 @@ def test_llava_next_anyres_tiles(keep):
 
 @pytest.mark.parametrize("n_tiles", [24, 40])
 def test_many_tiles_streamed_kmeans(n_tiles):
-    # more tiles than one wave of resident 16-CTA K-means clusters: the form that re-reads the rows
-    # from L2 runs (serving batches), with 8 CTAs per tile while those clusters fit in one wave at
-    # two CTAs an SM (24 tiles on 152 SMs), with 4 CTAs per tile beyond (40 tiles)
+    # more tiles than one wave of resident 16-CTA K-means clusters, and than the whole-GPU form takes: the
+    # form of one sweep over the rows an iteration, in clusters of as many CTAs (8, 4, 2, 1) as leave
+    # every tile's cluster an SM a CTA
     # (tiles conditioned one by one: a seed whose 24 tiles all have margins above 1e-3 is rare)
     vs, res = [], []
     for i in range(n_tiles):
