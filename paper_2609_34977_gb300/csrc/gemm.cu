@@ -1462,16 +1462,7 @@ __global__ void __launch_bounds__(kGemvThreads, 3)
 // the quarters with their rounding errors: 5.0e-8 / 6.3e-8 / 8.0e-8 / 1.3e-7 at K 256 / 1024 / 4096 / 18944 where
 // FMAs have 5.5e-8 / 6.9e-8 / 9.4e-8 / 1.9e-7. (Two CTAs an SM instead of three hold the tree without spills.)
 // Nine to 16 tokens keep the chain, whose error is the tiled kernel's that they would take otherwise.
-constexpr int kGemvMmaTok = 16;  // 20 tokens: 787 us against 715 with the tiled kernel
-
-__device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                          uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
+constexpr int kGemvMmaTok = 16;  // 20 tokens of LLaVA width: 787 us against 715 with the tiled kernel
 
 // (a + b) + (c + d) with the rounding errors of the three additions added back (Knuth's two-sum).
 __device__ __forceinline__ float sum4_compensated(float a, float b, float c, float d) {
@@ -1533,7 +1524,8 @@ __global__ void __launch_bounds__(kGemvThreads, 2)
     for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int q = 0; q < NT; ++q)
-        xv[u][q] = r + 8 * q < a.n_tok && st + u < steps ? xp[size_t(q) * a.k + 4 * (st + u)] : z;  // 8 rows of k / 8 int4
+        xv[u][q] = r + 8 * q < a.n_tok && st + u < steps ? xp[size_t(q) * a.k + 4 * (st + u)]  // 8 rows of k / 8 int4
+                                                         : z;
     if constexpr (NT == 1) {
       float p[2 * U][4];
 #pragma unroll
@@ -1570,7 +1562,8 @@ __global__ void __launch_bounds__(kGemvThreads, 2)
     float v[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-      const float q0 = red[0][lane][t0 + t], q1 = red[1][lane][t0 + t], q2 = red[2][lane][t0 + t], q3 = red[3][lane][t0 + t];
+      const float q0 = red[0][lane][t0 + t], q1 = red[1][lane][t0 + t];
+      const float q2 = red[2][lane][t0 + t], q3 = red[3][lane][t0 + t];
       v[t] = NT == 1 ? sum4_compensated(q0, q1, q2, q3) : (q0 + q1) + (q2 + q3);
     }
     epilogue8<EPI>(a, n0 + lane, (n0 >> 5) & 3, lane, n0 >> 7, t0, v, trow, tpos, 0);
@@ -1718,7 +1711,8 @@ bool vec_red_ok(const GemmProblem& p) {
 
 // One token: gemv_kernel (which can norm its input); up to 16: gemv_mma_kernel
 bool gemv_aligned(const GemmProblem& p) {
-  return p.w && p.k % kGemvChunk == 0 && ((reinterpret_cast<uintptr_t>(p.w) | reinterpret_cast<uintptr_t>(p.x)) & 15) == 0;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(p.w) | reinterpret_cast<uintptr_t>(p.x);
+  return p.w && p.k % kGemvChunk == 0 && (at & 15) == 0;
 }
 bool gemv_eligible(const GemmProblem& p) {
   if (p.norm_h && ((reinterpret_cast<uintptr_t>(p.norm_h) | reinterpret_cast<uintptr_t>(p.norm_gain)) & 15))
@@ -1726,7 +1720,8 @@ bool gemv_eligible(const GemmProblem& p) {
   return p.n_tok == 1 && gemv_aligned(p) && gemv_for<4>(p.epi) != nullptr;
 }
 bool gemv_mma_eligible(const GemmProblem& p) {
-  return p.n_tok >= 1 && p.n_tok <= kGemvMmaTok && gemv_aligned(p) && !p.norm_h && gemv_mma_for(p.epi, p.n_tok) != nullptr;
+  return p.n_tok >= 1 && p.n_tok <= kGemvMmaTok && gemv_aligned(p) && !p.norm_h &&
+         gemv_mma_for(p.epi, p.n_tok) != nullptr;
 }
 
 int gemv_run(const GemmProblem& p, const GemmScratch& s, cudaStream_t stream) {

@@ -186,7 +186,8 @@ __device__ __forceinline__ float block_max(float v, float* red) {
 }
 
 // One candidate visual token per CTA (Sec. 4.2.1 and Eq. 6): E_ii = entropy of softmax(logits
-// row) / log V from the statistics of EPI_LSE_F32, F_itc = (cos(h_i, q_t) + 1) / 2 (0.5 without text), S_sa = ReLU(1 - E - F);
+// row) / log V from the statistics of EPI_LSE_F32, F_itc = (cos(h_i, q_t) + 1) / 2 (0.5 without text),
+// S_sa = ReLU(1 - E - F);
 // s_skip[i] += w1 S_sa + w2 SLC^Norm(l), flag[n] = s_skip[i] >= T_skip.
 __global__ void __launch_bounds__(kThreads)
     skip_score_kernel(const float* lse, int V, const float* h, int D, const int32_t* cand,

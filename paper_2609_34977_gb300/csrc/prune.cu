@@ -332,8 +332,8 @@ __device__ __forceinline__ float sum_f32x2(uint64_t a) {
 // as one packed instruction. Every product is still one fp32 FMA in the order of the features.
 // The partial tiles are summed in rank order through distributed shared memory, each CTA finishing R / AS
 // rows. AS = 4 at serving batch, 8 where that still leaves at most three CTAs an SM (shorter chains per CTA),
-// and R = 64 where R = 128 would leave SMs idle at that. AW is 64, or 48 where that pads the anchors less. (64 tiles of 531 x 45 anchors x 1024: 148 -> 115 us; 2260 x 479 x 1280:
-// 98 -> 81 us.)
+// and R = 64 where R = 128 would leave SMs idle at that. AW is 64, or 48 where that pads the anchors less.
+// (64 tiles of 531 x 45 anchors x 1024: 148 -> 115 us; 2260 x 479 x 1280: 98 -> 81 us.)
 template <int SIM, int AS, int AW, int kSimRows>
 __global__ void __cluster_dims__(AS, 1, 1) __launch_bounds__(256)
     anchor_sim_kernel(PruneDims p, PruneWs w) {
@@ -362,7 +362,8 @@ __global__ void __cluster_dims__(AS, 1, 1) __launch_bounds__(256)
   // shared memory (broadcast reads); -1 for rows past the lists
   const float* tile_f = feat_row(p, p.fin, t, -p.off);
   __shared__ int uo[kSimRows], ao[AW];
-  __shared__ double ulse[kl ? kSimRows : 1];  // KL: the non-anchor operand is softmax(F^L_i) = exp(F^L_i - lse_i), in fp64
+  // KL: the non-anchor operand is softmax(F^L_i) = exp(F^L_i - lse_i), in fp64
+  __shared__ double ulse[kl ? kSimRows : 1];
   if (threadIdx.x < kSimRows) {
     const int r = threadIdx.x;
     const bool uv = u0 + r < p.m;
@@ -705,7 +706,8 @@ __device__ __forceinline__ void column_sums(float* part, int K, int D, int nl, c
 
 // The nearest of four centroids for each of RP rows from the lanes' packed partial distances.
 template <int RP>
-__device__ __forceinline__ void assign4_nearest(const uint64_t (&acc)[RP][4], int n, bool first, int8_t* asg, int* changed) {
+__device__ __forceinline__ void assign4_nearest(const uint64_t (&acc)[RP][4], int n, bool first, int8_t* asg,
+                                                int* changed) {
   constexpr int NV = 4 * RP;
   const int lane = threadIdx.x & 31;
   float v[NV];
@@ -745,11 +747,11 @@ __device__ __forceinline__ void assign4_nearest(const uint64_t (&acc)[RP][4], in
   }
 }
 
-// assign_rows for K = 4, the calling warp's next n (at most RP count) rows at a time: a centroid's 16 bytes serve RP rows, differences and
-// squares are packed, and the 4 RP partial distances are summed over the lanes by halving exchanges (lane bits
-// 4, 3, ... pick the value) instead of a butterfly each. The loop is bound by issue: about 155
-// instructions a row of 1024 at RP = 4 where a row at a time took about 450 (28 rows of a CTA of eight
-// warps: 4.3 -> 2.0 us).
+// assign_rows for K = 4, the calling warp's next n (at most RP count) rows at a time: a centroid's 16 bytes
+// serve RP rows, differences and squares are packed, and the 4 RP partial distances are summed over the lanes
+// by halving exchanges (lane bits 4, 3, ... pick the value) instead of a butterfly each. The loop is bound by
+// issue: about 155 instructions a row of 1024 at RP = 4 where a row at a time took about 450 (28 rows of a CTA
+// of eight warps: 4.3 -> 2.0 us).
 template <int RP, typename Row>
 __device__ __forceinline__ void assign4_rows(const float* cent, int D, int n, bool first, int8_t* asg, int* changed,
                                              Row xrow) {
@@ -963,7 +965,8 @@ __global__ void __launch_bounds__(kmeans_threads<KN>()) kmeans_kernel(PruneDims 
   if (RES && m > 0 && warp == 0) {
     if (lane == 0) mbar_arrive_expect_tx(&rows_bar, uint32_t(nl + K) * D * 4);
     __syncwarp();
-    for (int k = lane; k < K; k += 32) bulk_load(cent + size_t(k) * D, fin + (row0 + ul[(k * m) / K]) * D, uint32_t(D) * 4, &rows_bar);
+    for (int k = lane; k < K; k += 32)
+      bulk_load(cent + size_t(k) * D, fin + (row0 + ul[(k * m) / K]) * D, uint32_t(D) * 4, &rows_bar);
     for (int jj = lane; jj < nl; jj += 32)
       bulk_load(rows + size_t(jj) * D, fin + (row0 + idx[jj]) * D, uint32_t(D) * 4, &rows_bar);
   }
@@ -1164,7 +1167,9 @@ __global__ void __launch_bounds__(kmeans_threads<KN>()) kmeans_kernel(PruneDims 
 constexpr int kGridThreads = 512;
 constexpr int kGridMaxCtas = 160;  // all tiles (workspace)
 constexpr int kGridMaxRows = 512;  // a CTA
-constexpr int kGridMeta = 2 * SPD_MAX_CLUSTERS;  // ints a CTA: sizes, [15 + 1]: changed flag; then a_j sums
+// Ints a CTA: [0, 16) its clusters' sizes, the CTA's changed flag in bit 30 of each; [16, 32) the a_j sums as
+// float bits.
+constexpr int kGridMeta = 2 * SPD_MAX_CLUSTERS;
 
 // Barrier number `phase` (1, 2, ...) of the G CTAs sharing *counter (zero at the start of the call). The
 // wait is bounded: on expiry the status is set and the counter raised past every target, whichever CTAs
@@ -1287,9 +1292,10 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
     __syncthreads();
     cluster_lists(asg, nl, K, cnt, ord, start);
     __syncthreads();
-    column_sums(part + size_t(r) * p.L * KD, K, D, nl, ord, start, RowAccess{res ? rows : nullptr, fin, row0, idx, D, nullptr});
+    column_sums(part + size_t(r) * p.L * KD, K, D, nl, ord, start,
+                RowAccess{res ? rows : nullptr, fin, row0, idx, D, nullptr});
     __syncthreads();
-    // sizes of K <= 16 clusters and the flag in the first 16 ints of the CTA's block (a flag bit on size 0)
+    // sizes of K <= 16 clusters, the flag beside each (a reader of any cluster's sizes sees it)
     if (threadIdx.x < K) meta[r * kGridMeta + threadIdx.x] = cnt[threadIdx.x] | (changed ? 1 << 30 : 0);
     if (!(ok = tile_barrier(bar, G, ++phase, w.status, kWaitBudget))) break;
     if (threadIdx.x == 0) any_changed = 0;
@@ -1345,7 +1351,8 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
       dsum[(size_t(r) * p.L + l) * 16 + threadIdx.x] = a;
     }
     column_sums(part + (size_t(r) * p.L + l) * KD, K, D, nl, ord, start,
-                RowAccess{res && l == p.fin ? rows : nullptr, p.feat[l], row0, idx, D, COS ? rinv : static_cast<float*>(nullptr)});
+                RowAccess{res && l == p.fin ? rows : nullptr, p.feat[l], row0, idx, D,
+                          COS ? rinv : static_cast<float*>(nullptr)});
   }
   ok = tile_barrier(bar, G, ++phase, w.status, kWaitBudget) && ok;
   pdl_launch_dependents();
@@ -1380,10 +1387,10 @@ __global__ void __launch_bounds__(kGridThreads) kmeans_grid_kernel(PruneDims p, 
 // bytes are in flight: every thread copies its four columns of 16 rows at a time (8 where rows are wider
 // than 1024) with 16-byte asynchronous copies into a ring of such steps, and one sweep does the
 // assignment of a step's rows (two a warp) and then their column sums from shared memory, four columns a
-// thread in registers. (One bulk copy a row held the whole kernel at 2.5 TB/s: 165 us.) From the second sweep on it also adds the unit rows, which are the final layer's
-// cluster sums if the assignment repeats. Every second sweep runs backwards: the rows that the last one
-// read end up in L2. So a tile whose assignment repeats at once is read twice for K-means and once a
-// further layer, where the form that it replaces (4 CTAs a tile re-reading the rows through registers) read
+// thread in registers. (One bulk copy a row held the whole kernel at 2.5 TB/s: 165 us.) From the second sweep on
+// it also adds the unit rows, which are the final layer's cluster sums if the assignment repeats. Every second
+// sweep runs backwards: the rows that the last one read end up in L2. So a tile whose assignment repeats at once
+// is read twice for K-means and once a further layer, where 4 CTAs a tile re-reading the rows through registers read
 // it five times: 64 tiles 234 -> 156 us serialised, of which the copies alone take 76; the assignment (with
 // the centroids in registers up to 1024 columns) and the sums are chains of shared-memory loads of 8 warps.
 constexpr int kStreamThreads = 256;
@@ -2254,7 +2261,8 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
   SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, p.sim == SPD_SIM_COS ? rowstats_kernel<SPD_SIM_COS>
                           : p.sim == SPD_SIM_MSE ? rowstats_kernel<SPD_SIM_MSE> : rowstats_kernel<SPD_SIM_KL>,
                           dim3((p.n + 7) / 8, T), dim3(256), 0, st, p, attn, w));
-  SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, anchor_kernel, dim3(rank_ctas(p.n), T), dim3(kRankThreads), 0, st, p, w));
+  SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, anchor_kernel, dim3(rank_ctas(p.n), T), dim3(kRankThreads), 0, st,
+                                   p, w));
   if (int rc = kmeans_setup()) return rc;
   PrunePlan plan = prune_plan(p);
   if (plan.anchor_sim) {
@@ -2320,8 +2328,8 @@ extern "C" int spd_prune(const spd_prune_cfg* cfg, const float* const* feats, co
                    : p.sim == SPD_SIM_MSE ? score_kernel<SPD_SIM_MSE> : score_kernel<SPD_SIM_KL>;
       SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, score, dim3((p.m + 7) / 8, T), dim3(256), 0, st, p, w));
     }
-    SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, select_kernel, dim3(rank_ctas(p.m), T), dim3(kRankThreads), 0, st, p, w, keep_idx, kind, cluster,
-                            scores));
+    SPD_CUDA_TRY(launch_pdl_carveout(kPruneCarveout, select_kernel, dim3(rank_ctas(p.m), T), dim3(kRankThreads), 0, st,
+                                     p, w, keep_idx, kind, cluster, scores));
   }
   // algorithmic work per tile: every tapped layer's features and the attention read once, the
   // kept indices written; anchor similarities (n - N_anc) N_anc d multiply-adds
