@@ -387,9 +387,10 @@ int spd_decode(const spd_model* m, const uint16_t* x, int n_seqs, const int32_t*
 /* Single kernels, exposed for composition and per-kernel tests                                 */
 /* ------------------------------------------------------------------------------------------ */
 
-/* Epilogues of spd_linear. All but SPD_EPI_ADD_F32 give bit-identical results run to run; the
- * residual update adds with fire-and-forget atomics, so where K is split across CTAs the fp32
- * additions land in no fixed order (results agree to rounding). */
+/* Epilogues of spd_linear. Results are bit-identical run to run but for two schedules, whose fp32
+ * additions land in no fixed order (results agree to rounding): the residual update (SPD_EPI_ADD_F32) where
+ * K is split across CTAs, and the few tiles left over where the output has slightly more of them than the
+ * GPU takes at once. */
 typedef enum {
   SPD_EPI_F32 = 0,       /* out fp32 [M][N] = acc */
   SPD_EPI_BF16 = 1,      /* out bf16 [M][N] = bf16(acc) */
