@@ -29,8 +29,6 @@
 
 #include <cooperative_groups.h>
 
-#include <type_traits>
-
 #include "internal.h"
 #include "ptx.cuh"
 #include "trace.h"
@@ -342,20 +340,25 @@ int launch(const CUtensorMap& mq, const CUtensorMap& mkv, void* o, int ldo, cons
 // eight warps takes groups of 16 keys, 16 bytes a lane and load, and multiplies them with the legacy
 // m16n8k16 tensor instruction straight from registers (at most 8 of a tile's 128 rows would be
 // queries on the tcgen05 path, which would also have to stage K and V in shared memory).
-// For few CTAs, eight warps of 184 registers, one CTA an SM, were faster than four CTAs of four warps (a whole step of
-// 32 sequences 829 against 828 us, of one sequence 3142 against 3167) or 128 registers a thread (3199).
+// Eight warps of 224 registers, one CTA an SM: four CTAs of four warps were slower (a whole step of one sequence
+// 3167 against 3142 us), two CTAs of 128 registers spill and are no faster (64 sequences of 500 keys, 32 heads, four
+// layers: 1069 us both), and without the second launch bound the compiler takes 207 registers and 1162 us.
 // One layer's attention of 32 sequences (28 query heads on 4 K/V heads of 128, 1122 keys on average,
-// 73 MB, serialised): 143 us with one warp a key and one CTA a query head, 35.5 us here and 29 with the
+// 73 MB, serialised): 143 us with one warp a key and one CTA a query head, 35.5 us so and 29 with the
 // longest sequences first; the step of four layers 1256 -> 829 us. One sequence of 257 keys, 32 heads: 10.4 -> 7.2 us.
 //  * S = Q K^T: heads are the 16 rows of A (rows 8..15 stay zero), keys the 8 columns of B. The
 //    order of the contraction index is free, so lane (r = lane / 4, c = lane % 4) feeds the two
-//    MMAs of a 32-dim block from one 16-byte load of key r, dims 8 c .. 8 c + 7, of K and of Q alike.
-//  * O += P V: P is split into two bf16 terms, hi in rows 0..7 and the remainder lo in rows 8..15 of
-//    the same MMA (p - hi - lo is below 2^-17 p, far under the bf16 rounding of the output); V of key
-//    k, dims 8 r .. 8 r + 7 is one 16-byte load, byte-permuted into pairs of keys.
-// Error of the bf16 outputs against 64 bits, 12 shapes of 257 to 2047 keys, 4 seeds each: the same to seven
-// digits as with fp32 weights and FMAs (1.6760e-3 for 28 heads and 257 keys, 1.6635e-3 for 16 sequences of 32
-// heads); the two forms round differently where a value lies at a border, 0.07 to 0.2 % of the outputs.
+//    MMAs of a 32-dim block from one 16-byte load of key r, dims 8 c .. 8 c + 7, of K and of Q alike. Each MMA
+//    starts from zero and the sums are fp32 additions: a chain would lose its low bits.
+//  * O += P V: P is split into three bf16 terms, which hold all 24 bits of it: the first, hi, in rows 0..7 of two
+//    MMAs, half of it each, the others in rows 8..15 of the first and of the second. (hi has rows of its own
+//    since the others may be zero or negative, which an infinite V must not meet.) V of key k, dims
+//    8 r .. 8 r + 7 is one 16-byte load, byte-permuted into pairs of keys.
+// Error of the bf16 outputs against 64 bits, 12 shapes of 257 to 2047 keys, four seeds each: the same to seven digits
+// as with fp32 FMAs, and as many outputs at a border that round the other way (0.01 to 0.05 %; 0.05 to 0.2 %
+// with two terms and chained sums, which held 17 bits of P). The third term and the sums from zero change a step of
+// one sequence from 2842 to 2831 us, of 32 from 768 to 760, with 32 K/V heads of 10 / 16 / 64 sequences of 900 / 900 /
+// 500 keys from 608 / 642 / 1028 to 577 / 648 / 1069.
 // Online softmax a warp (running maximum m, sum l), O rescaled only when some maximum grew. The
 // warps' states are merged in warp order, the CTAs' in rank order through distributed shared memory,
 // each CTA finishing a share of the outputs.
@@ -374,8 +377,8 @@ __device__ __forceinline__ uint4 load8(const __nv_bfloat16* p) {
   }
 }
 
-template <int HD, bool A16, int MINB>
-__global__ void __launch_bounds__(kDecWarps * 32, MINB)
+template <int HD, bool A16>
+__global__ void __launch_bounds__(kDecWarps * 32, 1)
     attn_decode_kernel(const __nv_bfloat16* q, const __nv_bfloat16* kv, int ldkv, int v_off,
                        __nv_bfloat16* __restrict__ o, int ldo, const int4* tiles, int n_heads,
                        int n_kv_heads, int chunks, float scale_log2, unsigned long long* stamp) {
@@ -402,7 +405,7 @@ __global__ void __launch_bounds__(kDecWarps * 32, MINB)
     qf[i] = r < ng ? *reinterpret_cast<const uint4*>(q + size_t(tl.x) * (n_heads * HD) + (h0 + r) * HD + 32 * i + 8 * c)
                    : make_uint4(0u, 0u, 0u, 0u);
   float m = -INFINITY, l = 0.0f;
-  float acc[VB][8][4];  // rows r (hi) and r + 8 (lo), dims 64 b + 16 c + j and 64 b + 16 c + 8 + j
+  float acc[VB][8][4];  // rows r (hi) and r + 8 (the rest), dims 64 b + 16 c + j and 64 b + 16 c + 8 + j
 #pragma unroll
   for (int b = 0; b < VB; ++b)
 #pragma unroll
@@ -427,13 +430,16 @@ __global__ void __launch_bounds__(kDecWarps * 32, MINB)
         vf[u][b] = key < j_hi ? load8<A16>(kbase + size_t(key) * ldkv + v_off + 64 * b + 8 * r)
                               : make_uint4(0u, 0u, 0u, 0u);
     }
-    float s[2][4] = {{0.0f, 0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f, 0.0f}};
+    float s[2][2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
 #pragma unroll
     for (int i = 0; i < KB; ++i)
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
-        mma_16816(s[t], qf[i].x, 0u, qf[i].y, 0u, kf[t][i].x, kf[t][i].y);
-        mma_16816(s[t], qf[i].z, 0u, qf[i].w, 0u, kf[t][i].z, kf[t][i].w);
+        float p0[4] = {0.0f, 0.0f, 0.0f, 0.0f}, p1[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        mma_16816(p0, qf[i].x, 0u, qf[i].y, 0u, kf[t][i].x, kf[t][i].y);
+        mma_16816(p1, qf[i].z, 0u, qf[i].w, 0u, kf[t][i].z, kf[t][i].w);
+        s[t][0] += p0[0] + p1[0];
+        s[t][1] += p0[1] + p1[1];
       }
     // head r, keys k0 + 2 c + {0, 1} and k0 + 8 + 2 c + {0, 1}
     float x[4];
@@ -457,16 +463,18 @@ __global__ void __launch_bounds__(kDecWarps * 32, MINB)
           for (int e = 0; e < 4; ++e) acc[b][j][e] *= corr;
       m = mn;
     }
-    float hi[4], lo[4];
+    float hi[4], lo[4], rem[4];  // half of the first term; the others
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const float p = exp2f(x[u] - m);
+      const float p = exp2f(x[u] - m), first = __bfloat162float(__float2bfloat16_rn(p));
       l += p;
-      hi[u] = __bfloat162float(__float2bfloat16_rn(p));
-      lo[u] = p - hi[u];
+      hi[u] = 0.5f * first;
+      lo[u] = p - first;
+      rem[u] = lo[u] - __bfloat162float(__float2bfloat16_rn(lo[u]));
     }
-    const uint32_t a0 = pack_bf16(hi[0], hi[1]), a1 = pack_bf16(lo[0], lo[1]), a2 = pack_bf16(hi[2], hi[3]),
-                   a3 = pack_bf16(lo[2], lo[3]);
+    const uint32_t a0 = pack_bf16(hi[0], hi[1]), a2 = pack_bf16(hi[2], hi[3]);
+    const uint32_t a1 = pack_bf16(lo[0], lo[1]), a3 = pack_bf16(lo[2], lo[3]);
+    const uint32_t c1 = pack_bf16(rem[0], rem[1]), c3 = pack_bf16(rem[2], rem[3]);
 #pragma unroll
     for (int b = 0; b < VB; ++b) {
       const uint32_t w[4][4] = {{vf[0][b].x, vf[0][b].y, vf[0][b].z, vf[0][b].w},
@@ -474,9 +482,10 @@ __global__ void __launch_bounds__(kDecWarps * 32, MINB)
                                 {vf[2][b].x, vf[2][b].y, vf[2][b].z, vf[2][b].w},
                                 {vf[3][b].x, vf[3][b].y, vf[3][b].z, vf[3][b].w}};
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
+      for (int e = 0; e < 16; ++e) {  // independent products side by side
+        const int j = e & 7;
         const uint32_t sel = (j & 1) ? 0x7632u : 0x5410u;
-        mma_16816(acc[b][j], a0, a1, a2, a3, __byte_perm(w[0][j >> 1], w[1][j >> 1], sel),
+        mma_16816(acc[b][j], a0, e < 8 ? a1 : c1, a2, e < 8 ? a3 : c3, __byte_perm(w[0][j >> 1], w[1][j >> 1], sel),
                   __byte_perm(w[2][j >> 1], w[3][j >> 1], sel));
       }
     }
@@ -492,7 +501,7 @@ __global__ void __launch_bounds__(kDecWarps * 32, MINB)
     for (int b = 0; b < VB; ++b)
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        // an infinite V times lo = 0 is NaN: the remainder counts where the main term is finite
+        // an infinite V times a zero term is NaN: the others count where the first is finite
         const float x0 = acc[b][j][0], x1 = acc[b][j][1];
         wo[warp][r][64 * b + 16 * c + j] = isfinite(x0) ? x0 + acc[b][j][2] : x0;
         wo[warp][r][64 * b + 16 * c + 8 + j] = isfinite(x1) ? x1 + acc[b][j][3] : x1;
@@ -619,16 +628,8 @@ int attention_decode_run(const void* q, const void* kv, int ldkv, int v_off, voi
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   const bool a16 = (reinterpret_cast<uintptr_t>(kv) & 15) == 0 && (ldkv | v_off) % 8 == 0;
-  // Two CTAs an SM (128 registers, a few spilled) where there are more than that of them: 16 / 64 sequences of 500
-  // keys, 32 K/V heads, four layers 582 / 1114 -> 557 / 1021 us a step; but 256 CTAs of seven heads each (32
-  // sequences) 755 -> 781, one sequence and 32 layers 2829 -> 2887.
-  const bool two = groups * S > 2LL * num_sms();
-  auto pick = [&](auto minb) {
-    constexpr int M = decltype(minb)::value;
-    return head_dim == 128 ? (a16 ? attn_decode_kernel<128, true, M> : attn_decode_kernel<128, false, M>)
-                           : (a16 ? attn_decode_kernel<64, true, M> : attn_decode_kernel<64, false, M>);
-  };
-  auto kern = two ? pick(std::integral_constant<int, 2>()) : pick(std::integral_constant<int, 1>());
+  auto kern = head_dim == 128 ? (a16 ? attn_decode_kernel<128, true> : attn_decode_kernel<128, false>)
+                              : (a16 ? attn_decode_kernel<64, true> : attn_decode_kernel<64, false>);
   SPD_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, qb, kb, ldkv, v_off, ob, ldo, tiles, n_heads, n_kv_heads, chunks,
                                   scale_log2, stamp));
   trace_end(slot, stream, TR_ATTN, fl, by);

@@ -25,7 +25,7 @@ def _bf16(seed, *shape):
     (28, 4, 128, [65, 127, 128, 129, 500, 7], 0),   # seven heads a K/V head, shares of unequal length
     (18, 2, 64, [31, 260, 511], 0),                 # nine heads a K/V head: a second chunk of one head
     (16, 1, 128, [0, 1, 300, 511, 48, 47, 33, 2], 0),  # two full chunks; clusters of eight CTAs
-    (32, 32, 64, list(range(0, 500, 50)), 0),          # more CTAs than two an SM hold
+    (32, 32, 64, list(range(0, 500, 50)), 0),          # more CTAs than two an SM
 ])
 def test_decode_attention_edges(heads, kv_heads, head_dim, pos, offset):
     # one decoder layer over a given cache: logits and the appended K/V rows. Tolerance: every rounding of
@@ -68,6 +68,43 @@ def test_decode_attention_edges(heads, kv_heads, head_dim, pos, offset):
     for b in range(B):
         assert rowwise_rel(got[b, p[b]:p[b] + 1], np.concatenate([k[b:b + 1], v[b:b + 1]], 1)) < 2e-2
         assert not got[b, p[b] + 1:].any()
+
+
+def test_decode_attention_weights_hold_24_bits():
+    # two keys of nearly equal weight (2^-11 apart in one dimension) whose values cancel but for that difference,
+    # beside two keys that make the weights uneven and carry no value: the output is about 2^-15 of the weights,
+    # so a weight cut to 17 bits shows as tens of percent. Tolerance: the bf16 roundings of q and of the output,
+    # as in the other decode tests.
+    H, hd, B, max_len = 4, 64, 8, 16
+    cfg = dict(synth.TINY_DECODER, n_layers=1)
+    w = synth.decoder_weights(5, cfg, std=0.05)
+    lw = w["layers"][0]
+    for name in ("wk", "wv", "w_down"):
+        lw[name].zero_()
+    lw["wo"].copy_(64 * torch.eye(H * hd))
+    wd = {k: v.cuda() for k, v in w.items() if k != "layers"}
+    wd["layers"] = [{k: v.cuda() for k, v in lw.items()}]
+    c = torch.zeros(B, max_len, 2, H, hd)
+    c[:, 0, 0, :, 1] = 2.0 ** -11
+    c[:, 2, 0, :, 0], c[:, 3, 0, :, 0] = 8.0, -8.0
+    c[:, 0, 1], c[:, 1, 1] = 256.0, -256.0
+    cache = c.to(torch.bfloat16).reshape(B, max_len, -1).cuda()
+    x = (_bf16(7, B, H * hd).float() * 1e-3).to(torch.bfloat16)
+    out = torch.empty(B, cfg["vocab"], device="cuda")
+    model = N.SpdModel(cfg, wd)
+    ws = torch.zeros(N.spd_decode_workspace_size(model, B), dtype=torch.uint8, device="cuda")
+    N.spd_decode(model, x.cuda(), np.full(B, 4), cache, max_len, out, ws)
+    om = od.model_from_torch(w, cfg)
+    ow, rnd = om["layers"][0], od.bf16_round
+    h = bf16_np(x).astype(np.float64)
+    xa = rnd(od.rmsnorm(h, ow["attn_norm"], cfg["rms_eps"]))
+    q = rnd(od.rope(xa @ ow["wq"].T, np.full(B, 4), H, hd, cfg["rope_theta"]))
+    kv = c.double().numpy().reshape(B, max_len, 2, -1)
+    for b in range(B):
+        o = od.causal_attention(q[b:b + 1], kv[b, :5, 0], kv[b, :5, 1], np.array([4]), np.arange(5), H, H, hd)
+        h[b] += 64 * rnd(o)[0]
+    z = rnd(od.rmsnorm(h, om["final_norm"], cfg["rms_eps"]))
+    assert rowwise_rel(out.cpu().numpy(), z @ om["lm_head"].T) < 2e-2
 
 
 # ---- few-token GEMMs: m16n8k16 straight from the weight rows ------------------------------------------
